@@ -207,7 +207,7 @@ def run_reference(args, rank, world):
             "e2e": {"value": value, "unit": "spawn attempts/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
 
 
-KERNEL_NAMES = {"k_spawn": "k_spawn_draw + k_spawn_eval (split spawning)",
+KERNEL_NAMES = {"k_spawn": "k_spawn",
                 "k_annihilate": "k_annihilate_staged + k_annihilate_big"}
 
 WORKLOAD_NAMES = {

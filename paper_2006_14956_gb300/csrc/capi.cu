@@ -278,11 +278,9 @@ static int enqueue_iteration(fciqmc_handle *h, cudaEvent_t *ev)
 {
     const int units = 1 << h->bb;
     if (ev) cudaEventRecord(ev[0], h->stream);
-    const bool st = staged_spawn_fits(h->hi), split = st && h->hi.qcnt != nullptr && spawn_split_selected();
-    launch_spawn(h->dinst, h->dunit, 1, units, st, split, h->stream);
-    if (split) launch_spawn_eval(h->dinst, 1, h->stream);
+    launch_spawn(&h->hi, h->dinst, h->dunit, 1, units, h->hi.adaptive != 0, h->stream);
     if (ev) cudaEventRecord(ev[1], h->stream);
-    launch_spawn_heavy(h->dinst, 1, h->stream);
+    launch_spawn_heavy(&h->hi, h->dinst, 1, h->stream);
     if (ev) cudaEventRecord(ev[2], h->stream);
     if (h->nd > 0) launch_semistoch(h->dinst, 1, h->nd, h->stream);
     if (ev) cudaEventRecord(ev[3], h->stream);
@@ -313,57 +311,10 @@ static int count_kernel_nodes(cudaGraph_t g)
     return k;
 }
 
-// the attempt queues of split spawning, allocated when that mode is selected
-// (and the run's arrays suit the staged kernels): min(draw grid, buckets)
-// segments per class, each sized from the requested count (need, per class),
-// at least 4096 entries (two determinants' worth of light attempts)
-static int ensure_queues(fciqmc_handle *h, long long need0 = 0, long long need1 = 0)
-{
-    DevInst &I = h->hi;
-    if (!spawn_split_selected() || !staged_spawn_fits(I)) return FCIQMC_OK;
-    bool changed = false;
-    const int nseg = std::min(draw_segments(), 1 << h->bb);
-    if (I.qcnt && I.qnseg != nseg) {  // more buckets or another grid: new queues
-        dev_free(h, I.qcnt);
-        dev_free(h, I.qrec[0]);
-        dev_free(h, I.qrec[1]);
-        I.qcnt = nullptr;
-        I.qrec[0] = I.qrec[1] = nullptr;
-        I.qcap[0] = I.qcap[1] = 0;
-    }
-    if (!I.qcnt) {
-        I.qcnt = (int *)dev_alloc(h, 2 * (size_t)nseg * sizeof(int));
-        if (!I.qcnt) return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (attempt queues)");
-        CUDA_TRY(h, cudaMemsetAsync(I.qcnt, 0, 2 * (size_t)nseg * sizeof(int), h->stream));
-        I.qnseg = nseg;
-        changed = true;
-    }
-    const long long want[2] = {std::max<long long>(4096, need0), std::max<long long>(4096, need1)};
-    for (int c = 0; c < 2; c++) {
-        if (I.qrec[c] && I.qcap[c] >= want[c]) continue;
-        long long cap = I.qcap[c] > 0 ? I.qcap[c] : 4096;
-        while (cap < want[c]) cap = cap + cap / 2;
-        if (cap > (1LL << 30)) return fail(h, FCIQMC_ERR_CAPACITY, "attempt queue limit reached");
-        dev_free(h, I.qrec[c]);
-        I.qrec[c] = (QRec *)dev_alloc(h, (size_t)nseg * (size_t)cap * sizeof(QRec));
-        if (!I.qrec[c]) {
-            I.qcap[c] = 0;
-            return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (attempt queues)");
-        }
-        I.qcap[c] = cap;
-        changed = true;
-    }
-    return changed ? upload_inst(h) : FCIQMC_OK;  // the device copy of the descriptor follows
-}
-
 static int capture_graph(fciqmc_handle *h)
 {
     if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
     cudaGraph_t g;
-    {
-        const int rq = ensure_queues(h);
-        if (rq) return rq;
-    }
     CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     int rc = enqueue_iteration(h, nullptr);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
@@ -485,9 +436,6 @@ static int reset_after_error(fciqmc_handle *h)
     h->hst.need_main = 0;
     h->hst.n_spawn_over = 0;
     h->hst.new_n = 0;
-    h->hst.need_queue[0] = 0;
-    h->hst.need_queue[1] = 0;
-    if (h->hi.qcnt) CUDA_TRY(h, cudaMemsetAsync(h->hi.qcnt, 0, 2 * (size_t)h->hi.qnseg * sizeof(int), h->stream));
     CUDA_TRY(h, cudaMemsetAsync(h->hi.acc, 0, NSHARD * ACC_STRIDE * sizeof(u64), h->stream));  // partial totals
     // the failed iteration's adaptive-shift weight sums are discarded when the
     // descriptor is next uploaded (the device copy may still describe an old
@@ -1413,7 +1361,6 @@ static int handle_flags(fciqmc_handle *h, int *retries)
     if (++*retries > 64) return fail(h, FCIQMC_ERR_CAPACITY, "capacity growth did not converge");
     const long long need = h->hst.need_spawn;
     const int n_over = h->hst.n_spawn_over;
-    const long long needq0 = h->hst.need_queue[0], needq1 = h->hst.need_queue[1];
     rc = reset_after_error(h);
     if (rc) return rc;
     if (err & (ERRB_SPAWN_CAP | ERRB_MAIN_CAP)) {
@@ -1430,10 +1377,6 @@ static int handle_flags(fciqmc_handle *h, int *retries)
     }
     if (err & ERRB_HEAVY_CAP) {
         rc = grow_heavy(h);
-        if (rc) return rc;
-    }
-    if (err & ERRB_QUEUE_CAP) {  // a segment of the attempt queues was too short: a quarter above the need
-        rc = ensure_queues(h, needq0 + needq0 / 4, needq1 + needq1 / 4);
         if (rc) return rc;
     }
     rc = ensure_side(h);
@@ -1826,8 +1769,6 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         max_nd = 0;
         int max_bk = 1;
         for (int i = 0; i < k; i++) {
-            int rq = ensure_queues(hs[i]);
-            if (rq) return rq;
             tab[i] = hs[i]->hi;
             tab[i].partner = pidx[i];
             max_bk = std::max(max_bk, 1 << hs[i]->bb);
@@ -1842,14 +1783,10 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         cleanup();
         cudaGraph_t g;
         CUDA_TRY(h0, cudaStreamBeginCapture(h0->stream, cudaStreamCaptureModeThreadLocal));
-        bool sp_staged = true, split = spawn_split_selected();
-        for (int i = 0; i < k; i++) {
-            sp_staged = sp_staged && staged_spawn_fits(tab[i]);
-            split = split && tab[i].qcnt != nullptr;
-        }
-        launch_spawn(dinst, dunit, k, units, sp_staged, split, h0->stream);
-        if (split && sp_staged) launch_spawn_eval(dinst, k, h0->stream);
-        launch_spawn_heavy(dinst, k, h0->stream);
+        bool adaptive = false;
+        for (int i = 0; i < k; i++) adaptive = adaptive || tab[i].adaptive;
+        launch_spawn(nullptr, dinst, dunit, k, units, adaptive, h0->stream);
+        launch_spawn_heavy(nullptr, dinst, k, h0->stream);
         if (max_nd > 0) launch_semistoch(dinst, k, max_nd, h0->stream);
         bool general = false, staged = true;
         for (int i = 0; i < k; i++) {
@@ -2229,7 +2166,7 @@ struct fciqmc_server {
 };
 
 // device memory a request needs when admitted: its initial layout and
-// integrals, the attempt queues, and the first growth of the spawn regions (to 4 CAP_S0 slots per
+// integrals, and the first growth of the spawn regions (to 4 CAP_S0 slots per
 // bucket, old and new buffers held together, with the large-bucket scratch)
 static int64_t estimate_bytes(const Request &r)
 {
@@ -2244,9 +2181,7 @@ static int64_t estimate_bytes(const Request &r)
     int tb = TABBITS;
     while ((double)(1 << tb) < 2.0 * ecap) tb++;
     const double scratch = (double)BIG_BLOCKS * (ecap * 52.0 + 4.0 * (double)(1 << tb) + 256.0);
-    // the attempt queues of split spawning at their first size
-    const double queues = 2.0 * (double)std::min(draw_segments(), 1 << bb) * (4096.0 * sizeof(QRec) + 4.0);
-    return (int64_t)((double)(1LL << bb) * per_bucket + scratch + queues + 8.0 * (N * N + ne) + 48.0 * N * N +
+    return (int64_t)((double)(1LL << bb) * per_bucket + scratch + 8.0 * (N * N + ne) + 48.0 * N * N +
                      4096.0 * 88 + 1.0e6);
 }
 

@@ -29,13 +29,16 @@ __device__ __forceinline__ int nth_set(u64 x, int k)
     return pos;
 }
 
-// floor(w * m / 2^64): an integer in [0, m)
-__device__ __forceinline__ u64 pick(u64 w, u64 m) { return __umul64hi(w, m); }
+// floor(w m / 2^64): an integer in [0, m), from two 32 x 32 products
+__device__ __forceinline__ unsigned pick(u64 w, unsigned m)
+{
+    return (unsigned)(((u64)(unsigned)(w >> 32) * m + (((u64)(unsigned)w * m) >> 32)) >> 32);
+}
 
 // x / d for x < 2^32 by the precomputed M = ceil(2^64 / d) (M = 0: d = 1):
 // x M / 2^64 = x / d + x e / (d 2^64) with 0 <= e < d, and the second term
 // is below 2^-32 < 1/d, so the floor is exact
-__device__ __forceinline__ unsigned div_by(unsigned x, u64 M) { return M ? (unsigned)__umul64hi((u64)x, M) : x; }
+__device__ __forceinline__ unsigned div_by(unsigned x, u64 M) { return M ? pick(M, x) : x; }
 
 // number of occupied spin orbitals before canonical position pos, then flip it
 __device__ __forceinline__ int flip_parity(u64 &a, u64 &b, int N, int pos)
@@ -460,7 +463,7 @@ static __device__ double diag_exact_warp(const DevInst &I, u64 a, u64 b)
 }
 
 // exact H_ii - E_ref of one determinant by one thread (the same sum as the
-// warp version, term by term)
+// warp version, term by term; loads issued four at a time)
 static __device__ double diag_exact_thread(const DevInst &I, u64 a, u64 b)
 {
     const int N = I.norb;
@@ -471,19 +474,23 @@ static __device__ double diag_exact_thread(const DevInst &I, u64 a, u64 b)
             const int p = __ffsll((long long)w) - 1;
             w &= w - 1;
             x += fx_load(I.hfx, p);
-            u64 same = w;  // higher orbitals of the same spin
-            while (same) {
-                const int q = __ffsll((long long)same) - 1;
-                same &= same - 1;
-                x += fx_load(I.JKfx, p * N + q);
-            }
-            if (!s) {
-                u64 ob = b;
-                while (ob) {
-                    const int q = __ffsll((long long)ob) - 1;
-                    ob &= ob - 1;
-                    x += fx_load(I.Jfx, p * N + q);
+            u64 same = w, other = s ? 0ULL : b;  // higher orbitals of the same spin; beta partners of alpha ones
+            while (same | other) {
+                ulonglong2 v[4];
+#pragma unroll
+                for (int r = 0; r < 4; r++) {
+                    const ulonglong2 *tab = I.JKfx;
+                    u64 &from = same ? same : other;
+                    if (!same) tab = I.Jfx;
+                    v[r] = make_ulonglong2(0, 0);
+                    if (from) {
+                        const int q = __ffsll((long long)from) - 1;
+                        from &= from - 1;
+                        v[r] = __ldg(tab + p * N + q);
+                    }
                 }
+#pragma unroll
+                for (int r = 0; r < 4; r++) x += (i128)(((u128)v[r].y << 64) | (u128)v[r].x);
             }
         }
     }

@@ -27,16 +27,14 @@ enum {
     ERRB_STOP = 64,       // the run reached its stop iteration inside a batch (not an error)
     ERRB_PAUSE_TRIAL = 128,  // iteration boundary at which the trial space must be built (not an error)
     ERRB_PARTNER = 256,      // the other replica of a pair failed this iteration: repeat it (not an error)
-    ERRB_QUEUE_CAP = 512,    // a segment of the attempt queues overflowed (split spawning)
 };
 // errors raised before the finalize kernel: a replica commits its iteration
 // only if neither it nor its partner has one
-constexpr int ERRB_STAGE = ERRB_SPAWN_CAP | ERRB_MAIN_CAP | ERRB_HEAVY_CAP | ERRB_NUMERIC | ERRB_TIMEOUT | ERRB_QUEUE_CAP;
+constexpr int ERRB_STAGE = ERRB_SPAWN_CAP | ERRB_MAIN_CAP | ERRB_HEAVY_CAP | ERRB_NUMERIC | ERRB_TIMEOUT;
 enum { DFLAG_REF = 1, DFLAG_D = 2 };
 
 // launch geometry
-constexpr int K1_THREADS = 256;
-constexpr unsigned HEAVY_ATT = 2048;  // attempts per heavy chunk
+constexpr unsigned HEAVY_ATT = 512;   // attempts per heavy slice
 constexpr int K3_THREADS = 256;
 constexpr int EMAX = 1280;            // main + spawned records staged per bucket in shared memory (3 blocks per SM)
 constexpr int CAP_M = 1024;           // main-list capacity per bucket
@@ -56,19 +54,6 @@ struct HeavyChunk {  // a slice of the attempts of one determinant with many wal
     uint32_t flags;  // bit 0: initiator, bit 1: parent in D
     uint32_t slot;   // the determinant's main-list slot (adaptive shift)
     uint32_t pad;
-};
-
-// Split spawning: every drawn attempt is queued in global memory by class
-// (0: singles and lattice hops, 1: doubles), in the segment of the drawing
-// block (bucket b of a run goes to segment b mod the draw kernel's grid), and
-// evaluated by a flat kernel with one attempt per thread.
-constexpr int NSEG_MAX = 1024;  // segments per class (the draw kernel's grid) at most
-struct QRec {  // 48 bytes
-    u64 ka, kb;      // parent
-    double cper;     // C_i / n_att
-    u64 w2, w3;      // hole word, rounding word
-    unsigned slot;   // parent's main-list slot (adaptive shift)
-    unsigned info;   // electron (single, hop) or pair e1 | e2 << 8 (double) | parent flags << 16
 };
 
 struct Partial {  // per-bucket binary64 sums of one iteration (estimators that need them)
@@ -102,7 +87,12 @@ struct SideEnt {  // one determinant of a bucket in one replica's iteration (pai
     double srej;  // spawns removed by the initiator rule (exact sum, rounded once)
 };
 
-struct IterState {  // device-resident iteration state of one run
+// Device-resident iteration state of one run.  What every warp reads at the
+// start of a kernel lies in lines of its own, apart from the counters that
+// kernels add to: a line read and written by many warps of both dies goes
+// back and forth between their L2 halves, about 50 ns each time (4096 warps
+// that each stored a word of the line they had read: 200 us).
+struct IterState {
     long long iter;
     int parity;
     int vary;
@@ -110,19 +100,18 @@ struct IterState {  // device-resident iteration state of one run
     long long shift_start;
     long long cnt;
     u64 nwl_hi, nwl_lo;     // N_w(2^32 units) at the last shift update
-    int err;
-    int heavy_n;
-    double e_den;
     long long semi_built;   // 1 once D exists
-    int big_n;              // buckets deferred to the large-bucket kernel
+    long long stop_iter;    // the finalize kernel raises ERRB_STOP when iter reaches it
+    long long trial_built;  // 1 once the trial space exists
+    alignas(128) int err;
+    alignas(128) int err_at_start;  // err when the iteration's spawning began (nonzero: the iteration was skipped)
     int need_spawn;         // largest spawn count of an overflowing bucket
     int need_main;          // largest new-list size of an overflowing bucket
     int n_spawn_over;       // buckets whose spawns overflowed
-    long long stop_iter;    // K5 raises ERRB_STOP when iter reaches it
-    long long trial_built;  // 1 once the trial space exists
-    int new_n;              // determinants created in this iteration (their H_jj is computed by k_new_diag)
-    int err_at_start;       // err when the iteration's spawning began (nonzero: the iteration was skipped)
-    int need_queue[2];      // largest count a queue segment of each class needed (split spawning)
+    double e_den;
+    alignas(128) int heavy_n;
+    alignas(128) int big_n; // buckets deferred to the large-bucket kernel
+    alignas(128) int new_n; // determinants created in this iteration (their H_jj is computed by k_new_diag)
 };
 
 struct TrialEnt;
@@ -180,10 +169,6 @@ struct DevInst {
     size_t big_stride;
     HeavyChunk *heavy;
     int heavy_cap;
-    QRec *qrec[2];          // attempt queues by class: qnseg segments of qcap[class] entries each
-    int *qcnt;              // [2 * qnseg]: entries queued per segment, singles then doubles (cleared by k_finalize)
-    int qnseg;              // segments per class
-    long long qcap[2];
     Partial *part;
     u64 *acc;  // exact totals of the iteration: NSHARD lines of ACC_STRIDE words (see ACC_*)
     IterState *st;
@@ -241,13 +226,9 @@ struct TrialEnt {
 };
 
 // host-side launchers (kernels.cu)
-void launch_spawn(const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool staged, bool split,
+void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s);
-bool spawn_split_selected();
-int draw_segments();  // the draw kernel's largest grid: a run needs min(this, buckets) queue segments
-void launch_spawn_eval(const DevInst *dinst, int n_inst, cudaStream_t s);
-bool staged_spawn_fits(const DevInst &I);
-void launch_spawn_heavy(const DevInst *dinst, int n_inst, cudaStream_t s);
+void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cudaStream_t s);
 void launch_semistoch(const DevInst *dinst, int n_inst, int max_nd, cudaStream_t s);
 cudaError_t launch_annihilate(const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool general,
                               bool staged, cudaStream_t s);

@@ -2,18 +2,14 @@
 //
 // One iteration (Eq. (4) of Guther et al. 2020) is a handful of launches over
 // the bucketed walker list of every run in the batch:
-//   spawning       (a) ceil(|C_i|) attempts per determinant, one Philox block,
+//   k_spawn        (a) ceil(|C_i|) attempts per determinant, one Philox block,
 //                  one excitation and one Slater-Condon element per attempt;
 //                  survivors of the rounding of Eq. (3) are appended to the
-//                  spawn bucket of their target.  By default split in two:
-//                  k_spawn_draw (per bucket: attempts drawn, classified and
-//                  queued in global memory) and k_spawn_eval (one queued
-//                  attempt per thread); k_spawn_staged and k_spawn do both
-//                  halves inside one per-bucket block (bucket staged by bulk
-//                  copies, or loaded plainly).
-//   k_spawn_heavy  the same for determinants with more than HEAVY_ATT walkers,
-//                  split into fixed-size slices so no block waits on one
-//                  heavily populated determinant.
+//                  spawn bucket of their target.  Every warp works alone on
+//                  32 attempts at a time.
+//   k_spawn_heavy  the same for determinants with many walkers, split into
+//                  fixed-size slices so no warp waits on one heavily
+//                  populated determinant.
 //   annihilation   (b)+(c) per bucket: the bucket's walkers and spawns in
 //                  shared memory (k_annihilate_staged: bulk copies one bucket
 //                  ahead; k_annihilate: plain loads), equal determinants
@@ -69,19 +65,35 @@ __device__ __forceinline__ bool in_D(const DevInst &I, u64 a, u64 b)
 
 // ------------------------------------------------------------------ spawning
 // One spawning attempt k from parent (pa, pb) draws the Philox block
-// (pa, pb, iteration, (k << 8) | spawn).  The block's attempts are first
-// drawn and classified (single, double, lattice hop, failed), queued in
-// shared memory by class, and then each queue is processed by whole warps, so
-// that the long exact sum of a single excitation does not stall warps of
-// doubles.  The words each attempt consumes and every decision are the same
-// as if the attempts were processed one by one.
+// (pa, pb, iteration, (k << 8) | spawn); the words an attempt consumes and
+// every decision depend on that counter alone, so attempts may be evaluated
+// in any order and by any thread.
 
+// how a kernel finds the run of a bucket: one run whose descriptor is a
+// kernel parameter (its fields are constant-bank operands), or a table of
+// runs with the first unit (bucket) of each
+struct OneRun {
+    const DevInst &I;
+    __device__ __forceinline__ const DevInst &inst(int) const { return I; }
+    __device__ __forceinline__ int find(int) const { return 0; }
+};
+struct RunTable {
+    const DevInst *__restrict__ t;
+    const int *__restrict__ start;
+    int n;
+    __device__ __forceinline__ const DevInst &inst(int ii) const { return t[ii]; }
+    __device__ __forceinline__ int find(int u) const { return find_inst(start, n, u); }
+};
+
+struct AdaptQueue;
 // what the spawning code knows about the parent beyond its key: its
 // main-list slot, the list parity and the shift at the start of the iteration
+// (aq: the warp's queue of the adaptive shift)
 struct SpawnCtx {
     unsigned pslot;
     int par;
     double S;
+    AdaptQueue *aq;
 };
 
 // 128-bit add of q to the words p[0] (low), p[1] (high)
@@ -92,12 +104,24 @@ __device__ __forceinline__ void atomic_add128(u64 *p, u128 q)
     atomicAdd((unsigned long long *)(p + 1), (unsigned long long)(hi + (old + lo < old ? 1ULL : 0ULL)));
 }
 
+// a spawn whose weight in the adaptive shift's sums is still to be found
+struct AdaptRec {
+    u64 a, b;       // target
+    double H;
+    unsigned slot;  // parent's main-list slot
+    unsigned bt;    // target's bucket
+};
+struct AdaptQueue {
+    AdaptRec r[64];  // fewer than 32 before 32 attempts are evaluated
+    unsigned n;
+};
+
 // adaptive shift (Sec. V): the weight |H_ji| / |H_jj - E_ref - S| of a spawn
 // from a non-initiator, truncated to 2^-64, into T of the parent, and into A
 // as well when the target is occupied at the start of the iteration (the
 // initiator rule accepts it); weights of 2^36 or more (|H_jj - E_ref - S| far
 // below |H_ji|) and zero denominators are left out
-__device__ __noinline__ void adaptive_account(const DevInst &I, u64 ta, u64 tb, double H, int bt, const SpawnCtx &cx)
+__device__ __forceinline__ void adaptive_account(const DevInst &I, u64 ta, u64 tb, double H, int bt, const SpawnCtx &cx)
 {
     const unsigned short *kx = I.kidx[cx.par] + (size_t)bt * KIDX;
     unsigned s = (unsigned)det_hash(ta, tb) & (unsigned)(KIDX - 1);
@@ -131,7 +155,9 @@ __device__ __noinline__ void adaptive_account(const DevInst &I, u64 ta, u64 tb, 
     if (occ) atomic_add128(acc, q);
 }
 
-// append a surviving spawn (Eq. (3) rounding of the weight ws, D -> D filter) to its bucket
+// append a surviving spawn (Eq. (3) rounding of the weight ws, D -> D filter)
+// to its bucket: initiators' spawns from the front of the bucket's region,
+// the others from its back
 __device__ __forceinline__ void emit_weight(const DevInst &I, u64 ta, u64 tb, double ws, unsigned flags, u64 w3,
                                             double H, const SpawnCtx &cx)
 {
@@ -142,23 +168,16 @@ __device__ __forceinline__ void emit_weight(const DevInst &I, u64 ta, u64 tb, do
     if (!abs_lt(ws, 0x1p31)) { atomicOr(&I.st->err, ERRB_NUMERIC); return; }
     if ((flags & 2u) && in_D(I, ta, tb)) return;  // D -> D is applied exactly
     const int bt = bucket_of(det_hash(ta, tb), I.bb);
-    if (I.adaptive && !(flags & 1u)) adaptive_account(I, ta, tb, H, bt, cx);
-    const int cap_s = I.cap_s;
-    if (flags & 1u) {
-        const int s = atomicAdd(I.scnt_i + bt, 1);
-        if (s < cap_s) {
-            const size_t o = (size_t)bt * cap_s + s;
-            I.skey[o] = make_ulonglong2(ta, tb);
-            I.sw[o] = ws;
-        }
-    } else {
-        const int s = atomicAdd(I.scnt_n + bt, 1);
-        const int slot = cap_s - 1 - s;
-        if (slot >= 0) {
-            const size_t o = (size_t)bt * cap_s + slot;
-            I.skey[o] = make_ulonglong2(ta, tb);
-            I.sw[o] = ws;
-        }
+    if (cx.aq && I.adaptive && !(flags & 1u)) {  // weighed by full warps: H_jj of a new target is ~n^2/2 loads
+        AdaptRec &r = cx.aq->r[atomicAdd(&cx.aq->n, 1u)];
+        r.a = ta; r.b = tb; r.H = H; r.slot = cx.pslot; r.bt = (unsigned)bt;
+    }
+    const bool init = flags & 1u;
+    const int s = atomicAdd((init ? I.scnt_i : I.scnt_n) + bt, 1);
+    if (s < I.cap_s) {
+        const size_t o = (size_t)bt * I.cap_s + (init ? s : I.cap_s - 1 - s);
+        I.skey[o] = make_ulonglong2(ta, tb);
+        I.sw[o] = ws;
     }
 }
 
@@ -170,168 +189,148 @@ __device__ __forceinline__ void emit_spawn(const DevInst &I, u64 ta, u64 tb, dou
     emit_weight(I, ta, tb, neg_if(true, H * (I.lam[cls] * cper)), flags, w3, H, cx);
 }
 
+// the orbitals strictly between p and q (p != q, both below 64)
+__device__ __forceinline__ u64 between(int p, int q)
+{
+    const int lo = min(p, q), hi = max(p, q);
+    return (1ULL << hi) - (2ULL << lo);
+}
+
 // lattice hop (Hubbard): electron e (drawn from w1), neighbour slot w2
-__device__ void spawn_hop_e(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, int e, u64 w2, u64 w3,
-                            const SpawnCtx &cx)
+__device__ __forceinline__ void spawn_hop_e(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, int e, u64 w2,
+                                            u64 w3, const SpawnCtx &cx)
 {
     const int sp = e >= I.na;
     u64 x = sp ? pb : pa;
     const int p = nth_set(x, sp ? e - I.na : e);
-    const int q = __ldg(I.nbr + 4 * p + (int)pick(w2, (u64)I.z));
+    const int q = __ldg(I.nbr + 4 * p + (int)pick(w2, (unsigned)I.z));
     if (q < 0 || ((x >> q) & 1ULL)) return;
-    const u64 between = p < q ? (mask_below(q) & ~mask_below(p + 1)) : (mask_below(p) & ~mask_below(q + 1));
-    const double H = neg_if(__popcll(x & between) & 1, I.tmt);
+    const double H = neg_if(__popcll(x & between(p, q)) & 1, I.tmt);
     x ^= (1ULL << p) | (1ULL << q);
     emit_spawn(I, sp ? pa : x, sp ? x : pb, H, CLS_HOP, cper, flags, w3, cx);
 }
 
 // single excitation (App. A): electron e (drawn from w1), hole of its spin w2
-__device__ void spawn_single_e(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, int e, u64 w2, u64 w3,
-                               const SpawnCtx &cx)
+__device__ __forceinline__ void spawn_single_e(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, int e,
+                                               u64 w2, u64 w3, const SpawnCtx &cx)
 {
     const int sp = e >= I.na;
     u64 x = sp ? pb : pa;
     const int i = nth_set(x, sp ? e - I.na : e);
     const int m = sp ? I.mb : I.ma;
-    const int a = nth_set(~x & I.normask, (int)pick(w2, (u64)m));
-    const u64 between = i < a ? (mask_below(a) & ~mask_below(i + 1)) : (mask_below(i) & ~mask_below(a + 1));
+    const int a = nth_set(~x & I.normask, (int)pick(w2, (unsigned)m));
     const double v = single_exact(I, pa, pb, sp, i, a);
-    const double H = neg_if(__popcll(x & between) & 1, v);
+    const double H = neg_if(__popcll(x & between(i, a)) & 1, v);
     x ^= (1ULL << i) | (1ULL << a);
     emit_spawn(I, sp ? pa : x, sp ? x : pb, H, sp ? CLS_SINGLE_B : CLS_SINGLE_A, cper, flags, w3, cx);
 }
 
-// double excitation (App. A): ordered electron pair w1, hole pair w2
-__device__ void spawn_double(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, unsigned ep, u64 w2, u64 w3,
-                       const SpawnCtx &cx)
+// double excitation (App. A): ordered electron pair ep = e1 | e2 << 8 (drawn
+// from w1), then the hole pair from w2.  Uniform generator: any pair of empty
+// orbitals of the electrons' spins.  Pre-computed heat-bath sampling: the
+// alias table of that pair of spin orbitals, bin k = floor(w2 K / 2^64), coin
+// = the low 64 bits of w2 K (top 53 bits); an occupied hole or an empty table
+// fails the attempt, and with p_gen = p_pair |H| / S the weight is
+// -sign(H) lambda_ij C_i / n_att, lambda_ij = tau S / p_pair (per table).
+// The sign: a_a+ a_b+ a_j a_i = (a_a+ a_i)(a_b+ a_j) for distinct orbitals,
+// so it is the product of the two singles' signs, the second taken in the
+// determinant the first leaves (which differs only for equal spins).
+template <bool PCHB>
+__device__ __forceinline__ void spawn_double(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, unsigned ep,
+                                             u64 w2, u64 w3, const SpawnCtx &cx)
 {
-    const int N = I.norb, na = I.na;
-    const int e1 = (int)(ep & 0xffu), e2 = (int)(ep >> 8);  // the ordered pair drawn from w1 (classify)
+    const int na = I.na;
+    const int e1 = (int)(ep & 0xffu), e2 = (int)(ep >> 8);
     const int s1 = e1 >= na, s2 = e2 >= na;
     const int o1 = nth_set(s1 ? pb : pa, s1 ? e1 - na : e1);
     const int o2 = nth_set(s2 ? pb : pa, s2 ? e2 - na : e2);
-    int P0, P1, Q0, Q1, oi, oj, oa, ob, cls;
-    u64 ta, tb;
-    if (s1 != s2) {
-        oi = s1 ? o2 : o1;
-        oj = s1 ? o1 : o2;
-        const unsigned y = (unsigned)pick(w2, (u64)(I.ma * I.mb));
-        const unsigned ya = div_by(y, I.mg_mb);
-        oa = nth_set(~pa & I.normask, (int)ya);
-        ob = nth_set(~pb & I.normask, (int)(y - ya * (unsigned)I.mb));
-        P0 = oi; P1 = N + oj; Q0 = oa; Q1 = N + ob;
-        ta = pa ^ (1ULL << oi) ^ (1ULL << oa);
-        tb = pb ^ (1ULL << oj) ^ (1ULL << ob);
-        cls = CLS_DOUBLE_AB;
+    const bool opp = s1 != s2;
+    // opposite spins: (oi, oa) alpha and (oj, ob) beta; equal spins: oi < oj, oa < ob
+    const int oi = opp ? (s1 ? o2 : o1) : min(o1, o2), oj = opp ? (s1 ? o1 : o2) : max(o1, o2);
+    const u64 xi = (!opp && s1) ? pb : pa, xj = (opp || s1) ? pb : pa;  // the words oi and oj are in
+    int oa, ob;
+    double lamS = 0.0;
+    if (PCHB) {
+        const int N = I.norb;
+        int t, K;
+        u64 off;
+        if (opp) {
+            t = oi * N + oj;
+            K = N * N;
+            off = (u64)t * (u64)K;
+        } else {
+            const int p = oj * (oj - 1) / 2 + oi;
+            t = N * N + p;
+            K = N * (N - 1) / 2;
+            off = I.pchb_ss_base + (u64)p * (u64)K;
+        }
+        const double2 mt = __ldg(I.pchb_meta + t);
+        if (!(dbits(mt.y) != 0)) return;  // S = 0: nothing to propose
+        lamS = mt.x;
+        const u64 low = w2 * (u64)K;
+        const ulonglong2 e = __ldg(I.pchb_ent + off + pick(w2, (unsigned)K));
+        const unsigned hp = ((low >> 11) < e.x) ? (unsigned)(e.y & 0xffffu) : (unsigned)((e.y >> 16) & 0xffffu);
+        oa = (int)(hp & 0xffu);
+        ob = (int)(hp >> 8);
+        if (((xi >> oa) & 1ULL) || ((xj >> ob) & 1ULL)) return;
     } else {
-        const int m = s1 ? I.mb : I.ma;
-        u64 x = s1 ? pb : pa;
-        const unsigned y = (unsigned)pick(w2, (u64)(m * (m - 1)));
-        const unsigned yh = div_by(y, s1 ? I.mg_mb1 : I.mg_ma1);
-        const int h1 = (int)yh, rr = (int)(y - yh * (unsigned)(m - 1));
-        const int h2 = rr + (rr >= h1 ? 1 : 0);
-        const int q1 = nth_set(~x & I.normask, h1), q2 = nth_set(~x & I.normask, h2);
-        oi = min(o1, o2); oj = max(o1, o2); oa = min(q1, q2); ob = max(q1, q2);
-        const int off = s1 ? N : 0;
-        P0 = off + oi; P1 = off + oj; Q0 = off + oa; Q1 = off + ob;
-        x ^= (1ULL << oi) | (1ULL << oj) | (1ULL << oa) | (1ULL << ob);
-        ta = s1 ? pa : x;
-        tb = s1 ? x : pb;
-        cls = s1 ? CLS_DOUBLE_BB : CLS_DOUBLE_AA;
+        // two different holes of one spin are drawn as an ordered pair (h1, rank among the others)
+        const unsigned d = opp ? (unsigned)I.mb : (unsigned)((s1 ? I.mb : I.ma) - 1);
+        const unsigned tot = opp ? (unsigned)(I.ma * I.mb) : d * (d + 1u);
+        const unsigned y = pick(w2, tot);
+        const unsigned yh = div_by(y, opp ? I.mg_mb : (s1 ? I.mg_mb1 : I.mg_ma1));
+        const unsigned rr = y - yh * d;
+        const int q1 = nth_set(~xi & I.normask, (int)yh);
+        const int q2 = nth_set(~xj & I.normask, (int)(rr + (!opp && rr >= yh ? 1u : 0u)));
+        oa = opp ? q1 : min(q1, q2);
+        ob = opp ? q2 : max(q1, q2);
     }
-    u64 xa = pa, xb = pb;
-    int par = flip_parity(xa, xb, N, P0);
-    par ^= flip_parity(xa, xb, N, P1);
-    par ^= flip_parity(xa, xb, N, Q1);
-    par ^= flip_parity(xa, xb, N, Q0);
-    const double v = (cls == CLS_DOUBLE_AB) ? eri4(I, oa, oi, ob, oj) : eri4(I, oa, oi, ob, oj) - eri4(I, oa, oj, ob, oi);
-    emit_spawn(I, ta, tb, neg_if(par, v), cls, cper, flags, w3, cx);
+    const u64 fi = (1ULL << oi) | (1ULL << oa), fj = (1ULL << oj) | (1ULL << ob);
+    const u64 yi = opp ? xi : xi ^ fj;  // oi -> oa follows oj -> ob
+    const int par = (__popcll(xj & between(oj, ob)) ^ __popcll(yi & between(oi, oa))) & 1;
+    const u64 ta = pa ^ (opp ? fi : (s1 ? 0ULL : fi ^ fj)), tb = pb ^ (opp ? fj : (s1 ? fi ^ fj : 0ULL));
+    double v = eri4(I, oa, oi, ob, oj);
+    if (!opp) v = v - eri4(I, oa, oj, ob, oi);
+    const double H = neg_if(par, v);
+    if (PCHB) {
+        if (is_zero(H)) return;
+        emit_weight(I, ta, tb, neg_if(!(dbits(H) & SIGN64), lamS * cper), flags, w3, H, cx);
+    } else {
+        emit_spawn(I, ta, tb, H, opp ? CLS_DOUBLE_AB : (s1 ? CLS_DOUBLE_BB : CLS_DOUBLE_AA), cper, flags, w3, cx);
+    }
 }
 
-// heat-bath double (App. A, pre-computed heat-bath sampling): ordered electron
-// pair w1 as in the uniform generator, then the alias table of that pair of
-// spin orbitals: bin k = floor(w2 K / 2^64), coin = the low 64 bits of w2 K
-// (top 53 bits); an occupied hole or an empty table fails the attempt.  With
-// p_gen = p_pair |H| / S the weight is -sign(H) lambda_ij C_i / n_att,
-// lambda_ij = tau S / p_pair (stored per table).
-__device__ void spawn_double_pchb(const DevInst &I, u64 pa, u64 pb, double cper, unsigned flags, unsigned ep, u64 w2,
-                                  u64 w3, const SpawnCtx &cx)
+// How the attempts of a kernel are generated: the runs of a batch may differ
+// (GEN_ANY looks at each run), a kernel of one run holds that run's code only
+// (smaller code: the warps of the spawning kernel are at different places of
+// it, and instruction fetch was its largest stall).
+enum { GEN_UNIFORM = 0, GEN_PCHB = 1, GEN_HOP = 2, GEN_ANY = 3 };
+template <int GEN>
+__device__ __forceinline__ bool gen_is(const DevInst &I, int g)
 {
-    const int N = I.norb, na = I.na;
-    const int e1 = (int)(ep & 0xffu), e2 = (int)(ep >> 8);  // the ordered pair drawn from w1 (classify)
-    const int s1 = e1 >= na, s2 = e2 >= na;
-    const int o1 = nth_set(s1 ? pb : pa, s1 ? e1 - na : e1);
-    const int o2 = nth_set(s2 ? pb : pa, s2 ? e2 - na : e2);
-    int oi, oj, t, K;
-    u64 off;
-    if (s1 != s2) {
-        oi = s1 ? o2 : o1;  // alpha electron
-        oj = s1 ? o1 : o2;  // beta electron
-        t = oi * N + oj;
-        K = N * N;
-        off = (u64)t * (u64)K;
-    } else {
-        oi = min(o1, o2);
-        oj = max(o1, o2);
-        const int p = oj * (oj - 1) / 2 + oi;
-        t = N * N + p;
-        K = N * (N - 1) / 2;
-        off = I.pchb_ss_base + (u64)p * (u64)K;
-    }
-    const double2 mt = __ldg(I.pchb_meta + t);
-    if (!(dbits(mt.y) != 0)) return;  // S = 0: nothing to propose
-    const u64 k = __umul64hi(w2, (u64)K), low = w2 * (u64)K;
-    const ulonglong2 e = __ldg(I.pchb_ent + off + k);
-    const unsigned hp = ((low >> 11) < e.x) ? (unsigned)(e.y & 0xffffu) : (unsigned)((e.y >> 16) & 0xffffu);
-    const int oa = (int)(hp & 0xffu), ob = (int)(hp >> 8);
-    int P0, P1, Q0, Q1, cls;
-    u64 ta, tb;
-    if (s1 != s2) {
-        if (((pa >> oa) & 1ULL) || ((pb >> ob) & 1ULL)) return;
-        P0 = oi; P1 = N + oj; Q0 = oa; Q1 = N + ob;
-        ta = pa ^ (1ULL << oi) ^ (1ULL << oa);
-        tb = pb ^ (1ULL << oj) ^ (1ULL << ob);
-        cls = CLS_DOUBLE_AB;
-    } else {
-        u64 x = s1 ? pb : pa;
-        if (((x >> oa) & 1ULL) || ((x >> ob) & 1ULL)) return;
-        const int sh = s1 ? N : 0;
-        P0 = sh + oi; P1 = sh + oj; Q0 = sh + oa; Q1 = sh + ob;
-        x ^= (1ULL << oi) | (1ULL << oj) | (1ULL << oa) | (1ULL << ob);
-        ta = s1 ? pa : x;
-        tb = s1 ? x : pb;
-        cls = s1 ? CLS_DOUBLE_BB : CLS_DOUBLE_AA;
-    }
-    u64 xa = pa, xb = pb;
-    int par = flip_parity(xa, xb, N, P0);
-    par ^= flip_parity(xa, xb, N, P1);
-    par ^= flip_parity(xa, xb, N, Q1);
-    par ^= flip_parity(xa, xb, N, Q0);
-    const double v = (cls == CLS_DOUBLE_AB) ? eri4(I, oa, oi, ob, oj) : eri4(I, oa, oi, ob, oj) - eri4(I, oa, oj, ob, oi);
-    const double H = neg_if(par, v);
-    if (is_zero(H)) return;
-    const double wv = mt.x * cper;
-    emit_weight(I, ta, tb, neg_if(!(dbits(H) & SIGN64), wv), flags, w3, H, cx);
+    if (GEN != GEN_ANY) return GEN == g;
+    return g == GEN_HOP ? I.kind == FCIQMC_HUBBARD : (I.kind != FCIQMC_HUBBARD && (I.pchb != 0) == (g == GEN_PCHB));
 }
 
 // class of one attempt from its first two words, or -1 for a failed attempt;
 // *ep = the electron of a single or a hop, or for a double e1 | e2 << 8 (the
 // ordered electron pair), all drawn from w1
-enum { Q_DOUBLE = 0, Q_SINGLE = 1, Q_HOP = 2, NQ = 3 };
-__device__ __forceinline__ int classify(const DevInst &I, u64 pa, u64 pb, u64 w0, u64 w1, unsigned *ep)
+enum { Q_DOUBLE = 0, Q_SINGLE = 1, Q_HOP = 2 };
+template <int GEN>
+__device__ __forceinline__ int classify(const DevInst &I, u64 w0, u64 w1, unsigned *ep)
 {
-    if (I.kind == FCIQMC_HUBBARD) {
-        *ep = (unsigned)pick(w1, (u64)I.n);  // the electron that hops
+    const int n = I.n;
+    const bool hop = gen_is<GEN>(I, GEN_HOP), single = !hop && (w0 >> 11) < I.tsingle;
+    const unsigned xe = pick(w1, (unsigned)(hop || single ? n : n * (n - 1)));
+    if (hop) {
+        *ep = xe;
         return Q_HOP;
     }
-    if ((w0 >> 11) < I.tsingle) {
-        const int e = (int)pick(w1, (u64)I.n);
-        *ep = (unsigned)e;  // the excited electron
-        return (e >= I.na ? I.mb : I.ma) == 0 ? -1 : Q_SINGLE;
+    if (single) {
+        *ep = xe;
+        return ((int)xe >= I.na ? I.mb : I.ma) == 0 ? -1 : Q_SINGLE;
     }
-    const int n = I.n;
     if (n < 2) return -1;
-    const unsigned xe = (unsigned)pick(w1, (u64)(n * (n - 1)));
     const unsigned q1 = div_by(xe, I.mg_n1);
     const int e1 = (int)q1, r = (int)(xe - q1 * (unsigned)(n - 1));
     const int e2 = r + (r >= e1 ? 1 : 0);
@@ -341,344 +340,392 @@ __device__ __forceinline__ int classify(const DevInst &I, u64 pa, u64 pb, u64 w0
     return (s1 ? I.mb : I.ma) < 2 ? -1 : Q_DOUBLE;
 }
 
-// Division of C_i by n_att > 1 (binary64, correctly rounded) occupies the
-// binary64 pipe for a whole warp's turn whatever its active lanes, so the
-// determinants that need it are listed (one warp-aggregated shared atomic)
-// and divided afterwards by full warps.
-template <typename SM>
-__device__ __forceinline__ void queue_div(SM &S, bool dv, int d, int lane)
+// The spawning kernel.  Every warp works alone: it takes tiles of 32 list
+// slots, appends the occupied ones to a ring of parents in shared memory with
+// a running number of attempts, and evaluates 32 attempts at a time, one per
+// lane, whatever tiles (and buckets) their parents came from.  Doubles and
+// hops are evaluated where they are drawn; singles, whose exact sum is ten
+// times as long, wait in a queue of the warp until there are 32 of them.
+// Parents whose C / n_att needs a binary64 division (n_att not a power of two;
+// the division costs a whole warp's turn whatever its active lanes) wait too.
+// There is no block barrier and an attempt never leaves the chip: at 7.3e7
+// determinants and 9.1e7 attempts (50 orbitals) a block-per-bucket draw with
+// 48-byte attempt records in global memory and a second kernel for the
+// evaluation took 8.6 ms.
+constexpr int SP_THREADS = 256, SP_WARPS = SP_THREADS / 32, RING = 64;
+constexpr int CHUNK_S = 512;  // attempts per slice of a heavily populated determinant
+static_assert(HEAVY_ATT == (unsigned)CHUNK_S, "heavy slices");
+
+struct SpawnRec {    // a drawn single excitation
+    u64 ka, kb;      // parent
+    double cper;     // C_i / n_att
+    u64 w2, w3;      // hole word, rounding word
+    unsigned slot;   // parent's main-list slot (adaptive shift)
+    unsigned info;   // electron | parent flags << 16
+};
+struct SpawnWarp {
+    ulonglong2 key[RING];    // ring of parents: the pending ones hold fewer than 32
+    double cper[RING];       // attempts before a tile of at most 32 more is appended
+    unsigned off[RING];      // running number of the parent's first attempt
+    unsigned slot[RING];
+    SpawnRec q[RING];        // singles waiting (fewer than 32 before 32 attempts are drawn)
+    unsigned divq[RING];     // slots waiting for their division
+    unsigned char fl[RING];  // initiator | in-D bits
+};
+
+struct SpawnRun {  // the run a warp works on, at the start of the iteration
+    long long it;
+    double S;
+    int par;
+    AdaptQueue *aq;  // the warp's queue of the adaptive shift (NULL: no run of the launch uses it)
+};
+
+constexpr size_t SP_SMEM = SP_WARPS * sizeof(SpawnWarp), SP_SMEM_ADAPT = SP_SMEM + SP_WARPS * sizeof(AdaptQueue);
+static_assert(4 * (SP_SMEM + 1024) <= 233472 && 3 * (SP_SMEM_ADAPT + 1024) <= 233472, "resident spawning blocks per SM");
+
+// up to 32 of the spawns that wait to be weighed
+__device__ __forceinline__ void eval_adaptive(const DevInst &I, const SpawnRun &R)
 {
-    const unsigned md = __ballot_sync(0xffffffffu, dv);
-    if (!md) return;
-    int b0 = 0;
-    if (lane == 0) b0 = atomicAdd(&S.ndiv, __popc(md));
-    b0 = __shfl_sync(0xffffffffu, b0, 0);
-    if (dv) S.divl[b0 + __popc(md & ((1u << lane) - 1u))] = (unsigned short)d;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    const unsigned q = R.aq->n, n = min(q, 32u);
+    if (lane < n) {
+        const AdaptRec r = R.aq->r[q - n + lane];
+        adaptive_account(I, r.a, r.b, r.H, (int)r.bt, SpawnCtx{r.slot, R.par, R.S, nullptr});
+    }
+    __syncwarp();
+    if (lane == 0) R.aq->n = q - n;
+    __syncwarp();
 }
 
-// C / n_att in place for the listed determinants i0, i0 + stride, ...
-__device__ __forceinline__ void divide_listed(const unsigned short *divl, int nd, double *c, int i0, int stride)
+// up to 32 queued singles, from the end of the queue
+__device__ __forceinline__ void eval_singles(const DevInst &I, SpawnWarp &W, int &nq, const SpawnRun &R)
 {
-    for (int i = i0; i < nd; i += stride) {
-        const int d = divl[i];
-        const double x = c[d];
-        c[d] = x / (double)ceil_abs(x);
+    const int lane = threadIdx.x & 31;
+    const int n = min(nq, 32);
+    __syncwarp();
+    if (lane < n) {
+        const SpawnRec r = W.q[nq - n + lane];
+        const SpawnCtx cx{r.slot, R.par, R.S, R.aq};
+        spawn_single_e(I, r.ka, r.kb, r.cper, r.info >> 16, (int)(r.info & 0xffffu), r.w2, r.w3, cx);
+    }
+    nq -= n;
+    __syncwarp();
+}
+
+// one attempt per lane (lanes with `on`): draw, classify, evaluate or queue
+template <int GEN>
+__device__ __forceinline__ void attempts32(const DevInst &I, SpawnWarp &W, int &nq, const SpawnRun &R, bool on,
+                                           ulonglong2 key, u64 k, double cper, unsigned fl, unsigned slot)
+{
+    const int lane = threadIdx.x & 31;
+    u64 w[4];
+    philox(key.x, key.y, (u64)R.it, (k << 8) | (u64)PURPOSE_SPAWN, I.seed, I.replica, w);
+    unsigned ep = 0;
+    int cls = classify<GEN>(I, w[0], w[1], &ep);
+    if (!on) cls = -1;
+    const SpawnCtx cx{slot, R.par, R.S, R.aq};
+    if (!gen_is<GEN>(I, GEN_HOP)) {
+        const unsigned ms = __ballot_sync(0xffffffffu, cls == Q_SINGLE);
+        if (cls == Q_SINGLE) {
+            SpawnRec &r = W.q[nq + __popc(ms & ((1u << lane) - 1u))];
+            r.ka = key.x; r.kb = key.y; r.cper = cper; r.w2 = w[2]; r.w3 = w[3]; r.slot = slot; r.info = ep | (fl << 16);
+        }
+        nq += __popc(ms);
+        if (cls == Q_DOUBLE) {
+            if (gen_is<GEN>(I, GEN_PCHB)) spawn_double<true>(I, key.x, key.y, cper, fl, ep, w[2], w[3], cx);
+            else spawn_double<false>(I, key.x, key.y, cper, fl, ep, w[2], w[3], cx);
+        }
+    } else if (cls == Q_HOP) {
+        spawn_hop_e(I, key.x, key.y, cper, fl, (int)ep, w[2], w[3], cx);
     }
 }
 
-constexpr int CHUNK = 1024;  // attempts drawn and queued per round
-struct SpawnRec {
-    u64 w2, w3;
-    unsigned det;
-    unsigned ep;  // electron (single, hop) or electron pair (double) drawn from w1 (classify)
+struct SpawnCursor {       // running numbers: ring entries [r0, r1) pending, attempts [done, tot)
+    unsigned r0, r1, done, tot;
+    int nq, nd;            // singles and divisions waiting
 };
-struct K1Smem {
-    static constexpr int chunk = CHUNK;
-    ulonglong2 key[CAP_M];
-    double cper[CAP_M];
-    unsigned off[CAP_M + 1];
-    unsigned short att_det[CHUNK];  // parent of attempt a < CHUNK of a bucket, 0xffff: look it up in off[]
-    unsigned char fl[CAP_M];
-    SpawnRec rec[CHUNK];
-    unsigned short divl[CAP_M];  // determinants whose C / n_att (n_att > 1) is still to be divided
-    int ndiv;
-    int qn[NQ];
-    int next;  // evaluation counter of the chunk
-    unsigned wsum[K1_THREADS / 32];
-    int hdr_err, hdr_par;
-    long long hdr_it;
-    double hdr_S;
-};
-static_assert(3 * (sizeof(K1Smem) + 1024) <= 233472, "three spawn blocks per SM (228 KB, 1 KB reserved per block)");
 
-// draw and classify attempts a0 .. a1-1 of a bucket (attempt a of parent
-// `det`, slot k) and queue them by class in S.rec: doubles from the front,
-// singles and hops from the back (hops only exist without the others), with
-// the counts in qn[Q_DOUBLE], qn[Q_SINGLE] (zero on entry); each thread
-// draws two attempts per round, so that the two Philox evaluations overlap
-template <typename MAP, typename SM>
-__device__ __forceinline__ void draw_classify(const DevInst &I, SM &S, long long it, unsigned a0, unsigned a1,
-                                              const MAP &map, int *qn)
+// 32 pending attempts (or the last ones): lane l takes attempt done + l, whose
+// parent is found from the pending entries that start inside the window
+template <int GEN>
+__device__ __forceinline__ void spawn_window(const DevInst &I, SpawnWarp &W, SpawnCursor &C, const SpawnRun &R)
 {
-    constexpr int CHUNK = SM::chunk;
-    const int t = threadIdx.x, lane = t & 31;
-    for (unsigned ab = a0; ab < a1; ab += 2 * K1_THREADS) {
-        u64 w[2][4];
-        unsigned det[2], ep[2];
-        int cls[2];
+    const int lane = threadIdx.x & 31;
+    unsigned bit = 0;
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const unsigned a = ab + h * K1_THREADS + t;
-            cls[h] = -1;
-            det[h] = 0;
-            ep[h] = 0;
-            if (ab + h * K1_THREADS + (unsigned)(t & ~31) < a1) {  // a warp with no attempt left draws nothing
-                const unsigned ac = a < a1 ? a : a1 - 1;           // clamped: drawn, then discarded
-                u64 k;
-                det[h] = map.det_of(ac, k);
-                const ulonglong2 kk = map.key(det[h]);
-                philox(kk.x, kk.y, (u64)it, (k << 8) | (u64)PURPOSE_SPAWN, I.seed, I.replica, w[h]);
-                const int q = classify(I, kk.x, kk.y, w[h][0], w[h][1], &ep[h]);
-                cls[h] = a < a1 ? q : -1;
-            }
+    for (int h = 0; h < 2; h++) {
+        const unsigned j = (unsigned)(h * 32 + lane);
+        if (j < C.r1 - C.r0) {
+            const unsigned o = W.off[(C.r0 + j) & (RING - 1)] - C.done;
+            if (o - 1u < 31u) bit |= 1u << o;  // o in 1 .. 31 (the entry at r0 starts at or before `done`)
         }
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const bool front = cls[h] == Q_DOUBLE, back = cls[h] == Q_SINGLE || cls[h] == Q_HOP;
-            const unsigned mf = __ballot_sync(0xffffffffu, front), mb = __ballot_sync(0xffffffffu, back);
-            int bf = 0, bk = 0;
-            if (lane == 0) {
-                if (mf) bf = atomicAdd(&qn[Q_DOUBLE], __popc(mf));
-                if (mb) bk = atomicAdd(&qn[Q_SINGLE], __popc(mb));
-            }
-            bf = __shfl_sync(0xffffffffu, bf, 0);
-            bk = __shfl_sync(0xffffffffu, bk, 0);
-            const unsigned below = (1u << lane) - 1u;
-            if (front || back) {
-                const int slot = front ? bf + __popc(mf & below) : CHUNK - 1 - (bk + __popc(mb & below));
-                SpawnRec &r = S.rec[slot];
-                r.w2 = w[h][2]; r.w3 = w[h][3]; r.det = det[h]; r.ep = ep[h];
-            }
-        }
+    }
+    const unsigned m = __reduce_or_sync(0xffffffffu, bit);
+    const unsigned r = (C.r0 + __popc(m & (0xffffffffu >> (31 - lane)))) & (RING - 1);
+    const bool on = C.done + lane - C.tot >= 0x80000000u;
+    attempts32<GEN>(I, W, C.nq, R, on, W.key[r], (u64)(C.done + lane - W.off[r]), W.cper[r], W.fl[r], W.slot[r]);
+    C.done += 32;
+    if (C.tot - C.done - 1u >= 0x7fffffffu) {  // done >= tot: nothing is pending
+        C.done = C.tot;
+        C.r0 = C.r1;
+    } else {
+        C.r0 += __popc(m);
+        if (C.r0 + 1 != C.r1 && W.off[(C.r0 + 1) & (RING - 1)] == C.done) C.r0++;
     }
 }
 
-// draw and classify the attempts of a bucket chunk by chunk, queue them by
-// class, then evaluate them: warps take 32 queued attempts at a time from a
-// shared counter, singles (the long exact sums) first, so that no warp idles
-// at the chunk's closing barrier while others still hold a long queue
-template <typename MAP, typename SM>
-__device__ void run_attempts(const DevInst &I, SM &S, long long it, unsigned A, MAP map, int par, double shift)
+// the lanes' parents (valid lanes, nat >= 1 attempts each) into the ring
+__device__ __forceinline__ void spawn_append(SpawnWarp &W, SpawnCursor &C, bool valid, ulonglong2 key, unsigned nat,
+                                             double cper, unsigned fl, unsigned slot)
 {
-    constexpr int CHUNK = SM::chunk;
-    const int t = threadIdx.x, lane = t & 31;
-    for (unsigned a0 = 0; a0 < A; a0 += CHUNK) {
-        const unsigned a1 = min(A, a0 + CHUNK);
-        if (t < NQ) S.qn[t] = 0;
-        if (t == 0) S.next = 0;
-        __syncthreads();
-        draw_classify(I, S, it, a0, a1, map, S.qn);
-        __syncthreads();
-        const int nd = S.qn[Q_DOUBLE], ns = S.qn[Q_SINGLE], ntot = ns + nd;
-        while (true) {
-            int g = 0;
-            if (lane == 0) g = atomicAdd(&S.next, 32);
-            g = __shfl_sync(0xffffffffu, g, 0);
-            if (g >= ntot) break;
-            const int q = g + lane;
-            if (q < ns) {
-                const SpawnRec r = S.rec[CHUNK - 1 - q];
-                const unsigned d = r.det;
-                const ulonglong2 kk = map.key(d);
-                const SpawnCtx cx{map.slot(d), par, shift};
-                const int e = (int)r.ep;
-                if (I.kind == FCIQMC_HUBBARD)
-                    spawn_hop_e(I, kk.x, kk.y, map.cper(d), map.flags(d), e, r.w2, r.w3, cx);
-                else spawn_single_e(I, kk.x, kk.y, map.cper(d), map.flags(d), e, r.w2, r.w3, cx);
-            } else if (q < ntot) {
-                const SpawnRec r = S.rec[q - ns];
-                const unsigned d = r.det;
-                const ulonglong2 kk = map.key(d);
-                const SpawnCtx cx{map.slot(d), par, shift};
-                if (I.pchb) spawn_double_pchb(I, kk.x, kk.y, map.cper(d), map.flags(d), r.ep, r.w2, r.w3, cx);
-                else spawn_double(I, kk.x, kk.y, map.cper(d), map.flags(d), r.ep, r.w2, r.w3, cx);
-            }
-        }
-        __syncthreads();
-    }
-}
-
-struct BucketMap {
-    const K1Smem *S;
-    __device__ unsigned det_of(unsigned a, u64 &k) const
-    {
-        if (a < (unsigned)CHUNK) {
-            const unsigned d = S->att_det[a];
-            if (d != 0xffffu) {
-                k = a - S->off[d];
-                return d;
-            }
-        }
-        int lo = 0, hi = CAP_M;  // largest d with off[d] <= a (off[CAP_M] = total > a)
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (S->off[mid] <= a) lo = mid; else hi = mid;
-        }
-        k = a - S->off[lo];
-        return (unsigned)lo;
-    }
-    __device__ ulonglong2 key(unsigned d) const { return S->key[d]; }
-    __device__ double cper(unsigned d) const { return S->cper[d]; }
-    __device__ unsigned flags(unsigned d) const { return S->fl[d]; }
-    __device__ unsigned slot(unsigned d) const { return base + d; }
-    unsigned base;
-};
-
-// attempts k0 .. k0+count-1 of one heavy determinant
-struct HeavyMap {
-    HeavyChunk h;
-    __device__ unsigned det_of(unsigned a, u64 &k) const { k = h.k0 + a; return 0; }
-    __device__ ulonglong2 key(unsigned) const { return make_ulonglong2(h.a, h.b); }
-    __device__ double cper(unsigned) const { return h.cper; }
-    __device__ unsigned flags(unsigned) const { return h.flags; }
-    __device__ unsigned slot(unsigned) const { return h.slot; }
-};
-
-__global__ void __launch_bounds__(K1_THREADS, 3) k_spawn(const DevInst *__restrict__ insts, const int *__restrict__ unit_start,
-                                                      int n_inst, int n_units)
-{
-    extern __shared__ __align__(16) unsigned char k1_raw[];
-    K1Smem &S = *reinterpret_cast<K1Smem *>(k1_raw);
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    constexpr int PER = CAP_M / K1_THREADS;
-    // the run's state at the start of the iteration, read once per run a
-    // block meets (a flag raised by another block during this kernel makes the
-    // host repeat the iteration, whose output is then discarded)
-    int cur = -1, err = 0, par = 0;
-    long long it = 0;
-    double shift = 0.0;
-    if (t == 0) S.ndiv = 0;  // visible after the first run header's barrier
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
-        const int ii = find_inst(unit_start, n_inst, u);
-        const DevInst &I = insts[ii];
-        if (ii != cur) {
-            if (t == 0) {
-                S.hdr_err = *(volatile int *)&I.st->err;
-                S.hdr_par = I.st->parity;
-                S.hdr_it = I.st->iter;
-                S.hdr_S = I.st->S;
-                I.st->err_at_start = S.hdr_err;  // the same value from every block of the run
-            }
-            __syncthreads();
-            err = S.hdr_err;
-            par = S.hdr_par;
-            it = S.hdr_it;
-            shift = S.hdr_S;
-            cur = ii;
-            __syncthreads();
-        }
-        if (err) continue;
-        const int b = u - I.unit0;
-        const int m = I.cnt[par][b];
-        const size_t base = (size_t)b * CAP_M;
-        // load the bucket: thread t owns determinants PER*t .. PER*t+PER-1
-        long long att = 0;
-        unsigned mine = 0;
-        unsigned nl[PER];
-        for (int j = 0; j < PER; j++) {
-            const int d = PER * t + j;
-            nl[j] = 0;
-            bool dv = false;
-            if (d < m) {
-                const ulonglong2 kk = I.key[par][base + d];
-                const double c = I.c[par][base + d];
-                const uint8_t f = I.fl[par][base + d];
-                unsigned fl = 0;
-                double cper = 0.0;
-                u64 nat = 0;
-                if (!is_zero(c)) {
-                    if (!abs_lt(c, 0x1p31)) {
-                        atomicOr(&I.st->err, ERRB_NUMERIC);
-                    } else {
-                        nat = ceil_abs(c);
-                        const bool init = (dbits(c) & ~SIGN64) > dbits(I.n_a) || (f & (DFLAG_REF | DFLAG_D));
-                        fl = (init ? 1u : 0u) | ((f & DFLAG_D) ? 2u : 0u);
-                        cper = c;  // C / n_att: below for n_att > 1 (c / 1 is c)
-                        att += (long long)nat;
-                        if (nat > HEAVY_ATT) {  // sliced into the heavy queue
-                            cper = c / (double)nat;
-                            const unsigned nch = (unsigned)((nat + HEAVY_ATT - 1) / HEAVY_ATT);
-                            const int q0 = atomicAdd(&I.st->heavy_n, (int)nch);
-                            if ((long long)q0 + nch > (long long)I.heavy_cap) atomicOr(&I.st->err, ERRB_HEAVY_CAP);
-                            else
-                                for (unsigned q = 0; q < nch; q++) {
-                                    HeavyChunk h;
-                                    h.a = kk.x; h.b = kk.y; h.cper = cper; h.k0 = (u64)q * HEAVY_ATT;
-                                    const u64 left = nat - h.k0;
-                                    h.count = (unsigned)(left < HEAVY_ATT ? left : HEAVY_ATT);
-                                    h.flags = fl;
-                                    h.slot = (uint32_t)(base + d);
-                                    h.pad = 0;
-                                    I.heavy[q0 + q] = h;
-                                }
-                        } else {
-                            nl[j] = (unsigned)nat;
-                            dv = nat > 1;
-                        }
-                    }
-                }
-                S.key[d] = kk;
-                S.cper[d] = cper;
-                S.fl[d] = (unsigned char)fl;
-                mine += nl[j];
-            }
-            queue_div(S, dv, d, lane);
-        }
-        // the parents of the first CHUNK attempts, written below by the
-        // determinants with few attempts; the others are found by bisection
-        for (int q = t; q < CHUNK; q += K1_THREADS) S.att_det[q] = 0xffffu;
-        // exclusive scan of the light attempt counts in determinant order
-        unsigned v = mine;
+    const int lane = threadIdx.x & 31;
+    const unsigned mv = __ballot_sync(0xffffffffu, valid), below = (1u << lane) - 1u;
+    const unsigned many = __ballot_sync(0xffffffffu, valid && nat > 1);
+    const unsigned pos = (unsigned)__popc(mv & below);
+    unsigned ex = pos, total = (unsigned)__popc(mv);
+    if (many) {
+        unsigned v = valid ? nat : 0u;
+        const unsigned mine = v;
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
             if (lane >= o) v += y;
         }
-        if (lane == 31) S.wsum[warp] = v;
-        __syncthreads();
-        if (warp == 0) {
-            unsigned x = lane < K1_THREADS / 32 ? S.wsum[lane] : 0u;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (lane < K1_THREADS / 32) S.wsum[lane] = x;
-        } else {
-            divide_listed(S.divl, S.ndiv, S.cper, t - 32, K1_THREADS - 32);  // warp 0 scans meanwhile
-        }
-        __syncthreads();
-        if (t == 0) S.ndiv = 0;  // read by every thread before the barrier above
-        unsigned ex = v - mine + (warp ? S.wsum[warp - 1] : 0u);
-        for (int j = 0; j < PER; j++) {
-            S.off[PER * t + j] = ex;
-            if (nl[j] <= 8u && ex + nl[j] <= (unsigned)CHUNK)
-                for (unsigned q = 0; q < nl[j]; q++) S.att_det[ex + q] = (unsigned short)(PER * t + j);
-            ex += nl[j];
-        }
-        if (t == K1_THREADS - 1) S.off[CAP_M] = ex;
-        __syncthreads();
-        const unsigned total = S.off[CAP_M];
-        BucketMap map{&S, (unsigned)base};
-        run_attempts(I, S, it, total, map, par, shift);
-        // attempts of this bucket (light and heavy) into the run's exact total
-        for (int o = 16; o >= 1; o >>= 1) att += __shfl_xor_sync(0xffffffffu, att, o);
-        if (lane == 0 && att) red_add(&I.acc[(b % NSHARD) * ACC_STRIDE + ACC_ATT], (u64)att);
+        ex = v - mine;
+        total = __shfl_sync(0xffffffffu, v, 31);
+    }
+    __syncwarp();
+    if (valid) {
+        const unsigned r = (C.r1 + pos) & (RING - 1);
+        W.key[r] = key;
+        W.cper[r] = cper;
+        W.off[r] = C.tot + ex;
+        W.slot[r] = slot;
+        W.fl[r] = (unsigned char)fl;
+    }
+    __syncwarp();
+    C.r1 += (unsigned)__popc(mv);
+    C.tot += total;
+}
+
+// slices of a determinant with more attempts than one warp should draw
+__device__ __noinline__ void queue_heavy(const DevInst &I, ulonglong2 kk, double c, unsigned nat, unsigned fl, unsigned slot)
+{
+    const double ch = c / (double)nat;
+    const unsigned nch = (nat + HEAVY_ATT - 1) / HEAVY_ATT;
+    const int q0 = atomicAdd(&I.st->heavy_n, (int)nch);
+    if ((long long)q0 + nch > (long long)I.heavy_cap) {
+        atomicOr(&I.st->err, ERRB_HEAVY_CAP);
+        return;
+    }
+    for (unsigned q = 0; q < nch; q++) {
+        HeavyChunk h;
+        h.a = kk.x; h.b = kk.y; h.cper = ch; h.k0 = (u64)q * HEAVY_ATT;
+        const unsigned left = nat - q * HEAVY_ATT;
+        h.count = left < HEAVY_ATT ? left : HEAVY_ATT;
+        h.flags = fl;
+        h.slot = slot;
+        h.pad = 0;
+        I.heavy[q0 + q] = h;
     }
 }
 
-__global__ void __launch_bounds__(K1_THREADS) k_spawn_heavy(const DevInst *__restrict__ insts, int n_inst)
+// parts: warps per bucket, so that a small list still reaches every SM; part
+// p takes slots p, p + parts, ... (the oldest determinants, the most
+// populated ones, come first in a bucket).  Determinants with more than
+// heavy_min attempts go to the heavy queue.  The loop holds every piece of
+// work once (code size): each turn evaluates a full window of attempts or of
+// singles, or else appends parents; a run's last turns empty what is left.
+template <int GEN, bool ADAPT, typename RUNS>
+__device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int parts, unsigned heavy_min)
 {
-    extern __shared__ __align__(16) unsigned char k1_raw[];
-    K1Smem &S = *reinterpret_cast<K1Smem *>(k1_raw);
-    for (int ii = 0; ii < n_inst; ii++) {
-        const DevInst &I = insts[ii];
-        if (threadIdx.x == 0) {
-            S.hdr_err = *(volatile int *)&I.st->err;
-            S.qn[0] = I.st->heavy_n;
-            S.hdr_it = I.st->iter;
-            S.hdr_par = I.st->parity;
-            S.hdr_S = I.st->S;
-        }
-        __syncthreads();
-        const int err = S.hdr_err, nh = S.qn[0], par = S.hdr_par;
-        const long long it = S.hdr_it;
-        const double shift = S.hdr_S;
-        __syncthreads();
-        if (err) continue;
-        for (int q = blockIdx.x; q < nh; q += gridDim.x) {
-            HeavyMap map{I.heavy[q]};
-            run_attempts(I, S, it, map.h.count, map, par, shift);
-        }
+    extern __shared__ __align__(16) unsigned char sp_raw[];
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    SpawnWarp &W = reinterpret_cast<SpawnWarp *>(sp_raw)[threadIdx.x >> 5];
+    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
+    SpawnCursor C{0, 0, 0, 0, 0, 0};
+    SpawnRun R{0, 0.0, 0, nullptr};
+    if (ADAPT) {
+        R.aq = reinterpret_cast<AdaptQueue *>(sp_raw + SP_WARPS * sizeof(SpawnWarp)) + (threadIdx.x >> 5);
+        if (lane == 0) R.aq->n = 0;
+        __syncwarp();
     }
+    unsigned long long att = 0;
+    int cur = -1, err = 0;
+    int v = gw, u = 0, ii = -1, b = 0, t = 0, m = 0;  // unit and part; next tile of bucket b
+    bool have = false, drain = false;                 // v is set up (t, m valid); the run's list is done
+    while (true) {
+        if (ADAPT) {
+            __syncwarp();
+            const unsigned na = R.aq->n;
+            if (na >= 32 || (drain && na > 0 && C.nq == 0 && C.tot == C.done)) {
+                eval_adaptive(runs.inst(cur), R);
+                continue;
+            }
+        }
+        if (C.nq >= 32 || (drain && C.nq > 0)) {
+            eval_singles(runs.inst(cur), W, C.nq, R);
+            continue;
+        }
+        if (C.tot - C.done >= 32u || (drain && C.tot != C.done)) {  // a full window, or a run's last one
+            spawn_window<GEN>(runs.inst(cur), W, C, R);
+            continue;
+        }
+        // the next tile of this warp, in this run or another
+        while (!have || t >= m) {
+            if (have) { v += nw; have = false; }
+            if (v >= n_units * parts) { ii = -1; break; }
+            u = v / parts;
+            ii = runs.find(u);
+            if (ii != cur) break;
+            if (!err) {
+                b = u - runs.inst(ii).unit0;
+                m = runs.inst(ii).cnt[R.par][b];
+                t = v - u * parts;
+            } else {
+                m = t = 0;
+            }
+            have = true;
+        }
+        const bool more = have && t < m;
+        if (cur >= 0 && !err) {
+            const DevInst &I = runs.inst(cur);
+            const bool divide = C.nd >= 32 || (!more && C.nd > 0);
+            if (more || divide) {
+                // parents from the list (a tile) or from the division queue
+                const int n = min(C.nd, 32);
+                unsigned slot;
+                bool in;
+                __syncwarp();
+                if (divide) {
+                    in = lane < n;
+                    slot = W.divq[in ? C.nd - n + lane : 0];
+                    C.nd -= n;
+                } else {
+                    const int d = t + lane * parts;
+                    in = d < m;
+                    slot = (unsigned)((size_t)b * CAP_M + d);
+                    t += 32 * parts;
+                }
+                ulonglong2 kk = make_ulonglong2(0, 0);
+                double c = 0.0;
+                uint8_t f = 0;
+                if (in) {
+                    kk = I.key[R.par][slot];
+                    c = I.c[R.par][slot];
+                    f = I.fl[R.par][slot];
+                }
+                unsigned nat = 0;
+                bool valid = !is_zero(c), later = false;
+                double cper = c;  // C / 1 is C
+                const bool init = (dbits(c) & ~SIGN64) > dbits(I.n_a) || (f & (DFLAG_REF | DFLAG_D));
+                const unsigned fl = (init ? 1u : 0u) | ((f & DFLAG_D) ? 2u : 0u);
+                if (valid && !abs_lt(c, 0x1p31)) {
+                    atomicOr(&I.st->err, ERRB_NUMERIC);
+                    valid = false;
+                }
+                if (valid) nat = (unsigned)ceil_abs(c);
+                if (divide) {
+                    cper = c / (double)max(nat, 1u);
+                } else {
+                    att += nat;
+                    if (nat > heavy_min) {
+                        queue_heavy(I, kk, c, nat, fl, slot);
+                        valid = false;
+                    } else if (nat & (nat - 1)) {
+                        later = true;
+                        valid = false;
+                    } else if (valid) {  // n_att = 2^s <= 2 |C|: the quotient is C with its exponent lowered by s
+                        cper = bitsd(dbits(c) - ((u64)(31 - __clz(nat)) << 52));
+                    }
+                }
+                const unsigned md = __ballot_sync(0xffffffffu, later);
+                if (later) W.divq[C.nd + __popc(md & below)] = slot;
+                C.nd += __popc(md);
+                spawn_append(W, C, valid, kk, nat, cper, fl, slot);
+                continue;
+            }
+            // the run is at its end for this warp: what is still pending
+            if (C.tot != C.done || C.nq > 0 || (ADAPT && R.aq->n > 0)) {
+                drain = true;
+                continue;
+            }
+            for (int o = 16; o >= 1; o >>= 1) att += __shfl_xor_sync(0xffffffffu, att, o);
+            if (lane == 0 && att) red_add(&I.acc[(gw % NSHARD) * ACC_STRIDE + ACC_ATT], (u64)att);
+        }
+        if (ii < 0) return;
+        drain = false;
+        // a new run: its state, read once per run a warp meets (a flag raised
+        // by another warp during this kernel makes the host repeat the
+        // iteration, whose output is then discarded)
+        cur = ii;
+        const DevInst &I = runs.inst(cur);
+        C = SpawnCursor{0, 0, 0, 0, 0, 0};
+        att = 0;
+        err = __shfl_sync(0xffffffffu, *(volatile int *)&I.st->err, 0);
+        R.par = I.st->parity;
+        R.it = I.st->iter;
+        R.S = I.st->S;
+        if (lane == 0 && v == I.unit0 * parts) I.st->err_at_start = err;  // the state seen when this run's spawning began
+    }
+}
+
+template <int GEN, bool ADAPT>
+__global__ void __launch_bounds__(SP_THREADS, ADAPT ? 3 : 4) k_spawn(const __grid_constant__ DevInst I, int n_units,
+                                                                     int parts, unsigned heavy_min)
+{
+    spawn_body<GEN, ADAPT>(OneRun{I}, n_units, parts, heavy_min);
+}
+
+template <bool ADAPT>
+__global__ void __launch_bounds__(SP_THREADS, ADAPT ? 3 : 4) k_spawn_batch(const DevInst *__restrict__ insts,
+                                                                        const int *__restrict__ unit_start, int n_inst,
+                                                                        int n_units, int parts, unsigned heavy_min)
+{
+    spawn_body<GEN_ANY, ADAPT>(RunTable{insts, unit_start, n_inst}, n_units, parts, heavy_min);
+}
+
+// the slices of heavily populated determinants, one block each
+template <typename RUNS>
+__device__ __forceinline__ void heavy_body(const RUNS &runs, int n_inst)
+{
+    extern __shared__ __align__(16) unsigned char sp_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SpawnWarp &W = reinterpret_cast<SpawnWarp *>(sp_raw)[warp];
+    AdaptQueue *aq = reinterpret_cast<AdaptQueue *>(sp_raw + SP_WARPS * sizeof(SpawnWarp)) + warp;
+    if (lane == 0) aq->n = 0;
+    __syncwarp();
+    for (int ii = 0; ii < n_inst; ii++) {
+        const DevInst &I = runs.inst(ii);
+        const int nh = I.st->heavy_n;
+        const int err = __shfl_sync(0xffffffffu, *(volatile int *)&I.st->err, 0);  // one value for the whole warp
+        if ((int)blockIdx.x >= nh || err) continue;
+        const SpawnRun R{I.st->iter, I.st->S, I.st->parity, I.adaptive ? aq : nullptr};
+        int nq = 0;
+        for (int q = blockIdx.x; q < nh; q += gridDim.x) {
+            const HeavyChunk h = I.heavy[q];
+            for (unsigned a = 32u * warp; a < h.count; a += SP_THREADS)
+            {
+                attempts32<GEN_ANY>(I, W, nq, R, a + lane < h.count, make_ulonglong2(h.a, h.b), h.k0 + a + lane, h.cper,
+                                    h.flags, h.slot);
+                if (nq >= 32) eval_singles(I, W, nq, R);
+                while (R.aq && __shfl_sync(0xffffffffu, R.aq->n, 0) >= 32u) eval_adaptive(I, R);
+            }
+        }
+        if (nq > 0) eval_singles(I, W, nq, R);
+        while (R.aq && __shfl_sync(0xffffffffu, R.aq->n, 0) > 0u) eval_adaptive(I, R);
+    }
+}
+
+__global__ void __launch_bounds__(SP_THREADS, 3) k_spawn_heavy(const __grid_constant__ DevInst I)
+{
+    heavy_body(OneRun{I}, 1);
+}
+
+__global__ void __launch_bounds__(SP_THREADS, 3) k_spawn_heavy_batch(const DevInst *__restrict__ insts, int n_inst)
+{
+    heavy_body(RunTable{insts, nullptr, n_inst}, n_inst);
 }
 
 // ------------------------------------------------------------------ annihilation
@@ -1748,607 +1795,6 @@ __global__ void __launch_bounds__(K3_THREADS, 2) k_annihilate_staged(const DevIn
     if (cur >= 0) anni_flush(insts[cur], T);
 }
 
-// ------------------------------------------------------------------ staged spawning
-// The spawning kernel with every bucket's keys, amplitudes and flags brought
-// into shared memory by bulk copies one bucket ahead (the bucket's count one
-// bucket earlier still), as in the staged annihilation; C_i / n_att is
-// written over the staged amplitude.  Chunks of 512 attempts keep three
-// blocks per SM.
-constexpr int CHUNK_S = 512;
-struct K6Smem {
-    static constexpr int chunk = CHUNK_S;
-    ulonglong2 skey[2][CAP_M];
-    double sc[2][CAP_M];            // C as copied; C / n_att once the bucket is loaded
-    unsigned char sfl[2][CAP_M];
-    unsigned off[CAP_M + 1];
-    unsigned short att_det[CHUNK_S];
-    unsigned char fl[CAP_M];        // initiator | in-D bits of the current bucket
-    SpawnRec rec[CHUNK_S];
-    unsigned short divl[CAP_M];     // determinants whose C / n_att (n_att > 1) is still to be divided
-    int ndiv;
-    int qn[NQ];
-    int next;
-    unsigned wsum[K1_THREADS / 32];
-    u64 bar[2];
-    int binfo[2][4];                // per stage: bucket (-1: nothing staged), m, run, parity
-    long long bit[2];
-    double bS[2];
-};
-static_assert(3 * (sizeof(K6Smem) + 1024) <= 233472, "three staged spawning blocks per SM");
-
-struct StagedBucketMap {
-    const K6Smem *S;
-    int q;
-    __device__ unsigned det_of(unsigned a, u64 &k) const
-    {
-        if (a < (unsigned)CHUNK_S) {
-            const unsigned d = S->att_det[a];
-            if (d != 0xffffu) {
-                k = a - S->off[d];
-                return d;
-            }
-        }
-        int lo = 0, hi = CAP_M;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (S->off[mid] <= a) lo = mid; else hi = mid;
-        }
-        k = a - S->off[lo];
-        return (unsigned)lo;
-    }
-    __device__ ulonglong2 key(unsigned d) const { return S->skey[q][d]; }
-    __device__ double cper(unsigned d) const { return S->sc[q][d]; }
-    __device__ unsigned flags(unsigned d) const { return S->fl[d]; }
-    __device__ unsigned slot(unsigned d) const { return base + d; }
-    unsigned base;
-};
-
-struct SpawnMeta {
-    int u, ii, b, m, par, err;
-    long long it;
-    double S;
-};
-
-// thread 0: the run's state (once per run the block meets) and the bucket's count
-__device__ __forceinline__ void spawn_meta_load(const DevInst *__restrict__ insts, const int *__restrict__ unit_start,
-                                                int n_inst, int u, SpawnMeta &M)
-{
-    M.u = u;
-    if (u < 0) return;
-    const int ii = find_inst(unit_start, n_inst, u);
-    const DevInst &I = insts[ii];
-    if (ii != M.ii) {
-        M.ii = ii;
-        M.err = *(volatile int *)&I.st->err;
-        M.par = I.st->parity;
-        M.it = I.st->iter;
-        M.S = I.st->S;
-        I.st->err_at_start = M.err;  // the state seen when this run's spawning began
-    }
-    M.b = u - I.unit0;
-    M.m = I.cnt[M.par][M.b];
-}
-
-// thread 0: the bulk copies of unit M.u's bucket into stage q
-__device__ void spawn_stage_issue(const DevInst *__restrict__ insts, const SpawnMeta &M, K6Smem &S, int q)
-{
-    int *bi = S.binfo[q];
-    bi[0] = -1;
-    if (M.u < 0 || M.err) return;
-    const DevInst &I = insts[M.ii];
-    const int m = M.m, par = M.par;
-    const size_t base = (size_t)M.b * CAP_M;
-    const unsigned m2 = (unsigned)((m + 1) & ~1), m16 = (unsigned)((m + 15) & ~15);
-    const unsigned bytes = m ? (unsigned)m * 16u + m2 * 8u + m16 : 0u;
-    bi[1] = m; bi[2] = M.ii; bi[3] = par;
-    S.bit[q] = M.it;
-    S.bS[q] = M.S;
-    bi[0] = M.b;
-    if (bytes == 0) {
-        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(&S.bar[q]))
-                     : "memory");
-        return;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&S.bar[q], bytes);
-    bulk_g2s(S.skey[q], I.key[par] + base, (unsigned)m * 16u, &S.bar[q]);
-    bulk_g2s(S.sc[q], I.c[par] + base, m2 * 8u, &S.bar[q]);
-    bulk_g2s(S.sfl[q], I.fl[par] + base, m16, &S.bar[q]);
-}
-
-__global__ void __launch_bounds__(K1_THREADS, 3) k_spawn_staged(const DevInst *__restrict__ insts,
-                                                             const int *__restrict__ unit_start, int n_inst,
-                                                             int n_units)
-{
-    extern __shared__ __align__(128) unsigned char k6_raw[];
-    K6Smem &S = *reinterpret_cast<K6Smem *>(k6_raw);
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    constexpr int PER = CAP_M / K1_THREADS;
-    SpawnMeta nxt;
-    nxt.ii = -1;
-    if (t == 0) {
-        S.ndiv = 0;
-        mbar_init(&S.bar[0], 1);
-        mbar_init(&S.bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        SpawnMeta first;
-        first.ii = -1;
-        spawn_meta_load(insts, unit_start, n_inst, (int)blockIdx.x < n_units ? (int)blockIdx.x : -1, first);
-        spawn_stage_issue(insts, first, S, 0);
-        nxt.ii = first.ii;
-        nxt.err = first.err; nxt.par = first.par; nxt.it = first.it; nxt.S = first.S;
-        const int un = (int)blockIdx.x + (int)gridDim.x;
-        spawn_meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-    }
-    __syncthreads();
-    unsigned phase[2] = {0u, 0u};
-    int q = 0;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, q ^= 1) {
-        if (t == 0) {
-            spawn_stage_issue(insts, nxt, S, q ^ 1);
-            const int un = u + 2 * (int)gridDim.x;
-            spawn_meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-        }
-        const int b = S.binfo[q][0];
-        if (b < 0) {
-            __syncthreads();  // binfo[q ^ 1] is written before anyone reads it
-            continue;
-        }
-        const bool ok = mbar_wait(&S.bar[q], phase[q]);
-        const int m = S.binfo[q][1], ii = S.binfo[q][2], par = S.binfo[q][3];
-        const long long it = S.bit[q];
-        const double shift = S.bS[q];
-        const DevInst &I = insts[ii];
-        if (__syncthreads_or(!ok)) {  // the copies did not land within the bound
-            if (t == 0) atomicOr(&I.st->err, ERRB_TIMEOUT);
-            mbar_wait(&S.bar[q], phase[q]);
-            if (S.binfo[q ^ 1][0] >= 0) mbar_wait(&S.bar[q ^ 1], phase[q ^ 1]);
-            return;
-        }
-        phase[q] ^= 1u;
-        const size_t base = (size_t)b * CAP_M;
-        // the bucket from the stage: thread t owns determinants PER*t .. PER*t+PER-1
-        long long att = 0;
-        unsigned mine = 0;
-        unsigned nl[PER];
-        for (int j = 0; j < PER; j++) {
-            const int d = PER * t + j;
-            nl[j] = 0;
-            bool dv = false;
-            if (d < m) {
-                const double c = S.sc[q][d];
-                const uint8_t f = S.sfl[q][d];
-                unsigned fl = 0;
-                double cper = 0.0;
-                u64 nat = 0;
-                if (!is_zero(c)) {
-                    if (!abs_lt(c, 0x1p31)) {
-                        atomicOr(&I.st->err, ERRB_NUMERIC);
-                    } else {
-                        nat = ceil_abs(c);
-                        const bool init = (dbits(c) & ~SIGN64) > dbits(I.n_a) || (f & (DFLAG_REF | DFLAG_D));
-                        fl = (init ? 1u : 0u) | ((f & DFLAG_D) ? 2u : 0u);
-                        cper = c;  // C / n_att: below for n_att > 1 (c / 1 is c)
-                        att += (long long)nat;
-                        if (nat > HEAVY_ATT) {  // sliced into the heavy queue
-                            cper = c / (double)nat;
-                            const ulonglong2 kk = S.skey[q][d];
-                            const unsigned nch = (unsigned)((nat + HEAVY_ATT - 1) / HEAVY_ATT);
-                            const int q0 = atomicAdd(&I.st->heavy_n, (int)nch);
-                            if ((long long)q0 + nch > (long long)I.heavy_cap) atomicOr(&I.st->err, ERRB_HEAVY_CAP);
-                            else
-                                for (unsigned h = 0; h < nch; h++) {
-                                    HeavyChunk hc;
-                                    hc.a = kk.x; hc.b = kk.y; hc.cper = cper; hc.k0 = (u64)h * HEAVY_ATT;
-                                    const u64 left = nat - hc.k0;
-                                    hc.count = (unsigned)(left < HEAVY_ATT ? left : HEAVY_ATT);
-                                    hc.flags = fl;
-                                    hc.slot = (uint32_t)(base + d);
-                                    hc.pad = 0;
-                                    I.heavy[q0 + h] = hc;
-                                }
-                        } else {
-                            nl[j] = (unsigned)nat;
-                            dv = nat > 1;
-                        }
-                    }
-                }
-                S.sc[q][d] = cper;
-                S.fl[d] = (unsigned char)fl;
-                mine += nl[j];
-            }
-            queue_div(S, dv, d, lane);
-        }
-        for (int a = t; a < CHUNK_S; a += K1_THREADS) S.att_det[a] = 0xffffu;
-        // exclusive scan of the light attempt counts in determinant order
-        unsigned v = mine;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        if (lane == 31) S.wsum[warp] = v;
-        __syncthreads();
-        if (warp == 0) {
-            unsigned x = lane < K1_THREADS / 32 ? S.wsum[lane] : 0u;
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (lane < K1_THREADS / 32) S.wsum[lane] = x;
-        } else {
-            divide_listed(S.divl, S.ndiv, S.sc[q], t - 32, K1_THREADS - 32);  // warp 0 scans meanwhile
-        }
-        __syncthreads();
-        if (t == 0) S.ndiv = 0;  // read by every thread before the barrier above
-        unsigned ex = v - mine + (warp ? S.wsum[warp - 1] : 0u);
-        for (int j = 0; j < PER; j++) {
-            S.off[PER * t + j] = ex;
-            if (nl[j] <= 8u && ex + nl[j] <= (unsigned)CHUNK_S)
-                for (unsigned a = 0; a < nl[j]; a++) S.att_det[ex + a] = (unsigned short)(PER * t + j);
-            ex += nl[j];
-        }
-        if (t == K1_THREADS - 1) S.off[CAP_M] = ex;
-        __syncthreads();
-        const unsigned total = S.off[CAP_M];
-        StagedBucketMap map{&S, q, (unsigned)base};
-        run_attempts(I, S, it, total, map, par, shift);
-        for (int o = 16; o >= 1; o >>= 1) att += __shfl_xor_sync(0xffffffffu, att, o);
-        if (lane == 0 && att) red_add(&I.acc[(b % NSHARD) * ACC_STRIDE + ACC_ATT], (u64)att);
-    }
-}
-
-// ------------------------------------------------------------------ split spawning: the draw
-// The first half of split spawning: the staged bucket (bulk copies one bucket
-// ahead, as above), n_att and C_i / n_att per determinant, then the attempts
-// drawn, classified and written to the run's attempt queues for
-// k_spawn_eval.  The block that draws bucket b of a run owns segment
-// b mod (grid size) of both of the run's queues (every bucket of the run it
-// meets has the same residue), so its fill is a count every thread of the
-// block keeps alike and no global atomic is needed; a run needs
-// min(grid size, buckets) segments.  With double-buffered stage, flags and
-// class counters a bucket
-// takes three block barriers (one more per extra chunk of attempts):
-//   A  the bucket is in shared memory, n_att counted per warp
-//   B  the block scan of the attempt offsets and the divisions are done
-//   C  the chunk's attempts are drawn and queued in shared memory
-// after which the chunk's records go out while the next bucket starts.
-struct K7Smem {
-    static constexpr int chunk = CHUNK_S;
-    ulonglong2 skey[2][CAP_M];
-    double sc[2][CAP_M];            // C as copied; C / n_att once the bucket is loaded
-    unsigned char sfl[2][CAP_M];
-    unsigned char fl[2][CAP_M];     // initiator | in-D bits, per stage
-    unsigned off[CAP_M];
-    unsigned short att_det[CHUNK_S];
-    unsigned short divl[CAP_M];
-    SpawnRec rec[CHUNK_S];
-    int ndiv;
-    int qn[2][NQ];                  // class counts, by chunk parity
-    unsigned wsum[K1_THREADS / 32];
-    u64 bar[2];
-    int binfo[2][4];
-    long long bit[2];
-    double bS[2];
-};
-static_assert(3 * (sizeof(K7Smem) + 1024) <= 233472, "three draw blocks per SM");
-
-// Thread t of the draw block owns slots t, t + 256, t + 512, t + 768 of the
-// bucket (consecutive threads on consecutive slots: the per-determinant work
-// is spread over the block and the shared-memory accesses are conflict-free);
-// attempt offsets run over the owner-major order v = 4 t + j, j the slot's
-// round, so off[] is indexed by v and slot(v) = (v >> 2) + (v & 3) 256.
-__device__ __forceinline__ unsigned draw_slot(unsigned v) { return (v >> 2) + (v & 3u) * K1_THREADS; }
-__device__ __forceinline__ unsigned draw_order(unsigned d) { return (d % K1_THREADS) * 4u + d / K1_THREADS; }
-static_assert(CAP_M == 4 * K1_THREADS, "four slots per draw thread");
-
-struct DrawBucketMap {
-    const K7Smem *S;
-    int q;
-    unsigned base;
-    __device__ unsigned det_of(unsigned a, u64 &k) const
-    {
-        if (a < (unsigned)CHUNK_S) {
-            const unsigned d = S->att_det[a];
-            if (d != 0xffffu) {
-                k = a - S->off[draw_order(d)];
-                return d;
-            }
-        }
-        int lo = 0, hi = CAP_M;  // largest v with off[v] <= a (slots past the count hold the total)
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (S->off[mid] <= a) lo = mid; else hi = mid;
-        }
-        k = a - S->off[lo];
-        return draw_slot((unsigned)lo);
-    }
-    __device__ ulonglong2 key(unsigned d) const { return S->skey[q][d]; }
-    __device__ double cper(unsigned d) const { return S->sc[q][d]; }
-    __device__ unsigned flags(unsigned d) const { return S->fl[q][d]; }
-    __device__ unsigned slot(unsigned d) const { return base + d; }
-};
-
-// thread 0: the bulk copies of unit M.u's bucket into stage q of the draw kernel
-__device__ void draw_stage_issue(const DevInst *__restrict__ insts, const SpawnMeta &M, K7Smem &S, int q)
-{
-    int *bi = S.binfo[q];
-    bi[0] = -1;
-    if (M.u < 0 || M.err) return;
-    const DevInst &I = insts[M.ii];
-    const int m = M.m, par = M.par;
-    const size_t base = (size_t)M.b * CAP_M;
-    const unsigned m2 = (unsigned)((m + 1) & ~1), m16 = (unsigned)((m + 15) & ~15);
-    const unsigned bytes = m ? (unsigned)m * 16u + m2 * 8u + m16 : 0u;
-    bi[1] = m; bi[2] = M.ii; bi[3] = par;
-    S.bit[q] = M.it;
-    S.bS[q] = M.S;
-    bi[0] = M.b;
-    if (bytes == 0) {
-        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(&S.bar[q]))
-                     : "memory");
-        return;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(&S.bar[q], bytes);
-    bulk_g2s(S.skey[q], I.key[par] + base, (unsigned)m * 16u, &S.bar[q]);
-    bulk_g2s(S.sc[q], I.c[par] + base, m2 * 8u, &S.bar[q]);
-    bulk_g2s(S.sfl[q], I.fl[par] + base, m16, &S.bar[q]);
-}
-
-// thread 0: the queue fill of this block's segment of a run
-__device__ __forceinline__ void draw_flush(const DevInst &I, int seg, long long q0, long long q1)
-{
-    I.qcnt[seg] = (int)min(q0, 0x7fffffffLL);
-    I.qcnt[I.qnseg + seg] = (int)min(q1, 0x7fffffffLL);
-}
-
-__global__ void __launch_bounds__(K1_THREADS, 3) k_spawn_draw(const DevInst *__restrict__ insts,
-                                                              const int *__restrict__ unit_start, int n_inst,
-                                                              int n_units)
-{
-    extern __shared__ __align__(128) unsigned char k7_raw[];
-    K7Smem &S = *reinterpret_cast<K7Smem *>(k7_raw);
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    constexpr int PER = CAP_M / K1_THREADS;
-    // the last thread (its determinants are the last slots of a bucket, mostly
-    // empty) issues the copies and keeps the meta data of the next bucket
-    constexpr int ISSUER = K1_THREADS - 1;
-    SpawnMeta nxt;
-    nxt.ii = -1;
-    if (t == ISSUER) {
-        S.ndiv = 0;
-        for (int k = 0; k < 2 * NQ; k++) S.qn[k / NQ][k % NQ] = 0;
-        mbar_init(&S.bar[0], 1);
-        mbar_init(&S.bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        SpawnMeta first;
-        first.ii = -1;
-        spawn_meta_load(insts, unit_start, n_inst, (int)blockIdx.x < n_units ? (int)blockIdx.x : -1, first);
-        draw_stage_issue(insts, first, S, 0);
-        nxt.ii = first.ii;
-        nxt.err = first.err; nxt.par = first.par; nxt.it = first.it; nxt.S = first.S;
-        const int un = (int)blockIdx.x + (int)gridDim.x;
-        spawn_meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-    }
-    __syncthreads();
-    unsigned phase[2] = {0u, 0u};
-    int q = 0, cp = 0;             // stage, chunk parity
-    int cur = -1, seg = 0;         // the run whose segment (seg) fill is held in qf0, qf1
-    long long qf0 = 0, qf1 = 0;    // entries this block queued for run `cur` (singles, doubles)
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, q ^= 1) {
-        const int b = S.binfo[q][0];
-        bool ok = true;
-        int m = 0, ii = 0;
-        if (b >= 0) {
-            ok = mbar_wait(&S.bar[q], phase[q]);
-            m = S.binfo[q][1];
-            ii = S.binfo[q][2];
-        }
-        const DevInst &I = insts[ii];
-        // A: the bucket from the stage; thread t owns slots t + 256 j (draw_slot)
-        long long att = 0;
-        unsigned mine = 0;
-        unsigned nl[PER];
-        for (int j = 0; j < PER; j++) {
-            const int d = t + j * K1_THREADS;
-            nl[j] = 0;
-            bool dv = false;
-            if (d < m && ok) {
-                const double c = S.sc[q][d];
-                const uint8_t f = S.sfl[q][d];
-                unsigned fl = 0;
-                double cper = 0.0;
-                u64 nat = 0;
-                if (!is_zero(c)) {
-                    if (!abs_lt(c, 0x1p31)) {
-                        atomicOr(&I.st->err, ERRB_NUMERIC);
-                    } else {
-                        nat = ceil_abs(c);
-                        const bool init = (dbits(c) & ~SIGN64) > dbits(I.n_a) || (f & (DFLAG_REF | DFLAG_D));
-                        fl = (init ? 1u : 0u) | ((f & DFLAG_D) ? 2u : 0u);
-                        cper = c;  // C / n_att: after A for n_att > 1 (c / 1 is c)
-                        att += (long long)nat;
-                        if (nat > HEAVY_ATT) {  // sliced into the heavy queue
-                            cper = c / (double)nat;
-                            const ulonglong2 kk = S.skey[q][d];
-                            const unsigned nch = (unsigned)((nat + HEAVY_ATT - 1) / HEAVY_ATT);
-                            const int q0 = atomicAdd(&I.st->heavy_n, (int)nch);
-                            if ((long long)q0 + nch > (long long)I.heavy_cap) atomicOr(&I.st->err, ERRB_HEAVY_CAP);
-                            else
-                                for (unsigned h = 0; h < nch; h++) {
-                                    HeavyChunk hc;
-                                    hc.a = kk.x; hc.b = kk.y; hc.cper = cper; hc.k0 = (u64)h * HEAVY_ATT;
-                                    const u64 left = nat - hc.k0;
-                                    hc.count = (unsigned)(left < HEAVY_ATT ? left : HEAVY_ATT);
-                                    hc.flags = fl;
-                                    hc.slot = (uint32_t)((size_t)b * CAP_M + d);
-                                    hc.pad = 0;
-                                    I.heavy[q0 + h] = hc;
-                                }
-                        } else {
-                            nl[j] = (unsigned)nat;
-                            dv = nat > 1;
-                        }
-                    }
-                }
-                S.sc[q][d] = cper;
-                S.fl[q][d] = (unsigned char)fl;
-                mine += nl[j];
-            }
-            queue_div(S, dv, d, lane);
-        }
-        for (int a = t; a < CHUNK_S; a += K1_THREADS) S.att_det[a] = 0xffffu;
-        unsigned v = mine;  // inclusive warp scan of the light attempt counts in owner-major order
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        if (lane == 31) S.wsum[warp] = v;
-        if (__syncthreads_or(!ok)) {  // A; the copies did not land within the bound
-            if (t == 0) atomicOr(&I.st->err, ERRB_TIMEOUT);
-            mbar_wait(&S.bar[q], phase[q]);
-            return;
-        }
-        if (t == ISSUER) {  // every thread is past the last reads of stage q ^ 1 (bucket u - grid)
-            draw_stage_issue(insts, nxt, S, q ^ 1);
-            const int un = u + 2 * (int)gridDim.x;
-            spawn_meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-        }
-        if (b < 0) {
-            __syncthreads();  // stage q ^ 1's info is written before anyone reads it
-            continue;
-        }
-        phase[q] ^= 1u;
-        if (ii != cur) {  // a new run: the previous run's segment fill is final
-            if (t == 0 && cur >= 0) draw_flush(insts[cur], seg, qf0, qf1);
-            cur = ii;
-            seg = b % (int)gridDim.x;
-            qf0 = qf1 = 0;
-        }
-        const long long it = S.bit[q];
-        // B: attempt offsets (each warp sums the warp totals before its own), parents of the first
-        // CHUNK_S attempts, and C / n_att of the listed determinants
-        unsigned ex = v - mine, total = 0;
-        for (int w = 0; w < K1_THREADS / 32; w++) {
-            const unsigned x = S.wsum[w];
-            ex += w < warp ? x : 0u;
-            total += x;
-        }
-        for (int j = 0; j < PER; j++) {
-            S.off[PER * t + j] = ex;
-            if (nl[j] <= 8u && ex + nl[j] <= (unsigned)CHUNK_S)
-                for (unsigned a = 0; a < nl[j]; a++) S.att_det[ex + a] = (unsigned short)(t + j * K1_THREADS);
-            ex += nl[j];
-        }
-        divide_listed(S.divl, S.ndiv, S.sc[q], t, K1_THREADS);
-        __syncthreads();  // B
-        if (t == 0) S.ndiv = 0;
-        const DrawBucketMap map{&S, q, (unsigned)((size_t)b * CAP_M)};
-        for (unsigned a0 = 0; a0 < total; a0 += CHUNK_S) {
-            if (a0) __syncthreads();  // the previous chunk's records are out before rec[] is reused
-            draw_classify(I, S, it, a0, min(total, a0 + CHUNK_S), map, S.qn[cp]);
-            __syncthreads();  // C
-            const int nd = S.qn[cp][Q_DOUBLE], ns = S.qn[cp][Q_SINGLE], ntot = ns + nd;
-            if (t < NQ) S.qn[cp ^ 1][t] = 0;  // every thread read the other counts before C
-            cp ^= 1;
-            const long long b0 = qf0, b1 = qf1;
-            qf0 += ns;
-            qf1 += nd;
-            bool over = false;
-            for (int r = t; r < ntot; r += K1_THREADS) {
-                const bool single = r < ns;
-                const SpawnRec rr = single ? S.rec[CHUNK_S - 1 - r] : S.rec[r - ns];
-                const int c = single ? 0 : 1;
-                const long long idx = single ? b0 + r : b1 + (r - ns);
-                if (idx >= I.qcap[c]) { over = true; continue; }
-                const unsigned d = rr.det;
-                const ulonglong2 kk = map.key(d);
-                QRec o;
-                o.ka = kk.x; o.kb = kk.y; o.cper = map.cper(d); o.w2 = rr.w2; o.w3 = rr.w3;
-                o.slot = map.slot(d);
-                o.info = (rr.ep & 0xffffu) | (map.flags(d) << 16);
-                I.qrec[c][(size_t)seg * I.qcap[c] + idx] = o;
-            }
-            if (over) atomicOr(&I.st->err, ERRB_QUEUE_CAP);
-            if (t == 0) {
-                if (qf0 > I.qcap[0]) atomicMax(&I.st->need_queue[0], (int)min(qf0, 0x7fffffffLL));
-                if (qf1 > I.qcap[1]) atomicMax(&I.st->need_queue[1], (int)min(qf1, 0x7fffffffLL));
-            }
-        }
-        for (int o = 16; o >= 1; o >>= 1) att += __shfl_xor_sync(0xffffffffu, att, o);
-        if (lane == 0 && att) red_add(&I.acc[(b % NSHARD) * ACC_STRIDE + ACC_ATT], (u64)att);
-    }
-    if (t == 0 && cur >= 0) draw_flush(insts[cur], seg, qf0, qf1);
-}
-
-// The evaluation of the queued attempts of every run: one attempt per
-// thread, doubles first, then singles and hops, with no block barrier; the
-// parent's key, C_i / n_att, flags and slot travel in the record.
-__global__ void __launch_bounds__(256) k_spawn_eval(const DevInst *__restrict__ insts, int n_inst)
-{
-    __shared__ long long s_off[2][NSEG_MAX + 1];
-    __shared__ int s_err, s_par;
-    __shared__ double s_S;
-    const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x, gs = (long long)gridDim.x * blockDim.x;
-    for (int ii = 0; ii < n_inst; ii++) {
-        const DevInst &I = insts[ii];
-        const int ns = I.qnseg;
-        if (threadIdx.x < 32) {  // warp 0: the segment offsets of both classes by a warp scan
-            const int lane = threadIdx.x;
-            if (lane == 0) {
-                s_err = I.st->err_at_start;  // the state this run's spawning began with
-                s_par = I.st->parity;
-                s_S = I.st->S;
-            }
-            const int per = (ns + 31) / 32;  // segments lane*per .. lane*per+per-1
-            for (int c = 0; c < 2; c++) {
-                long long mine = 0;
-                for (int r = 0; r < per; r++) {
-                    const int g = lane * per + r;
-                    if (g < ns) mine += min((long long)I.qcnt[c * ns + g], I.qcap[c]);
-                }
-                long long inc = mine;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const long long y = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += y;
-                }
-                long long ex = inc - mine;
-                for (int r = 0; r < per; r++) {
-                    const int g = lane * per + r;
-                    if (g < ns) {
-                        s_off[c][g] = ex;
-                        ex += min((long long)I.qcnt[c * ns + g], I.qcap[c]);
-                    }
-                }
-                if (lane == 31) s_off[c][ns] = inc;
-            }
-        }
-        __syncthreads();
-        const int err = s_err, par = s_par;
-        const double shift = s_S;
-        const long long nd = s_off[1][ns], ntot = nd + s_off[0][ns];
-        if (!err)
-            for (long long i = gt; i < ntot; i += gs) {
-                const int c = i < nd ? 1 : 0;
-                const long long j = c ? i : i - nd;
-                int lo = 0, hi = ns;  // the segment holding entry j: the last g with s_off[c][g] <= j
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if (s_off[c][mid] <= j) lo = mid; else hi = mid;
-                }
-                const QRec r = I.qrec[c][(size_t)lo * I.qcap[c] + (j - s_off[c][lo])];
-                const SpawnCtx cx{r.slot, par, shift};
-                const unsigned flags = r.info >> 16, sel = r.info & 0xffffu;
-                if (c == 1) {
-                    if (I.pchb) spawn_double_pchb(I, r.ka, r.kb, r.cper, flags, sel, r.w2, r.w3, cx);
-                    else spawn_double(I, r.ka, r.kb, r.cper, flags, sel, r.w2, r.w3, cx);
-                } else if (I.kind == FCIQMC_HUBBARD) spawn_hop_e(I, r.ka, r.kb, r.cper, flags, (int)sel, r.w2, r.w3, cx);
-                else spawn_single_e(I, r.ka, r.kb, r.cper, flags, (int)sel, r.w2, r.w3, cx);
-            }
-        __syncthreads();
-    }
-}
-
 // GENERAL: the batch holds a run with replica side lists or adaptive shift,
 // whose buckets take the general path (anni_bucket); the others the
 // three-phase one.  Without it the kernel holds the three-phase path alone.
@@ -2552,8 +1998,6 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
     u64 w[NACC];
 #pragma unroll
     for (int k = 0; k < NACC; k++) w[k] = __shfl_sync(0xffffffffu, v, k);
-    if (I.qcnt)  // the attempt queues of split spawning start empty
-        for (int g = lane; g < 2 * I.qnseg; g += 32) I.qcnt[g] = 0;
     if (lane != 0) return;
     const u128 W = (u128)limb_total(w + ACC_NW);
     const i128 A = limb_total(w + ACC_ANN), EN = limb_total(w + ACC_ENUM);
@@ -2757,13 +2201,12 @@ void launch_build_kidx(const DevInst *dinst, int parity, int nb, cudaStream_t s)
 }
 
 // launch geometry, chosen by fciqmc_autotune (grid blocks per SM; beyond the
-// resident count, here 3 per SM for the spawning and annihilation kernels, the
-// hardware hands the next block to whichever slot frees first, which evens out
-// buckets of unequal size)
-// g_spawn_bps = 0 and g_anni_bps = 0 select the staged kernels (one resident
-// wave, bulk copies one bucket ahead) wherever the batch fits them, and
-// g_spawn_bps = 1 the staged draw with the flat evaluation (split spawning);
-// otherwise the plain-load kernels with that many blocks per SM
+// resident count, here 4 per SM for the spawning kernel and 3 for the plain
+// annihilation kernel, the hardware hands the next block to whichever slot
+// frees first, which evens out buckets of unequal size)
+// g_spawn_bps = 0 and 1 select one resident wave of spawning blocks;
+// g_anni_bps = 0 selects the staged annihilation kernel (one resident wave,
+// bulk copies one bucket ahead) wherever the batch fits it
 static int g_spawn_bps = 1, g_heavy_bps = 2, g_anni_bps = 0;
 static int g_geometry_gen = 0;  // changes with every set_launch_geometry
 int launch_geometry_generation() { return g_geometry_gen; }
@@ -2781,46 +2224,38 @@ void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps)
     *anni_bps = g_anni_bps;
 }
 
-// the staged spawning kernel (g_spawn_bps = 0: one resident wave of three
-// blocks per SM) where every run's list arrays are 16-byte aligned; else the
-// plain-load kernel with g_spawn_bps blocks per SM
-void launch_spawn(const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool staged, bool split,
+// spawning of one run (`one`, the host image of its descriptor) or of a table
+// of runs (one = NULL).  A bucket's slots are dealt to as many warps as it
+// takes to reach every resident warp of the GPU.  adaptive: some run uses the
+// adaptive shift.
+template <int GEN>
+static void launch_spawn_one(const DevInst *one, int grid, int n_units, int parts, unsigned heavy_min, cudaStream_t s)
+{
+    if (one->adaptive) k_spawn<GEN, true><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(*one, n_units, parts, heavy_min);
+    else k_spawn<GEN, false><<<grid, SP_THREADS, SP_SMEM, s>>>(*one, n_units, parts, heavy_min);
+}
+void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s)
 {
-    if (staged && (g_spawn_bps == 0 || g_spawn_bps == 1)) {
-        int grid = n_units < num_sms() * 3 ? n_units : num_sms() * 3;
-        if (grid < 1) grid = 1;
-        if (split && g_spawn_bps == 1)  // grid <= draw_segments(): at most one queue segment per block and run
-            k_spawn_draw<<<grid, K1_THREADS, sizeof(K7Smem), s>>>(dinst, unit_start, n_inst, n_units);
-        else k_spawn_staged<<<grid, K1_THREADS, sizeof(K6Smem), s>>>(dinst, unit_start, n_inst, n_units);
-        return;
-    }
-    const int bps = g_spawn_bps > 0 ? g_spawn_bps : 8;
-    int grid = n_units < num_sms() * bps ? n_units : num_sms() * bps;
-    if (grid < 1) grid = 1;
-    k_spawn<<<grid, K1_THREADS, sizeof(K1Smem), s>>>(dinst, unit_start, n_inst, n_units);
+    const int bps = g_spawn_bps > 1 ? g_spawn_bps : (adaptive ? 3 : 4);
+    const int warps = num_sms() * 4 * SP_WARPS;
+    int parts = 1;
+    while (parts < CAP_M / 32 && (long long)n_units * parts < 2 * warps) parts *= 2;
+    const unsigned heavy_min = parts > 1 ? 64 : HEAVY_ATT;
+    const long long need = ((long long)n_units * parts + SP_WARPS - 1) / SP_WARPS;
+    const int grid = (int)(need < (long long)num_sms() * bps ? need : (long long)num_sms() * bps);
+    if (one && one->kind == FCIQMC_HUBBARD) launch_spawn_one<GEN_HOP>(one, grid, n_units, parts, heavy_min, s);
+    else if (one && one->pchb) launch_spawn_one<GEN_PCHB>(one, grid, n_units, parts, heavy_min, s);
+    else if (one) launch_spawn_one<GEN_UNIFORM>(one, grid, n_units, parts, heavy_min, s);
+    else if (adaptive) k_spawn_batch<true><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
+    else k_spawn_batch<false><<<grid, SP_THREADS, SP_SMEM, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
 }
 
-// split spawning (queues in global memory, flat evaluation): geometry 1
-bool spawn_split_selected() { return g_spawn_bps == 1 && draw_segments() <= NSEG_MAX; }
-int draw_segments() { return num_sms() * 3; }
-
-void launch_spawn_eval(const DevInst *dinst, int n_inst, cudaStream_t s)
+void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cudaStream_t s)
 {
-    k_spawn_eval<<<num_sms() * 4, 256, 0, s>>>(dinst, n_inst);  // one resident wave (64 registers)
-}
-
-bool staged_spawn_fits(const DevInst &I)
-{
-    auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
-    for (int k = 0; k < 2; k++)
-        if (!al(I.key[k]) || !al(I.c[k]) || !al(I.fl[k])) return false;
-    return true;
-}
-
-void launch_spawn_heavy(const DevInst *dinst, int n_inst, cudaStream_t s)
-{
-    k_spawn_heavy<<<num_sms() * g_heavy_bps, K1_THREADS, sizeof(K1Smem), s>>>(dinst, n_inst);
+    const int grid = num_sms() * g_heavy_bps;
+    if (one) k_spawn_heavy<<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(*one);
+    else k_spawn_heavy_batch<<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(dinst, n_inst);
 }
 
 cudaError_t init_kernels()
@@ -2832,13 +2267,22 @@ cudaError_t init_kernels()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_annihilate_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(K4Smem<STAGED_SCAP>));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_spawn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K1Smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_spawn_staged, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K6Smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_spawn_draw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K7Smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_spawn_heavy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K1Smem));
+    auto spawn_smem = [&](auto *f, size_t bytes, int blocks) {  // the resident blocks need their shared memory at once
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)((blocks * (bytes + 1024) * 100 + 233471) / 233472));
+    };
+    spawn_smem(k_spawn<GEN_UNIFORM, false>, SP_SMEM, 4);
+    spawn_smem(k_spawn<GEN_PCHB, false>, SP_SMEM, 4);
+    spawn_smem(k_spawn<GEN_HOP, false>, SP_SMEM, 4);
+    spawn_smem(k_spawn_batch<false>, SP_SMEM, 4);
+    spawn_smem(k_spawn<GEN_UNIFORM, true>, SP_SMEM_ADAPT, 3);
+    spawn_smem(k_spawn<GEN_PCHB, true>, SP_SMEM_ADAPT, 3);
+    spawn_smem(k_spawn<GEN_HOP, true>, SP_SMEM_ADAPT, 3);
+    spawn_smem(k_spawn_batch<true>, SP_SMEM_ADAPT, 3);
+    spawn_smem(k_spawn_heavy, SP_SMEM_ADAPT, 3);
+    spawn_smem(k_spawn_heavy_batch, SP_SMEM_ADAPT, 3);
     return e;
 }
 

@@ -1,0 +1,81 @@
+"""Imported lists at the edges of the spawning and annihilation kernels.
+
+One list per system with amplitudes around every boundary of the spawning
+kernel: windows of 32 attempts, powers of two (C / n_att by the exponent) and
+other counts (by division), slices of 512 attempts and the smaller slices of
+short lists, zero and fractional amplitudes; orbitals 0 and 63 in use; one
+bucket (many warps per bucket, crowded buckets) and many buckets (one warp per
+bucket).  Everything is an exact sum or a keyed draw, so the GPU's list and
+statistics must equal the oracle's bit for bit.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from tests.test_gpu_parity import _fq, assert_states_equal, assert_stats_equal
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [0.25, 0.75, 1.0, 1.5, 2.0, 2.5, 3.0, 4.0, 5.5, 7.0, 8.0, 15.5, 16.0, 31.0, 32.0, 32.5, 33.0, 63.5, 64.0, 64.5, 65.0,
+         127.0, 128.0, 511.5, 512.0, 512.5, 513.0, 1024.0, 1500.25, 3000.0]
+
+
+def _words(rng, norb, n_el, n):
+    out = []
+    for _ in range(n):
+        w = 0
+        for p in rng.choice(norb, n_el, replace=False):
+            w |= 1 << int(p)
+        out.append(w)
+    return np.array(out, np.uint64)
+
+
+def _list(sysd, norb, n, seed):
+    """n distinct determinants (a third with orbitals 0 and norb - 1 occupied), amplitudes through EDGES, the
+    reference among them."""
+    rng = np.random.default_rng(seed)
+    s = oracle.system_from_workload(sysd)
+    ra, rb = s.ref
+    a, b = _words(rng, norb, sysd["n_alpha"], n), _words(rng, norb, sysd["n_beta"], n)
+    a[0], b[0] = ra, rb
+    key = sorted({(int(x), int(y)) for x, y in zip(a, b)}, key=lambda k: (k != (ra, rb), rng.random()))
+    a = np.array([k[0] for k in key], np.uint64)
+    b = np.array([k[1] for k in key], np.uint64)
+    c = np.ones(a.size)
+    c[1::2] = rng.choice([0.5, 1.0, 1.25, 2.0, 3.0], c[1::2].size)
+    k = min(len(EDGES), a.size)
+    c[:k] = np.array(EDGES[::-1])[:k]
+    return s, a, b, c * rng.choice([-1.0, 1.0], c.size)
+
+
+def _abinitio(norb, na, nb, seed):
+    h, eri = workloads.synthetic_abinitio(norb, 8, seed)
+    return dict(kind="abinitio", norb=norb, n_alpha=na, n_beta=nb, h1=h, eri=eri, ecore=0.0)
+
+
+CASES = {
+    "orb64": (lambda: _abinitio(64, 3, 2, 3), 64, dict(tau=2e-4, p_single=0.3, initiator_threshold=3.0)),
+    "orb33_one_beta": (lambda: _abinitio(33, 4, 1, 4), 33, dict(tau=2e-4, c_min=0.3, initiator_threshold=1.0)),
+    "orb20_heatbath": (lambda: _abinitio(20, 4, 3, 5), 20, dict(tau=5e-4, generator=1, initiator_threshold=3.0)),
+    "orb20_adaptive": (lambda: _abinitio(20, 4, 3, 6), 20, dict(tau=5e-4, adaptive_shift=1, initiator_threshold=3.0)),
+    "hubbard_8x8": (lambda: dict(workloads.hubbard_2d(8, 8, 4.0)), 64, dict(tau=2e-3)),
+}
+
+
+@pytest.mark.parametrize("max_dets", [16, 20000, 8000000])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_imported_list_at_the_edges_bit_exact(name, max_dets):
+    fq = _fq()
+    make, norb, prm = CASES[name]
+    sysd = make()
+    prm = dict(dict(target_walkers=1e9, seed=77, shift_damping=0.5, shift_interval=5), **prm)
+    s, a, b, c = _list(sysd, norb, 700, 11)
+    g = fq.fciqmc_create(sysd, dict(prm, max_dets=max_dets))
+    o = oracle.Run(s, **prm)
+    fq.fciqmc_import_state(g, a, b, c, 0, 0.1)
+    o.import_state(a, b, c, 0, 0.1)
+    fq.fciqmc_step(g, 3)
+    o.step(3)
+    assert_states_equal(fq.fciqmc_export_state(g), o.export())
+    assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats(), first=0)
