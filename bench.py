@@ -208,7 +208,7 @@ def run_reference(args, rank, world):
 
 
 KERNEL_NAMES = {"k_spawn": "k_spawn",
-                "k_annihilate": "k_annihilate_staged + k_annihilate_big"}
+                "k_annihilate": "k_annihilate + k_annihilate_big (H_jj of new determinants included)"}
 
 WORKLOAD_NAMES = {
     "abinitio50": "abinitio-50orb-10a10b (synthetic: 200 Cholesky vectors, seed 4), D = 1e4, ~1e8 walkers",

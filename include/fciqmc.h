@@ -296,12 +296,12 @@ int fciqmc_export_shift(fciqmc_handle *h, int64_t *iteration, double *S, int32_t
 /* Replaces the walker list and the shift state (a restart from a checkpoint).
  * Keys must be distinct, with the right electron counts; the reference
  * determinant is kept (added with C = 0 when absent).  The bucket count grows
- * (one allocation) until every bucket holds at most half its capacity.  The
+ * (one allocation) until every bucket holds at most five sixths of its capacity.  The
  * entries are checked, counted and placed on the device in transient scratch
  * (about 24 bytes per determinant, from the run's allocator); when
  * max_device_bytes leaves no room for it, on the host.
  * FCIQMC_ERR_INVALID_ARG for a wrong electron count, an orbital beyond norb,
- * a non-finite amplitude, or keys that crowd one bucket even at 2^22 buckets
+ * a non-finite amplitude, or keys that crowd one bucket even at 2^24 buckets
  * (duplicates); duplicates that do not are not detected. */
 int fciqmc_import_state(fciqmc_handle *h, int64_t n, const uint64_t *alpha, const uint64_t *beta,
                         const double *c, int64_t iteration, double S, int32_t vary, int64_t shift_start,
@@ -434,9 +434,8 @@ void fciqmc_server_destroy(fciqmc_server *srv);
  * annihilation).  Candidates: for the spawning kernel 0 or 1 = one resident
  * wave of blocks (four 256-thread blocks per SM), 2, 4, 8, 16 = that many
  * blocks per SM; the heavy-spawning kernel's grid (1, 2, 4 blocks per SM);
- * for the annihilation 0 = the staged kernel (two 256-thread blocks per SM,
- * bulk copies one bucket ahead) or 3, 9, 24 = the plain-load kernel (three
- * resident per SM) with that grid.
+ * for the annihilation 0 = one resident wave of blocks (three 256-thread
+ * blocks per SM) or 3, 9, 24 = that many blocks per SM.
  * Defaults: 1, 2, 0.  Results of the runs do not depend on the
  * configuration. */
 int fciqmc_autotune(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t out[3]);
@@ -453,8 +452,9 @@ int fciqmc_get_launch_config(int32_t out[3]);
 /* Device timing of the kernels of the last fciqmc_step call (milliseconds per
  * iteration, averaged), measured with CUDA events on the handle's stream:
  * out[0] spawn, out[1] heavy-determinant spawn, out[2] annihilation,
- * out[3] finalize, out[4] semi-stochastic, out[5] H_jj of the determinants
- * created in the iteration.  Enabled by fciqmc_set_profiling. */
+ * out[3] finalize, out[4] semi-stochastic; out[5] was H_jj of the determinants
+ * created in the iteration, which is now part of the annihilation (out[2]).
+ * Enabled by fciqmc_set_profiling. */
 int fciqmc_set_profiling(fciqmc_handle *h, int32_t on);
 int fciqmc_kernel_times(fciqmc_handle *h, double out[6]);
 

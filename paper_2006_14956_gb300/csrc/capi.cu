@@ -129,6 +129,9 @@ static void dev_free(fciqmc_handle *h, void *ptr)
     else cudaFree(ptr);
 }
 
+// determinants per bucket a run starts with when its list is as long as expected
+constexpr double START_M = 140.0;
+
 static int64_t pair_index(int64_t i, int64_t j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
 
 // binary64 -> (mantissa, exponent) with x = m 2^e, m odd (or 0)
@@ -284,12 +287,10 @@ static int enqueue_iteration(fciqmc_handle *h, cudaEvent_t *ev)
     if (ev) cudaEventRecord(ev[2], h->stream);
     if (h->nd > 0) launch_semistoch(h->dinst, 1, h->nd, h->stream);
     if (ev) cudaEventRecord(ev[3], h->stream);
-    cudaError_t e = launch_annihilate(h->dinst, h->dunit, 1, units, h->hi.side || h->hi.adaptive,
-                                      staged_annihilation_fits(h->hi), h->stream);
+    cudaError_t e = launch_annihilate(&h->hi, h->dinst, h->dunit, 1, units, h->hi.side || h->hi.adaptive, h->stream);
     if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("annihilation launch: ") + cudaGetErrorString(e));
     launch_annihilate_big(h->dinst, 1, h->stream);
     if (ev) cudaEventRecord(ev[4], h->stream);
-    launch_new_diag(h->dinst, 1, h->stream);
     if (ev) cudaEventRecord(ev[5], h->stream);
     launch_finalize(h->dinst, 1, h->stream);
     if (ev) cudaEventRecord(ev[6], h->stream);
@@ -345,7 +346,7 @@ static int write_state(fciqmc_handle *h)
 // split every bucket in two (one more hash bit)
 static int grow_buckets(fciqmc_handle *h)
 {
-    if (h->bb >= MAX_BB) return fail(h, FCIQMC_ERR_CAPACITY, "walker list exceeds 2^22 buckets");
+    if (h->bb >= MAX_BB) return fail(h, FCIQMC_ERR_CAPACITY, "walker list exceeds 2^24 buckets");
     DevInst nI = h->hi;
     if (nI.cap_s > CAP_S0) nI.cap_s /= 2;  // each new bucket receives about half the spawns
     int rc = alloc_layout(h, nI, h->bb + 1);
@@ -435,7 +436,6 @@ static int reset_after_error(fciqmc_handle *h)
     h->hst.need_spawn = 0;
     h->hst.need_main = 0;
     h->hst.n_spawn_over = 0;
-    h->hst.new_n = 0;
     CUDA_TRY(h, cudaMemsetAsync(h->hi.acc, 0, NSHARD * ACC_STRIDE * sizeof(u64), h->stream));  // partial totals
     // the failed iteration's adaptive-shift weight sums are discarded when the
     // descriptor is next uploaded (the device copy may still describe an old
@@ -1013,7 +1013,7 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
         if (P.max_dets <= 0) dets_hint = std::min(dets_hint, std::max(1.0, fci));
     }
     int bb = 0;
-    while (((double)(1LL << bb)) * 640.0 < dets_hint && bb < MAX_BB) bb++;
+    while (((double)(1LL << bb)) * START_M < dets_hint && bb < MAX_BB) bb++;
     I.cap_s = CAP_S0;
     int rc = alloc_layout(h, I, bb);
     if (rc) return bail(rc, "out of device memory (walker buffers)");
@@ -1308,10 +1308,10 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         }
         rc = pull_history(h, start, h->hst.iter);
         if (rc) return rc;
-        if (!h->hst.err && !h->hist.empty() && h->hist.back().ndet > (1LL << h->bb) * (long long)(CAP_M / 2) &&
+        if (!h->hst.err && !h->hist.empty() && h->hist.back().ndet > (1LL << h->bb) * (long long)FILL_M &&
             h->bb < MAX_BB) {
             // keep head-room in the main buckets: split once the average
-            // occupancy passes half the capacity
+            // occupancy passes FILL_M
             rc = grow_buckets(h);
             if (rc) return rc;
             rc = reset_after_error(h);
@@ -1556,7 +1556,7 @@ static int import_device(fciqmc_handle *h, int64_t n, const uint64_t *alpha, con
     int rc = read_state(h);  // also completes the copies above
     if (rc) return rc;
     // the fewest buckets (at least the current number) that hold every
-    // bucket's determinants within half the main capacity; one allocation
+    // bucket's determinants within IMPORT_M; one allocation
     int bb = h->bb;
     for (;; bb++) {
         int *cntb = (int *)dev_alloc(h, ((size_t)1 << bb) * sizeof(int));
@@ -1616,7 +1616,7 @@ static int import_host(fciqmc_handle *h, int64_t n, const uint64_t *alpha, const
         std::vector<int> cnt_b((size_t)1 << bb, 0);
         bool over = false;
         for (int64_t i = 0; i < nt && !over; i++)
-            if (++cnt_b[bb ? (size_t)(hash[i] >> (64 - bb)) : 0] > CAP_M / 2) over = true;
+            if (++cnt_b[bb ? (size_t)(hash[i] >> (64 - bb)) : 0] > IMPORT_M) over = true;
         if (!over) break;
         if (bb >= MAX_BB)
             return fail(h, FCIQMC_ERR_INVALID_ARG, "imported keys crowd one bucket (duplicate determinants?)");
@@ -1671,7 +1671,7 @@ static int import_state_impl(fciqmc_handle *h, int64_t n, const uint64_t *alpha,
     if (rc) return rc;
     rc = upload_inst(h);
     if (rc) return rc;
-    if (listed) launch_diag_list(h->dinst, par, h->hi.newdet, (int)nt, h->stream);
+    if (listed) launch_diag_list(&h->hi, par, h->hi.newdet, (int)nt, h->stream);
     else launch_diag(h->dinst, par, (int)nbk, h->stream);
     if (h->p.adaptive_shift) launch_build_kidx(h->dinst, par, (int)nbk, h->stream);
     CUDA_TRY(h, cudaGetLastError());
@@ -1788,14 +1788,10 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         launch_spawn(nullptr, dinst, dunit, k, units, adaptive, h0->stream);
         launch_spawn_heavy(nullptr, dinst, k, h0->stream);
         if (max_nd > 0) launch_semistoch(dinst, k, max_nd, h0->stream);
-        bool general = false, staged = true;
-        for (int i = 0; i < k; i++) {
-            general = general || tab[i].side || tab[i].adaptive;
-            staged = staged && staged_annihilation_fits(tab[i]);
-        }
-        cudaError_t le = launch_annihilate(dinst, dunit, k, units, general, staged, h0->stream);
+        bool extra = false;
+        for (int i = 0; i < k; i++) extra = extra || tab[i].side || tab[i].adaptive;
+        cudaError_t le = launch_annihilate(nullptr, dinst, dunit, k, units, extra, h0->stream);
         launch_annihilate_big(dinst, k, h0->stream);
-        launch_new_diag(dinst, k, h0->stream);
         cudaError_t xe = any_pair ? launch_replica_cross(dinst, k, max_bk, h0->stream) : cudaSuccess;
         launch_finalize(dinst, k, h0->stream);
         cudaError_t e = cudaStreamEndCapture(h0->stream, &g);
@@ -2174,7 +2170,7 @@ static int64_t estimate_bytes(const Request &r)
     const double np = (double)N * (N + 1) / 2, ne = np * (np + 1) / 2;
     double dets = r.p.max_dets > 0 ? (double)r.p.max_dets : std::min(std::max(4096.0, r.p.target_walkers), 8388608.0);
     int bb = 0;
-    while (((double)(1LL << bb)) * (CAP_M / 2.5) < dets && bb < MAX_BB) bb++;
+    while (((double)(1LL << bb)) * (START_M * 0.64) < dets && bb < MAX_BB) bb++;
     const double per_bucket = 2.0 * CAP_M * (16 + 8 + 8 + 1) + 5.0 * CAP_S0 * 24.0 + 2 * 8 + sizeof(Partial) + 3 * 4 +
                               4.0 * CAP_M;
     const double ecap = CAP_M + 4.0 * CAP_S0;

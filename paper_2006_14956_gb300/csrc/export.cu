@@ -182,13 +182,13 @@ __global__ void k_import_check(const u64 *__restrict__ a, const u64 *__restrict_
 }
 
 // import, step 2: bucket counts at 2^bb buckets; *over = 1 once a bucket
-// holds more than half its capacity
+// holds more than IMPORT_M
 __global__ void k_import_count(const u64 *__restrict__ a, const u64 *__restrict__ b, long long n, int bb, int *cnt,
                                int *over)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const int o = atomicAdd(&cnt[bucket_of(det_hash(a[i], b[i]), bb)], 1);
-        if (o == CAP_M / 2) atomicOr(over, 1);
+        if (o == IMPORT_M) atomicOr(over, 1);
     }
 }
 

@@ -64,11 +64,13 @@ __device__ __forceinline__ int bucket_of(u64 h, int bb) { return bb ? (int)(h >>
 
 // ---------------------------------------------------------------- Philox4x64-10
 // Salmon, Moraes, Dror, Shaw, SC'11: ten rounds of two 64x64->128 products.
+// (UNROLL: rounds per loop turn; a kernel short of instruction cache rolls them)
+template <int UNROLL = 10>
 __device__ __forceinline__ void philox(u64 c0, u64 c1, u64 c2, u64 c3, u64 k0, u64 k1, u64 out[4])
 {
     const u64 M0 = 0xD2E7470EE14C6C93ULL, M1 = 0xCA5A826395121157ULL;
     const u64 W0 = 0x9E3779B97F4A7C15ULL, W1 = 0xBB67AE8584CAA73BULL;
-#pragma unroll
+#pragma unroll UNROLL
     for (int r = 0; r < 10; r++) {
         if (r) { k0 += W0; k1 += W1; }
         const u128 p0 = (u128)M0 * c0, p1 = (u128)M1 * c2;  // one 128-bit product each (fewer
@@ -128,21 +130,18 @@ __device__ __forceinline__ u64 ceil_abs(double c)
 
 // Eq. (3) decision "u < |v| / c_min" with u = (w >> 11) 2^-53, for 0 < |v| < c_min.
 // When c_min = 2^k the quotient is exact and the test is the integer
-// comparison (w >> 11) < ceil(|v| 2^(53-k)); otherwise binary64 as written.
+// comparison (w >> 11) < ceil(M / 2^s) for |v| 2^(53-k) = M / 2^s, that is
+// (w >> 11) <= floor((M - 1) / 2^s); otherwise binary64 as written.
+static __device__ __noinline__ bool draw_keeps_div(u64 w, double v, double cmin) { return u53(w) < fabs(v) / cmin; }
 __device__ __forceinline__ bool draw_keeps(u64 w, double v, double cmin, int cmin_log2, bool pow2)
 {
-    if (!pow2) return u53(w) < fabs(v) / cmin;
+    if (!pow2) return draw_keeps_div(w, v, cmin);
     u64 M;
     int E;
     split_abs(v, M, E);
-    int sh = E + 53 - cmin_log2;
-    u64 T;
-    if (sh >= 0) T = M << sh;
-    else {
-        int s = -sh;
-        T = s >= 64 ? 1ULL : ((M + ((1ULL << s) - 1ULL)) >> s);
-    }
-    return (w >> 11) < T;
+    const int s = cmin_log2 - 53 - E;  // |v| < c_min: s >= 0, but for a subnormal v's M below 2^52
+    const u64 t = s > 63 ? 0ULL : (M - 1) >> s;
+    return (w >> 11) <= t;
 }
 
 // Eq. (3): |v| >= c_min kept; else sign(v) c_min with probability |v|/c_min, else 0

@@ -36,15 +36,19 @@ enum { DFLAG_REF = 1, DFLAG_D = 2 };
 // launch geometry
 constexpr unsigned HEAVY_ATT = 512;   // attempts per heavy slice
 constexpr int K3_THREADS = 256;
-constexpr int EMAX = 1280;            // main + spawned records staged per bucket in shared memory (3 blocks per SM)
-constexpr int CAP_M = 1024;           // main-list capacity per bucket
-constexpr int MAX_BB = 22;            // at most 2^22 buckets: slot indices (bucket * CAP_M + position) fit 32 bits
-constexpr int CAP_S0 = EMAX - CAP_M;  // initial spawn capacity per bucket (grows at run time)
-constexpr int TABBITS = 12;           // shared-memory hash table of the annihilation (2 x EMAX slots)
+constexpr int EMAX = 1280;            // main + spawned records a large-bucket block holds in shared memory
+// A bucket holds what one warp annihilates: 48 to 96 determinants on average
+// once a list has grown (a list gets twice the buckets above 96); 96 and their
+// 0.4 x 96 spawns stay 4.7 sigma below the 192 records a warp holds.
+constexpr int CAP_M = 192;            // main-list capacity per bucket
+constexpr int FILL_M = 96;            // average occupancy above which a list is given twice the buckets
+constexpr int IMPORT_M = 160;         // determinants of an imported list per bucket at most
+constexpr int MAX_BB = 24;            // at most 2^24 buckets: slot indices (bucket * CAP_M + position) fit 32 bits
+constexpr int CAP_S0 = 96;            // initial spawn capacity per bucket (grows at run time)
+constexpr int TABBITS = 12;           // shared-memory hash table of the large-bucket kernel (2 x EMAX slots)
 constexpr int BIG_BLOCKS = 64;        // blocks of the large-bucket annihilation kernel
 constexpr int K5_THREADS = 256;
-constexpr int KIDX = 2048;            // slots of the per-bucket list index (adaptive shift)
-constexpr int STAGED_SCAP = 256;      // spawn records per bucket the staged annihilation holds
+constexpr int KIDX = 512;             // slots of the per-bucket list index (adaptive shift)
 
 struct HeavyChunk {  // a slice of the attempts of one determinant with many walkers
     u64 a, b;
@@ -111,7 +115,6 @@ struct IterState {
     double e_den;
     alignas(128) int heavy_n;
     alignas(128) int big_n; // buckets deferred to the large-bucket kernel
-    alignas(128) int new_n; // determinants created in this iteration (their H_jj is computed by k_new_diag)
 };
 
 struct TrialEnt;
@@ -164,7 +167,7 @@ struct DevInst {
     int cap_s;              // spawn capacity per bucket
     int big_tabbits;        // hash-table bits of the large-bucket path
     int *big_list;          // deferred bucket ids (capacity = buckets)
-    unsigned *newdet;       // main-list slots of the determinants created in this iteration
+    unsigned *newdet;       // main-list slots of an imported list
     unsigned char *big_scratch;  // BIG_BLOCKS slices of big_stride bytes
     size_t big_stride;
     HeavyChunk *heavy;
@@ -230,20 +233,17 @@ void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_star
                   cudaStream_t s);
 void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cudaStream_t s);
 void launch_semistoch(const DevInst *dinst, int n_inst, int max_nd, cudaStream_t s);
-cudaError_t launch_annihilate(const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool general,
-                              bool staged, cudaStream_t s);
-bool staged_annihilation_fits(const DevInst &I);
+cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units,
+                              bool extra, cudaStream_t s);
 cudaError_t init_kernels();
-size_t annihilate_smem_bytes();
 void launch_annihilate_big(const DevInst *dinst, int n_inst, cudaStream_t s);
 void launch_finalize(const DevInst *dinst, int n_inst, cudaStream_t s);
-void launch_new_diag(const DevInst *dinst, int n_inst, cudaStream_t s);
 void launch_build_kidx(const DevInst *dinst, int parity, int nb, cudaStream_t s);
 cudaError_t launch_replica_cross(const DevInst *dinst, int n_inst, int max_buckets, cudaStream_t s);
 cudaError_t replica_kernel_init();
 void launch_rebucket(const DevInst *src, const DevInst *dst, int nb_src, int parity, cudaStream_t s);
 void launch_diag(const DevInst *dinst, int parity, int nb, cudaStream_t s);
-void launch_diag_list(const DevInst *dinst, int par, const unsigned *list, int nn, cudaStream_t s);
+void launch_diag_list(const DevInst *one, int par, const unsigned *list, int nn, cudaStream_t s);
 cudaError_t launch_import_check(const u64 *a, const u64 *b, const double *c, long long n, int na, int nb, u64 normask,
                                 u64 ra, u64 rb, int *flags, cudaStream_t s);
 cudaError_t launch_import_count(const u64 *a, const u64 *b, long long n, int bb, int *cnt, int *over, cudaStream_t s);

@@ -10,16 +10,14 @@
 //   k_spawn_heavy  the same for determinants with many walkers, split into
 //                  fixed-size slices so no warp waits on one heavily
 //                  populated determinant.
-//   annihilation   (b)+(c) per bucket: the bucket's walkers and spawns in
-//                  shared memory (k_annihilate_staged: bulk copies one bucket
-//                  ahead; k_annihilate: plain loads), equal determinants
-//                  grouped in a shared open-addressing table, death and
-//                  rounding, the spawns summed exactly, the initiator rule and
-//                  rounding, the new bucket written, the new determinants
-//                  listed, and N_w, E_num (Eq. (9)) and the counts added to
-//                  the run's exact totals by global reductions.
-//   k_annihilate_big  the same for buckets too large for shared memory.
-//   k_new_diag     exact H_jj of the determinants created in the iteration.
+//   k_annihilate   (b)+(c) one warp per bucket, the bucket's walkers and
+//                  spawns in the warp's shared memory: equal determinants
+//                  found through a small hash table, death and rounding, the
+//                  spawns summed exactly, the initiator rule and rounding, the
+//                  new bucket written, exact H_jj of the new determinants, and
+//                  N_w, E_num (Eq. (9)) and the counts added to the run's
+//                  exact totals by global reductions.
+//   k_annihilate_big  the same for buckets with more records, a block each.
 //   k_finalize     per run: read and clear the exact totals, update the
 //                  shift, append the statistics row, flip the buffers.
 // Options add work to these launches or one more: the semi-stochastic
@@ -73,11 +71,13 @@ __device__ __forceinline__ bool in_D(const DevInst &I, u64 a, u64 b)
 // kernel parameter (its fields are constant-bank operands), or a table of
 // runs with the first unit (bucket) of each
 struct OneRun {
+    static constexpr bool SINGLE = true;
     const DevInst &I;
     __device__ __forceinline__ const DevInst &inst(int) const { return I; }
     __device__ __forceinline__ int find(int) const { return 0; }
 };
 struct RunTable {
+    static constexpr bool SINGLE = false;
     const DevInst *__restrict__ t;
     const int *__restrict__ start;
     int n;
@@ -351,7 +351,8 @@ __device__ __forceinline__ int classify(const DevInst &I, u64 w0, u64 w1, unsign
 // There is no block barrier and an attempt never leaves the chip: at 7.3e7
 // determinants and 9.1e7 attempts (50 orbitals) a block-per-bucket draw with
 // 48-byte attempt records in global memory and a second kernel for the
-// evaluation took 8.6 ms.
+// evaluation took 8.6 ms; this takes 4.7 ms, issue slots 64 % used (the ten
+// Philox rounds' 32 x 32 products alone keep the heavy FMA pipe at 42 %).
 constexpr int SP_THREADS = 256, SP_WARPS = SP_THREADS / 32, RING = 64;
 constexpr int CHUNK_S = 512;  // attempts per slice of a heavily populated determinant
 static_assert(HEAVY_ATT == (unsigned)CHUNK_S, "heavy slices");
@@ -411,6 +412,18 @@ __device__ __forceinline__ void eval_singles(const DevInst &I, SpawnWarp &W, int
     }
     nq -= n;
     __syncwarp();
+}
+
+// ... until fewer than `keep` wait
+__device__ __forceinline__ void drain_adaptive(const DevInst &I, const SpawnRun &R, unsigned keep)
+{
+    if (!R.aq) return;
+    for (;;) {
+        __syncwarp();
+        if (R.aq->n < keep) return;
+        __syncwarp();
+        eval_adaptive(I, R);
+    }
 }
 
 // one attempt per lane (lanes with `on`): draw, classify, evaluate or queue
@@ -709,12 +722,13 @@ __device__ __forceinline__ void heavy_body(const RUNS &runs, int n_inst)
             {
                 attempts32<GEN_ANY>(I, W, nq, R, a + lane < h.count, make_ulonglong2(h.a, h.b), h.k0 + a + lane, h.cper,
                                     h.flags, h.slot);
+                drain_adaptive(I, R, 32);  // each step below and above queues at most 32 more
                 if (nq >= 32) eval_singles(I, W, nq, R);
-                while (R.aq && __shfl_sync(0xffffffffu, R.aq->n, 0) >= 32u) eval_adaptive(I, R);
+                drain_adaptive(I, R, 32);
             }
         }
         if (nq > 0) eval_singles(I, W, nq, R);
-        while (R.aq && __shfl_sync(0xffffffffu, R.aq->n, 0) > 0u) eval_adaptive(I, R);
+        drain_adaptive(I, R, 1);
     }
 }
 
@@ -728,15 +742,604 @@ __global__ void __launch_bounds__(SP_THREADS, 3) k_spawn_heavy_batch(const DevIn
     heavy_body(RunTable{insts, nullptr, n_inst}, n_inst);
 }
 
+// slot of determinant (a, b) in the trial-estimator table, or -1
+__device__ __forceinline__ int trial_find(const DevInst &I, u64 a, u64 b)
+{
+    const u64 mask = (1ULL << I.trial_bits) - 1;
+    u64 s = det_hash(a, b) & mask;
+    for (u64 probe = 0; probe <= mask; probe++) {
+        if (__ldg(I.trial_state + s) == 0u) return -1;
+        if (__ldg(&I.trial_tab[s].a) == a && __ldg(&I.trial_tab[s].b) == b) return (int)s;
+        s = (s + 1) & mask;
+    }
+    return -1;
+}
+
 // ------------------------------------------------------------------ annihilation
-// Per bucket, one block: the bucket's walkers and spawns are staged (shared
-// memory for up to EMAX records, a global scratch slice for larger buckets)
-// and every distinct determinant gets one owner record through an
-// open-addressing table: walkers are inserted first, then every spawn finds
-// its target or inserts itself as the owner of a new determinant.  Accepted
-// weights are added to the owner's exact 128-bit accumulator with two 64-bit
-// atomics (the low word's carry goes to the high word), so the sum does not
-// depend on the order of arrival.
+// One warp per bucket: the bucket's walkers and spawns (up to AW_E records;
+// larger buckets go to k_annihilate_big) meet in the warp's own shared
+// memory, without a block barrier:
+//   A  walkers: keys and C into shared memory and into a small hash table
+//      (one byte per slot: the record);
+//   B  spawns: each finds its target or becomes the record of a new
+//      determinant; the initiator rule (Sec. I: a non-initiator's spawn
+//      survives only onto a determinant occupied at the start of the
+//      iteration); an accepted spawn is pushed on its target's list;
+//   C  rounds of 32 records: walkers (death (b) and Eq. (3), then their
+//      spawns added), new determinants (the sum of their spawns), and last
+//      the records whose sum needs the rounding draw of the annihilation,
+//      few enough that they are collected first.  Kept records go to the new
+//      bucket in order.  Sums are exact and rounded once, so no order matters.
+// New determinants wait in a queue of the warp for H_jj until there are 32.
+// The table needs no atomics: lanes claim a free slot by writing their record
+// and look who stayed.  A block of 256 threads per bucket of 1024 slots (three
+// barriers per bucket, 128-bit shared accumulators, two blocks per SM) spent
+// 5.6 of 14 stall cycles per instruction at those barriers: 7.13 ms at 7.3e7
+// determinants and 3.5e7 spawns (50 orbitals), and 0.87 ms more for H_jj in a
+// kernel of its own; this takes 4.93 ms for both.  It is bound by instruction
+// fetch (the warps of an SM are at different places of a long code) and
+// latency, DRAM at 10 %.
+constexpr int AN_THREADS = 256, AN_WARPS = AN_THREADS / 32;
+constexpr int AW_E = 192;          // records per warp (bytes of the table index them: below 255)
+constexpr int AW_TAB = 512;
+constexpr unsigned AW_NONE = 0xffu;
+constexpr int ND_MAX = 64;         // electrons the pair table covers
+constexpr int ND_PAIRS = ND_MAX * (ND_MAX - 1) / 2;
+
+struct AnniWarp {
+    ulonglong2 key[AW_E];          // walkers [0, m), spawns [m, m + s)
+    double val[AW_E];              // C (walkers), w (spawns); the sum of a record waiting for its draw
+    int head[AW_E];                // the record last pushed on this record's list, -1: none
+    unsigned short next[AW_E];     // the one pushed before it (0xffff: none); bit 15 of the index: rejected
+    unsigned char tab[AW_TAB];
+    unsigned char list[2 * AW_E];  // records of new determinants, then those waiting for the annihilation draw
+    unsigned newq[32 + AW_E];      // slots of new determinants waiting for H_jj
+    unsigned enq[32 + AW_E];       // slots of determinants connected to the reference waiting for their E_num term
+    unsigned char orb[4][ND_MAX];
+};
+constexpr size_t AN_SMEM = AN_WARPS * sizeof(AnniWarp) + ND_PAIRS * sizeof(unsigned short);
+static_assert(KIDX * sizeof(unsigned short) <= AW_E * sizeof(ulonglong2), "the new list's index is built over the keys");
+static_assert(3 * (AN_SMEM + 1024) <= 233472, "resident annihilation blocks per SM");
+static_assert(AW_E < (int)AW_NONE && CAP_M <= 0x7fff, "records in a byte, list links in 15 bits");
+
+// A warp's share of a run's exact integer totals over the buckets it meets
+// in one launch (integer sums: any order gives the same total)
+struct AnniTotals {
+    u128 nw = 0;            // N_w * 2^32
+    i128 ann = 0;           // annihilated walkers * 2^32
+    i128 enm = 0;           // E_num * 2^Fe (terms truncated to the grid)
+    long long rej = 0;      // rejected non-initiator spawns
+    long long ndet = 0;     // determinants kept (lane 0)
+    long long spawns = 0;   // spawns received (lane 0)
+};
+
+// the totals of a warp into the run's accumulators (line w % NSHARD), then zero
+__device__ __forceinline__ void anni_flush(const DevInst &I, AnniTotals &T, int w)
+{
+    const int lane = threadIdx.x & 31;
+    for (int mm = 16; mm >= 1; mm >>= 1) {
+        T.rej += __shfl_xor_sync(0xffffffffu, T.rej, mm);
+        T.ann += shfl_xor_i128(T.ann, mm);
+        T.nw += (u128)shfl_xor_i128((i128)T.nw, mm);
+        T.enm += shfl_xor_i128(T.enm, mm);
+    }
+    if (lane == 0) {
+        u64 *acc = I.acc + (w % NSHARD) * ACC_STRIDE;
+        limb_add(acc + ACC_NW, (i128)T.nw);
+        limb_add(acc + ACC_ANN, T.ann);
+        limb_add(acc + ACC_ENUM, T.enm);
+        if (T.rej) red_add(&acc[ACC_REJ], (u64)T.rej);
+        if (T.ndet) red_add(&acc[ACC_NDET], (u64)T.ndet);
+        if (T.spawns) red_add(&acc[ACC_SPAWNS], (u64)T.spawns);
+    }
+    T = AnniTotals{};
+}
+
+// the E_num term of a determinant connected to the reference, on the grid
+// 2^-Fe (R12)
+__device__ __noinline__ i128 enum_term(const DevInst &I, u64 a, u64 b, double c)
+{
+    if (I.kind == FCIQMC_HUBBARD) {  // only a hop along a bond couples: H = -+ t = h_ai
+        const u64 d = a == I.ref_a ? b ^ I.ref_b : a ^ I.ref_a, x = a == I.ref_a ? b : a;
+        if ((a != I.ref_a && b != I.ref_b) || __popcll(d) != 2) return 0;
+        const int i = __ffsll((long long)d) - 1, j = 63 - __clzll((long long)d);
+        const double H = neg_if(__popcll(x & between(i, j)) & 1, __ldg(I.h + i * I.norb + j));
+        return is_zero(H) ? (i128)0 : to_fixed(H * c, I.Fe);
+    }
+    return to_fixed(hoff_generic(I, a, b, I.ref_a, I.ref_b) * c, I.Fe);
+}
+
+// death of a determinant in D (the exact projection's result) or, with the
+// adaptive shift (Sec. V), of a non-initiator: S_i = f_i S
+__device__ __noinline__ double death_special(const DevInst &I, u64 a, u64 b, double c, double hd, unsigned f, int par,
+                                             size_t slot, double shift)
+{
+    if (f & DFLAG_D) return I.dc_new[d_index_of(I, a, b)];
+    double Si = shift;
+    if ((dbits(c) & ~SIGN64) <= dbits(I.n_a) && !(f & DFLAG_REF)) {
+        const u64 *acc = I.facc[par] + slot * 4;
+        const u128 A = ((u128)acc[1] << 64) | acc[0], T = ((u128)acc[3] << 64) | acc[2];
+        if (T != 0) Si = (u128_to_double(A) / u128_to_double(T)) * shift;
+    }
+    return c * (1.0 - I.tau * (hd - Si));
+}
+
+// a kept determinant of D, and the reference
+__device__ __noinline__ void keep_special(const DevInst &I, u64 a, u64 b, double c, unsigned f, int np)
+{
+    if (f & DFLAG_REF) I.st->e_den = c;
+    if (f & DFLAG_D) I.dc_buf[np][d_index_of(I, a, b)] = c;
+}
+
+// H_jj - E_ref of a lattice: U times the doubly occupied sites
+__device__ __noinline__ double lattice_diag(const DevInst &I, u64 a, u64 b)
+{
+    const i128 xr = (i128)(((u128)I.xref_hi << 64) | (u128)I.xref_lo);
+    return fixed_to_double((i128)__popcll(a & b) * fx_load(I.Jfx, 0) - xr, I.F);
+}
+
+// (numerator, denominator) of the trial-wave-function estimator (Sec. IV)
+__device__ __noinline__ double2 trial_terms(const DevInst &I, u64 a, u64 b, double c)
+{
+    const int ts = is_zero(c) ? -1 : trial_find(I, a, b);
+    if (ts < 0) return make_double2(0.0, 0.0);
+    return make_double2(__ldg(&I.trial_tab[ts].w) * c, __ldg(&I.trial_tab[ts].cT) * c);
+}
+
+// the lines of bucket b that its warp will read, into L2: one line per lane
+// (the first 64 keys, C and H_ii, the flags, the spawns at both ends of their region)
+__device__ __forceinline__ void prefetch_bucket(const DevInst &I, int b, int par)
+{
+    const int lane = threadIdx.x & 31;
+    const size_t base = (size_t)b * CAP_M, s0 = (size_t)b * I.cap_s, s1 = s0 + I.cap_s;
+    const char *p;
+    if (lane < 8) p = (const char *)(I.key[par] + base) + 128 * lane;
+    else if (lane < 12) p = (const char *)(I.c[par] + base) + 128 * (lane - 8);
+    else if (lane < 16) p = (const char *)(I.hd[par] + base) + 128 * (lane - 12);
+    else if (lane == 16) p = (const char *)(I.fl[par] + base);
+    else if (lane < 19) p = (const char *)(I.skey + s0) + 128 * (lane - 17);
+    else if (lane < 22) p = (const char *)(I.skey + s1) - 16 - 128 * (lane - 19);
+    else if (lane == 22) p = (const char *)(I.sw + s0);
+    else if (lane < 25) p = (const char *)(I.sw + s1) - 8 - 128 * (lane - 23);
+    else return;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// exact sum of a list of three or more accepted spawns, rounded once
+__device__ __noinline__ double list_sum(const AnniWarp &W, int h, int Fw)
+{
+    i128 x = 0;
+    for (int e = h; e >= 0;) {
+        const unsigned nx = W.next[e & 0x7fff];
+        if (!(e & 0x8000)) x += to_fixed(W.val[e], Fw);
+        e = nx == 0xffffu ? -1 : (int)nx;
+    }
+    return fixed_to_double(x, Fw);
+}
+
+// exact sum of the rejected spawns of a list, rounded once (replica pairs)
+__device__ __noinline__ double list_sum_rejected(const AnniWarp &W, int h, int Fw)
+{
+    i128 x = 0;
+    for (int e = h; e >= 0;) {
+        const unsigned nx = W.next[e & 0x7fff];
+        if (e & 0x8000) x += to_fixed(W.val[e & 0x7fff], Fw);
+        e = nx == 0xffffu ? -1 : (int)nx;
+    }
+    return fixed_to_double(x, Fw);
+}
+
+// H_jj - E_ref of up to four determinants of list `np` (slots q[0 .. cnt)),
+// eight lanes each: their terms h_pp (electron e1) and pairs e1 < e2 (listed
+// in `pair`, e1 | e2 << 8), four loads in flight per lane, exact sum, rounded once
+__device__ __forceinline__ void diag_four(const DevInst &I, const unsigned *q, int cnt, int np,
+                                          const unsigned short *pair, unsigned char (*orb)[ND_MAX])
+{
+    const int lane = threadIdx.x & 31, g = lane >> 3, sl = lane & 7;
+    const int n = I.n, na = I.na, N = I.norb, T = n + n * (n - 1) / 2;
+    const unsigned d = q[g < cnt ? g : 0];
+    const ulonglong2 key = I.key[np][d];
+    for (int e = sl; e < n; e += 8)
+        orb[g][e] = (unsigned char)(e < na ? nth_set(key.x, e) : nth_set(key.y, e - na));
+    __syncwarp();
+    i128 part = 0;
+    for (int t0 = sl; t0 < T; t0 += 32) {
+        ulonglong2 v[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const int t = t0 + 8 * r;
+            v[r] = make_ulonglong2(0, 0);
+            if (t < n) v[r] = __ldg(I.hfx + orb[g][t]);
+            else if (t < T) {
+                const unsigned tm = pair[t - n];
+                const int e1 = (int)(tm & 0xffu), e2 = (int)(tm >> 8);
+                v[r] = __ldg((((e1 < na) == (e2 < na)) ? I.JKfx : I.Jfx) + orb[g][e1] * N + orb[g][e2]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++) part += (i128)(((u128)v[r].y << 64) | (u128)v[r].x);
+    }
+    for (int m = 4; m >= 1; m >>= 1) part += shfl_xor_i128(part, m);
+    const i128 xref = (i128)(((u128)I.xref_hi << 64) | (u128)I.xref_lo);
+    if (sl == 0 && g < cnt) I.hd[np][d] = fixed_to_double(part - xref, I.F);
+    __syncwarp();
+}
+
+// the same for more electrons than the pair table covers
+__device__ __noinline__ void diag_generic(const DevInst &I, const unsigned *q, int cnt, int np)
+{
+    for (int k = 0; k < cnt; k++) {
+        const ulonglong2 kk = I.key[np][q[k]];
+        const double hdv = diag_exact_warp(I, kk.x, kk.y);
+        if ((threadIdx.x & 31) == 0) I.hd[np][q[k]] = hdv;
+    }
+    __syncwarp();
+}
+
+// the pairs e1 < e2 of up to ND_MAX electrons, in the order of e2 (whole block)
+__device__ __forceinline__ void fill_pairs(unsigned short *pair)
+{
+    for (int c = 1 + (int)(threadIdx.x >> 5); c < ND_MAX; c += (int)(blockDim.x >> 5))
+        for (int r = (int)(threadIdx.x & 31); r < c; r += 32) pair[c * (c - 1) / 2 + r] = (unsigned short)(r | (c << 8));
+    __syncthreads();
+}
+
+// H_jj of queued new determinants: 32 at a time, one per lane (half the
+// instructions of eight lanes per determinant, and no reduction); a run's
+// last few by eight lanes each (a quarter of the latency)
+__device__ __forceinline__ void new_diag(const DevInst &I, AnniWarp &W, int &nq, int np, const unsigned short *pair, bool all)
+{
+    __syncwarp();
+    while (nq >= 32 || (all && nq > 8)) {
+        const int lane = threadIdx.x & 31, cnt = min(nq, 32);
+        nq -= cnt;
+        if (lane < cnt) {
+            const unsigned d = W.newq[nq + lane];
+            const ulonglong2 kk = I.key[np][d];
+            I.hd[np][d] = diag_exact_thread(I, kk.x, kk.y);
+        }
+        __syncwarp();
+    }
+    while (all && nq > 0) {
+        const int cnt = min(nq, 4);
+        nq -= cnt;
+        if (I.n <= ND_MAX) diag_four(I, W.newq + nq, cnt, np, pair, W.orb);
+        else diag_generic(I, W.newq + nq, cnt, np);
+    }
+}
+
+// the E_num terms of queued determinants, 32 at a time (one determinant in a
+// hundred is connected to the reference, but its term costs a warp hundreds of
+// instructions whatever its active lanes: taken where it was found it was 235
+// of 756 us at 7.6e6 determinants, 50 orbitals)
+__device__ __forceinline__ void enum_queue(const DevInst &I, AnniWarp &W, int &ne, int np, bool all, AnniTotals &T)
+{
+    __syncwarp();
+    while (ne >= 32 || (all && ne > 0)) {
+        const int lane = threadIdx.x & 31, cnt = min(ne, 32);
+        ne -= cnt;
+        if (lane < cnt) {
+            const unsigned d = W.enq[ne + lane];
+            const ulonglong2 kk = I.key[np][d];
+            T.enm += enum_term(I, kk.x, kk.y, I.c[np][d]);
+        }
+        __syncwarp();
+    }
+}
+
+// EXTRA: some run of the launch has replica side lists or the adaptive shift
+template <bool EXTRA>
+__device__ __forceinline__ void anni_bucket_warp(const DevInst &I, AnniWarp &W, int b, int par, long long it,
+                                                 double shift, int m, int si, int sn, AnniTotals &T, int &nq, int &ne)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u, full = 0xffffffffu;
+    const int E = m + si + sn, np = par ^ 1;
+    const size_t base = (size_t)b * CAP_M, sbase = (size_t)b * I.cap_s;
+    constexpr unsigned tmask = AW_TAB - 1;
+    const bool side = EXTRA && I.side != nullptr, adaptive = EXTRA && I.adaptive;
+
+    // A
+    __syncwarp();
+    {
+        uint4 *tz = reinterpret_cast<uint4 *>(W.tab);
+        for (int q = lane; q < AW_TAB / 16; q += 32) tz[q] = make_uint4(full, full, full, full);
+    }
+    for (int e = lane; e < E; e += 32) W.head[e] = -1;
+    __syncwarp();
+    // A and B in rounds of 32 records: walkers and spawns share the rounds'
+    // code; a round holds one kind
+    const int ra = (m + 31) >> 5, rb = (si + sn + 31) >> 5;
+    long long rejected = 0;
+    for (int r = 0; r < ra + rb; r++) {
+        const bool walk = r < ra;
+        const int q = (walk ? r : r - ra) * 32 + lane;    // walker or spawn number
+        const bool on = q < (walk ? m : si + sn);
+        const int e = walk ? q : m + q;
+        ulonglong2 k = make_ulonglong2(0, 0);
+        double v = 0.0;
+        if (on) {
+            const size_t o = walk ? base + q : sbase + (q < si ? q : I.cap_s - 1 - (q - si));
+            k = (walk ? I.key[par] : I.skey)[o];
+            v = (walk ? I.c[par] : I.sw)[o];
+            W.key[e] = k;
+            W.val[e] = v;
+        }
+        __syncwarp();
+        unsigned s = (unsigned)det_hash(k.x, k.y) & tmask;
+        int target = -1;
+        bool open = on;
+        while (__any_sync(full, open)) {
+            unsigned x = AW_NONE;
+            if (open) {
+                x = W.tab[s];
+                if (x == AW_NONE) W.tab[s] = (unsigned char)e;
+            }
+            __syncwarp();
+            if (open) {
+                if (x == AW_NONE) x = W.tab[s];  // the claim that stayed
+                if ((int)x == e) { target = e; open = false; }
+                else {
+                    bool same = false;
+                    if (!walk) {  // walkers are distinct
+                        const ulonglong2 kk = W.key[x];
+                        same = kk.x == k.x && kk.y == k.y;
+                    }
+                    if (same) { target = (int)x; open = false; }
+                    else s = (s + 1) & tmask;
+                }
+            }
+        }
+        if (!walk && on) {
+            const bool accepted = q < si || (target < m && !is_zero(W.val[target]));
+            if (accepted || side) {
+                const int old = atomicExch(&W.head[target], accepted ? e : (e | 0x8000));
+                W.next[e] = (unsigned short)(old < 0 ? 0xffff : old);
+            }
+            if (!accepted) rejected++;
+        }
+    }
+    __syncwarp();
+    T.rej += rejected;
+
+    // new determinants that hold spawns (side lists: every new one)
+    int nown = 0;
+    for (int q0 = 0; q0 < si + sn; q0 += 32) {
+        const bool own = q0 + lane < si + sn && W.head[m + q0 + lane] >= 0;
+        const unsigned mo = __ballot_sync(full, own);
+        if (own) W.list[nown + __popc(mo & below)] = (unsigned char)(m + q0 + lane);
+        nown += __popc(mo);
+    }
+    __syncwarp();
+
+    // C: items [0, m) walkers, [m, m + nown) new determinants, then those
+    // waiting for their draw (W.list past nown), which join as they appear
+    int total = 0, items = m + nown;
+    bool bad = false;
+    double tnum = 0.0, tden = 0.0;
+    for (int i0 = 0; i0 < items;) {
+        const int i = i0 + lane;
+        const bool on = i < items, walk = i < m, pend = i >= m + nown;
+        i0 = min(i0 + 32, items);
+        const int e = !on ? 0 : (walk ? i : (int)W.list[i - m]);
+        const bool old = on && e < m;  // a determinant of the old list
+        int h = -1;
+        ulonglong2 k = make_ulonglong2(0, 0);
+        double v = 0.0, hd = 0.0;
+        unsigned f = 0;
+        if (on) {
+            k = W.key[e];
+            if (!pend) h = W.head[e];
+            if (walk || pend) v = W.val[e];
+            if (old) {
+                hd = I.hd[par][base + e];
+                f = I.fl[par][base + e];
+            }
+        }
+        const double c0 = v;
+        bool draw = on && pend;
+        if (on && walk) {
+            if ((f & DFLAG_D) || adaptive) v = death_special(I, k.x, k.y, v, hd, f, par, base + e, shift);
+            else v = v * (1.0 - I.tau * (hd - shift));  // C (1 - tau (H_ii - E_ref - S))
+            draw = !(f & DFLAG_D) && !is_zero(v) && abs_lt(v, I.cmin);
+        }
+        if (__any_sync(full, draw)) {
+            u64 w[4];
+            philox<2>(k.x, k.y, (u64)it, (u64)(pend ? PURPOSE_ANNIH : PURPOSE_DEATH), I.seed, I.replica, w);
+            if (draw) v = round_stoch(v, I.cmin, I.cmin_log2, I.cmin_pow2, w[0]);
+        }
+        bool later = false;
+        double sacc = 0.0;
+        if (h >= 0) {
+            // the accepted spawns: one is exact, the exact sum of two rounded
+            // once is the binary64 sum; more go through the fixed-point sum
+            const double cp = v;
+            int cnt = 0;
+            for (int x = h; x >= 0;) {
+                const unsigned nx = W.next[x & 0x7fff];
+                if (!EXTRA || !(x & 0x8000)) {
+                    const double wv = W.val[x];
+                    sacc = cnt ? sacc + wv : wv;
+                    cnt++;
+                    T.ann += (i128)fx32(wv);
+                }
+                x = nx == 0xffffu ? -1 : (int)nx;
+            }
+            if (cnt > 2) sacc = list_sum(W, h, I.Fw);
+            if (cnt) {
+                v = walk ? cp + sacc : sacc;
+                T.ann += (walk ? (i128)fx32(cp) : (i128)0) - (i128)fx32(v);
+                later = !(f & DFLAG_D) && !is_zero(v) && abs_lt(v, I.cmin);
+            }
+        }
+        if (side && on && !pend) {  // replica pair: the record's entry
+            SideEnt &se = I.side[(size_t)b * I.side_cap + i];
+            se.a = k.x; se.b = k.y;
+            se.c0 = walk ? c0 : 0.0;
+            se.hd = walk ? hd : 0.0;
+            se.sacc = sacc;
+            se.srej = h >= 0 ? list_sum_rejected(W, h, I.Fw) : 0.0;
+        }
+        const unsigned ml = __ballot_sync(full, later);
+        if (later) {
+            W.list[items - m + __popc(ml & below)] = (unsigned char)e;
+            W.val[e] = v;
+        }
+        items += __popc(ml);
+        const bool keep = on && !later && (!is_zero(v) || (f & (DFLAG_REF | DFLAG_D)));
+        const unsigned mk = __ballot_sync(full, keep);
+        const int pos = total + __popc(mk & below);
+        total += __popc(mk);
+        const bool write = keep && pos < CAP_M, lattice = I.kind == FCIQMC_HUBBARD;
+        const unsigned mn = __ballot_sync(full, write && !old && !lattice);
+        if (write) {
+            const size_t dst = base + pos;
+            I.key[np][dst] = k;
+            I.c[np][dst] = v;
+            I.fl[np][dst] = (uint8_t)(f & (DFLAG_REF | DFLAG_D));
+            if (!old && lattice) hd = lattice_diag(I, k.x, k.y);
+            if (old || lattice) I.hd[np][dst] = hd;
+            else W.newq[nq + __popc(mn & below)] = (unsigned)dst;
+            if (!abs_lt(v, 0x1p31)) bad = true;
+            else T.nw += fx32(v);
+            if (f & (DFLAG_REF | DFLAG_D)) keep_special(I, k.x, k.y, v, f, np);
+            if (I.trial_bits) {
+                const double2 x = trial_terms(I, k.x, k.y, v);
+                tnum = tnum + x.x;
+                tden = tden + x.y;
+            }
+            if (adaptive) {
+                u64 *acc = I.facc[np] + dst * 4;
+                acc[0] = 0; acc[1] = 0; acc[2] = 0; acc[3] = 0;
+            }
+        }
+        nq += __popc(mn);
+        const bool conn = write && !(f & DFLAG_REF) && !is_zero(v) &&
+                          __popcll(k.x ^ I.ref_a) + __popcll(k.y ^ I.ref_b) <= 4;
+        const unsigned me = __ballot_sync(full, conn);
+        if (conn) W.enq[ne + __popc(me & below)] = (unsigned)(base + pos);
+        ne += __popc(me);
+        __syncwarp();
+    }
+    if (bad) atomicOr(&I.st->err, ERRB_NUMERIC);
+    if (adaptive && total <= CAP_M) {
+        // the new list's index (hash -> position + 1) for the next iteration's
+        // spawns, built where the keys were
+        unsigned short *kx = reinterpret_cast<unsigned short *>(W.key);
+        for (int q = lane; q < KIDX; q += 32) kx[q] = 0;
+        __syncwarp();
+        for (int p0 = 0; p0 < total; p0 += 32) {
+            const int p = p0 + lane;
+            bool open = p < total;
+            unsigned s = 0;
+            if (open) {
+                const ulonglong2 k = I.key[np][base + p];
+                s = (unsigned)det_hash(k.x, k.y) & (unsigned)(KIDX - 1);
+            }
+            while (__any_sync(full, open)) {
+                unsigned x = 1;
+                if (open) {
+                    x = kx[s];
+                    if (x == 0) kx[s] = (unsigned short)(p + 1);
+                }
+                __syncwarp();
+                if (open) {
+                    if (x == 0 && kx[s] == (unsigned short)(p + 1)) open = false;
+                    else s = (s + 1) & (unsigned)(KIDX - 1);
+                }
+            }
+        }
+        __syncwarp();
+        for (int q = lane; q < KIDX; q += 32) I.kidx[np][(size_t)b * KIDX + q] = kx[q];
+    }
+    if (I.trial_bits)  // binary64 sums, only when the estimator is on
+        for (int mm = 16; mm >= 1; mm >>= 1) {
+            tnum = tnum + __shfl_xor_sync(full, tnum, mm);
+            tden = tden + __shfl_xor_sync(full, tden, mm);
+        }
+    if (lane == 0) {
+        if (total > CAP_M) { atomicOr(&I.st->err, ERRB_MAIN_CAP); atomicMax(&I.st->need_main, total); }
+        else I.cnt[np][b] = total;
+        T.ndet += total;
+        T.spawns += si + sn;
+        if (I.trial_bits) { I.part[b].t_num = tnum; I.part[b].t_den = tden; }
+        if (side) I.side_cnt[b] = m + nown;
+        I.scnt_i[b] = 0;
+        I.scnt_n[b] = 0;
+    }
+}
+
+template <bool EXTRA, typename RUNS>
+__device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
+{
+    extern __shared__ __align__(16) unsigned char an_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    AnniWarp &W = reinterpret_cast<AnniWarp *>(an_raw)[warp];
+    unsigned short *pair = reinterpret_cast<unsigned short *>(an_raw + AN_WARPS * sizeof(AnniWarp));
+    const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
+    fill_pairs(pair);
+    AnniTotals T;
+    int cur = -1, err = 0, par = 0, nq = 0, ne = 0;
+    long long it = 0;
+    double shift = 0.0;
+    for (int u = gw;; u += nw) {
+        const int ii = u < n_units ? runs.find(u) : -1;
+        if (ii < 0 && cur < 0) return;  // a warp without buckets
+        if (cur >= 0 && (nq >= 32 || (ii != cur && nq > 0))) new_diag(runs.inst(cur), W, nq, par ^ 1, pair, ii != cur);
+        if (cur >= 0 && (ne >= 32 || (ii != cur && ne > 0))) enum_queue(runs.inst(cur), W, ne, par ^ 1, ii != cur, T);
+        if (ii != cur) {
+            // the run's state at the start of the iteration, read once per run a warp meets
+            if (cur >= 0) anni_flush(runs.inst(cur), T, gw);
+            if (ii < 0) return;
+            const DevInst &I = runs.inst(ii);
+            cur = ii;
+            err = __shfl_sync(0xffffffffu, *(volatile int *)&I.st->err, 0);
+            par = I.st->parity;
+            it = I.st->iter;
+            shift = I.st->S;
+        }
+        if (err) continue;
+        const DevInst &I = runs.inst(cur);
+        const int b = u - I.unit0;
+        const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
+        if (RUNS::SINGLE && u + nw < n_units) prefetch_bucket(I, b + nw, par);
+        if (si + sn > I.cap_s) {
+            if (lane == 0) {
+                atomicOr(&I.st->err, ERRB_SPAWN_CAP);
+                atomicMax(&I.st->need_spawn, si + sn);
+                atomicAdd(&I.st->n_spawn_over, 1);
+            }
+        } else if (m + si + sn > AW_E) {  // deferred to k_annihilate_big
+            if (lane == 0) I.big_list[atomicAdd(&I.st->big_n, 1)] = b;
+        } else {
+            anni_bucket_warp<EXTRA>(I, W, b, par, it, shift, m, si, sn, T, nq, ne);
+        }
+    }
+}
+
+template <bool EXTRA>
+__global__ void __launch_bounds__(AN_THREADS, 3) k_annihilate(const __grid_constant__ DevInst I, int n_units)
+{
+    anni_body<EXTRA>(OneRun{I}, n_units);
+}
+
+template <bool EXTRA>
+__global__ void __launch_bounds__(AN_THREADS, 3) k_annihilate_batch(const DevInst *__restrict__ insts,
+                                                                            const int *__restrict__ unit_start,
+                                                                            int n_inst, int n_units)
+{
+    anni_body<EXTRA>(RunTable{insts, unit_start, n_inst}, n_units);
+}
+
+// ------------------------------------------------------------------ large buckets
+// A bucket with more records than a warp holds: one block, the records staged
+// (shared memory for up to EMAX, a global scratch slice beyond) and every
+// distinct determinant given one owner record through an open-addressing
+// table: walkers are inserted first, then every spawn finds its target or
+// inserts itself as the owner of a new determinant.  Accepted weights are
+// added to the owner's exact 128-bit accumulator with two 64-bit atomics (the
+// low word's carry goes to the high word), so the sum does not depend on the
+// order of arrival.
 template <typename IDX>
 struct Stage {
     ulonglong2 *key;
@@ -773,7 +1376,7 @@ struct K3Smem {
     unsigned short tab[1 << TABBITS];
     unsigned short opos[EMAX];
 };
-static_assert(3 * (sizeof(K3Smem) + 1024) <= 233472, "three annihilation blocks per SM");
+static_assert(3 * (sizeof(K3Smem) + 1024) <= 233472, "three large-bucket blocks per SM");
 
 __device__ __forceinline__ int block_excl_scan(int v, int *wsum, int *total)
 {
@@ -797,19 +1400,6 @@ __device__ __forceinline__ int block_excl_scan(int v, int *wsum, int *total)
     int r = x - v + (warp ? wsum[warp - 1] : 0);
     *total = wsum[K3_THREADS / 32 - 1];
     return r;  // wsum is written again only after the caller's next barrier
-}
-
-// slot of determinant (a, b) in the trial-estimator table, or -1
-__device__ __forceinline__ int trial_find(const DevInst &I, u64 a, u64 b)
-{
-    const u64 mask = (1ULL << I.trial_bits) - 1;
-    u64 s = det_hash(a, b) & mask;
-    for (u64 probe = 0; probe <= mask; probe++) {
-        if (__ldg(I.trial_state + s) == 0u) return -1;
-        if (__ldg(&I.trial_tab[s].a) == a && __ldg(&I.trial_tab[s].b) == b) return (int)s;
-        s = (s + 1) & mask;
-    }
-    return -1;
 }
 
 // Death, annihilation and the reductions of one bucket b (steps (b) and (c)
@@ -1125,18 +1715,15 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
         __syncthreads();
         for (int q = t; q < KIDX; q += K3_THREADS) I.kidx[np][(size_t)b * KIDX + q] = (unsigned short)W.tab[q];
     }
-    // 7. new determinants: their slots go to the run's list; H_jj - E_ref is
-    //    computed for all of them at once by k_new_diag, whose warps are not
-    //    held back by this block's barriers
-    if (!overflow) {  // each warp reserves the entries it writes (q = 32 warp + lane + K3_THREADS k)
+    // 7. H_jj - E_ref of the new determinants, a warp each
+    if (!overflow) {
         const int nnew = S.n_new;
-        int cntw = 0;
-        for (int q0 = warp * 32; q0 < nnew; q0 += K3_THREADS) cntw += min(32, nnew - q0);
-        int nb0 = 0;
-        if (lane == 0 && cntw > 0) nb0 = atomicAdd(&I.st->new_n, cntw);
-        nb0 = __shfl_sync(0xffffffffu, nb0, 0);
-        for (int q = t, k = 0; q < nnew; q += K3_THREADS, k++)
-            I.newdet[nb0 + 32 * k + lane] = (unsigned)(base + W.opos[W.nacc[q]]);
+        for (int q = warp; q < nnew; q += K3_THREADS / 32) {
+            const int e = W.nacc[q];
+            const ulonglong2 k = W.key[e];
+            const double hdv = diag_exact_warp(I, k.x, k.y);
+            if (lane == 0) nhd[base + W.opos[e]] = hdv;
+        }
     }
     // 8. bucket reductions (fixed order: lanes by xor tree, warps in index order)
     if (I.trial_bits)  // binary64 adds are slow on this part: only when the estimator is on
@@ -1198,680 +1785,11 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
     // again only after the next bucket's barriers
 }
 
-// The same steps for a run without replica side lists or adaptive shift, in
-// three block phases per bucket: (A) walkers inserted into the table, death
-// and Eq. (3); (B) every spawn finds its target or becomes the owner of a new
-// determinant, initiator rule, exact accumulation; (C) owners finalised
-// (Eq. (3) with the annihilation draw), each kept one written straight to the
-// new bucket at a position taken from a shared counter (the order inside a
-// bucket affects no result), the new determinants listed, the bucket's totals
-// reduced, and the table cleared for the next bucket.  Writes beyond the
-// bucket's capacity are skipped: the overflow flag makes the host repeat the
-// iteration after growth.
-//
-// Where the records come from is a policy: LoadStage reads them from global
-// memory in phase A into the block's shared arrays; BulkStage finds them
-// already in shared memory, placed there by bulk copies issued while the
-// previous bucket was processed.
-struct Work3 {       // per-record working arrays shared by both policies
-    u64 *acc_lo, *acc_hi;
-    int *eflag;
-    unsigned short *tab;
-};
-
-struct LoadStage {
-    ulonglong2 *key;  // [EMAX]: walkers, then spawns
-    double *val;      // [EMAX]: C' after death (walkers), w (spawns)
-    int m, si, sn, cap_s;
-    size_t base, sbase;
-    const DevInst *I;
-    int par;
-    __device__ void walker(int e, ulonglong2 &k, double &c, double &hd, uint8_t &f) const
-    {
-        k = I->key[par][base + e];
-        c = I->c[par][base + e];
-        hd = I->hd[par][base + e];
-        f = I->fl[par][base + e];
-    }
-    __device__ void put_walker(int e, ulonglong2 k) const { key[e] = k; }
-    __device__ void stage_spawns(int t) const  // spawns: initiator [m, m+si), the others [m+si, E)
-    {
-        for (int e = m + t; e < m + si + sn; e += K3_THREADS) {
-            const int q = e - m;
-            const size_t o = sbase + (q < si ? q : cap_s - 1 - (q - si));
-            key[e] = I->skey[o];
-            val[e] = I->sw[o];
-        }
-    }
-    __device__ ulonglong2 k(int e) const { return key[e]; }
-    __device__ double v(int e) const { return val[e]; }
-    __device__ void set_v(int e, double x) const { val[e] = x; }
-    __device__ double hd_out(int e) const { return I->hd[par][base + e]; }  // read again: an L2 hit
-};
-
-// one bucket's raw records in shared memory, filled by bulk copies
-template <int SCAP>
-struct AStage {
-    ulonglong2 wkey[CAP_M];
-    ulonglong2 skey[SCAP];      // initiator spawns [0, si), the others [si, si + sn)
-    double wc[CAP_M];           // C; after death C'
-    double whd[CAP_M];
-    double sw[SCAP + 2];        // initiator weights [0, si), the others from swo (16-byte aligned copies)
-    uint8_t wfl[CAP_M];
-};
-
-template <int SCAP>
-struct BulkStage {
-    AStage<SCAP> *st;
-    int m, si, swo;
-    __device__ void walker(int e, ulonglong2 &k, double &c, double &hd, uint8_t &f) const
-    {
-        k = st->wkey[e];
-        c = st->wc[e];
-        hd = st->whd[e];
-        f = st->wfl[e];
-    }
-    __device__ void put_walker(int, ulonglong2) const {}
-    __device__ void stage_spawns(int) const {}
-    __device__ ulonglong2 k(int e) const { return e < m ? st->wkey[e] : st->skey[e - m]; }
-    __device__ double v(int e) const
-    {
-        if (e < m) return st->wc[e];
-        const int q = e - m;
-        return q < si ? st->sw[q] : st->sw[swo + (q - si)];
-    }
-    __device__ void set_v(int e, double x) const { st->wc[e] = x; }  // walkers only
-    __device__ double hd_out(int e) const { return st->whd[e]; }
-};
-
-// A thread's share of a run's exact integer totals over the buckets its
-// block meets in one annihilation launch (integer sums: any order gives the
-// same total), added to the run's accumulators once, when the block leaves
-// the run
-struct AnniTotals {
-    u128 nw = 0;            // N_w * 2^32
-    i128 ann = 0;           // annihilated walkers * 2^32
-    i128 enm = 0;           // E_num * 2^Fe (terms truncated to the grid)
-    long long rej = 0;      // rejected non-initiator spawns
-    long long ndet = 0;     // determinants kept (thread 0)
-    long long spawns = 0;   // spawns received (thread 0)
-};
-
-// every thread of the block: the totals into the run's accumulators (line
-// blockIdx.x % NSHARD), then zero
-__device__ void anni_flush(const DevInst &I, AnniTotals &T)
-{
-    const int lane = threadIdx.x & 31;
-    for (int mm = 16; mm >= 1; mm >>= 1) {
-        T.rej += __shfl_xor_sync(0xffffffffu, T.rej, mm);
-        T.ann += shfl_xor_i128(T.ann, mm);
-        T.nw += (u128)shfl_xor_i128((i128)T.nw, mm);
-        T.enm += shfl_xor_i128(T.enm, mm);
-    }
-    u64 *acc = I.acc + (blockIdx.x % NSHARD) * ACC_STRIDE;
-    if (lane == 0) {
-        limb_add(acc + ACC_NW, (i128)T.nw);
-        limb_add(acc + ACC_ANN, T.ann);
-        limb_add(acc + ACC_ENUM, T.enm);
-        if (T.rej) red_add(&acc[ACC_REJ], (u64)T.rej);
-    }
-    if (threadIdx.x == 0) {
-        if (T.ndet) red_add(&acc[ACC_NDET], (u64)T.ndet);
-        if (T.spawns) red_add(&acc[ACC_SPAWNS], (u64)T.spawns);
-    }
-    T = AnniTotals{};
-}
-
-template <typename SRC>
-__device__ void anni_bucket_3p(const DevInst &I, K3Shared &S, const Work3 &W, const SRC &R, int b, int par,
-                               long long it, double shift, int m, int si, int sn, AnniTotals &T)
-{
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int E = m + si + sn;
-    constexpr u64 tmask = (u64)((1 << TABBITS) - 1);
-    const size_t base = (size_t)b * CAP_M;
-    const unsigned below = (1u << lane) - 1u;
-
-    // A. walkers, two per thread at a time: loads issued first, then
-    //    insertion and death (b) with Eq. (3)
-    static_assert(CAP_M <= 4 * K3_THREADS, "walkers per thread");
-#pragma unroll
-    for (int r0 = 0; r0 < 4; r0 += 2) {
-        ulonglong2 k[2];
-        double c[2], hd[2];
-        int f[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int e = t + (r0 + h) * K3_THREADS;
-            k[h] = make_ulonglong2(0, 0);
-            c[h] = 0.0;
-            hd[h] = 0.0;
-            f[h] = 0;
-            if (e < m) {
-                uint8_t fl;
-                R.walker(e, k[h], c[h], hd[h], fl);
-                f[h] = EF_OWNER | ((fl & DFLAG_REF) ? EF_REF : 0) | ((fl & DFLAG_D) ? EF_D : 0);
-            }
-        }
-        double cp[2];
-        bool draw[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int e = t + (r0 + h) * K3_THREADS;
-            draw[h] = false;
-            cp[h] = 0.0;
-            if (e < m) {
-                R.put_walker(e, k[h]);
-                W.acc_lo[e] = 0;
-                W.acc_hi[e] = 0;
-                W.eflag[e] = f[h] | (!is_zero(c[h]) ? EF_OCC : 0);
-                u64 sl = det_hash(k[h].x, k[h].y) & tmask;
-                while (atomicCAS(&W.tab[sl], (unsigned short)0, (unsigned short)(e + 1)) != 0) sl = (sl + 1) & tmask;
-                if (f[h] & EF_D) cp[h] = I.dc_new[d_index_of(I, k[h].x, k[h].y)];
-                else {
-                    cp[h] = c[h] * (1.0 - I.tau * (hd[h] - shift));
-                    draw[h] = !is_zero(cp[h]) && abs_lt(cp[h], I.cmin);
-                }
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int e = t + (r0 + h) * K3_THREADS;
-            if (draw[h]) {
-                u64 w[4];
-                philox(k[h].x, k[h].y, (u64)it, (u64)PURPOSE_DEATH, I.seed, I.replica, w);
-                cp[h] = round_stoch(cp[h], I.cmin, I.cmin_log2, I.cmin_pow2, w[0]);
-            }
-            if (e < m) R.set_v(e, cp[h]);
-        }
-    }
-    R.stage_spawns(t);
-    for (int e = m + t; e < E; e += K3_THREADS) {
-        W.acc_lo[e] = 0;
-        W.acc_hi[e] = 0;
-        W.eflag[e] = 0;
-    }
-    __syncthreads();
-
-    // B. spawns: find the target or become the owner of a new determinant;
-    //    initiator rule (Sec. I): a non-initiator spawn survives only onto a
-    //    determinant occupied at the start of the iteration
-    long long rejected = 0;
-    i128 ann = 0;
-    for (int e = m + t; e < E; e += K3_THREADS) {
-        const ulonglong2 k = R.k(e);
-        u64 sl = det_hash(k.x, k.y) & tmask;
-        int target = -1;
-        while (true) {
-            unsigned short v = ((volatile unsigned short *)W.tab)[sl];
-            if (v == 0) {
-                const unsigned short old = atomicCAS(&W.tab[sl], (unsigned short)0, (unsigned short)(e + 1));
-                if (old == 0) { target = e; break; }
-                v = old;
-            }
-            const int tt = (int)v - 1;
-            const ulonglong2 kk = R.k(tt);
-            if (kk.x == k.x && kk.y == k.y) { target = tt; break; }
-            sl = (sl + 1) & tmask;
-        }
-        if (target == e) atomicOr(&W.eflag[e], EF_OWNER);  // EF_ACC may be arriving from another spawn
-        const bool accepted = (e < m + si) || (target < m && (W.eflag[target] & EF_OCC));
-        if (!accepted) { rejected++; continue; }
-        const double w = R.v(e);
-        const i128 x = to_fixed(w, I.Fw);
-        const u64 lo = (u64)x, hi = (u64)((u128)x >> 64);
-        const u64 old = atomicAdd((unsigned long long *)&W.acc_lo[target], (unsigned long long)lo);
-        atomicAdd((unsigned long long *)&W.acc_hi[target], (unsigned long long)(hi + (old + lo < old ? 1ULL : 0ULL)));
-        atomicOr(&W.eflag[target], EF_ACC);
-        ann += (i128)fx32(w);
-    }
-    __syncthreads();
-
-    // C. owners: sum = C' + exact spawn sum, Eq. (3) with the annihilation
-    //    draw; kept determinants written to the new bucket
-    const int np = par ^ 1;
-    ulonglong2 *nkey = I.key[np];
-    double *nc = I.c[np], *nhd = I.hd[np];
-    uint8_t *nfl = I.fl[np];
-    u128 nw = 0;
-    double tnum = 0.0, tden = 0.0;
-    bool bad = false;
-    for (int e0 = 0; e0 < E; e0 += K3_THREADS) {
-        const int e = e0 + t;
-        int f = 0;
-        double accv = 0.0;
-        bool keep = false;
-        if (e < E) {
-            f = W.eflag[e];
-            if (f & EF_OWNER) {
-                const bool present = e < m;
-                const double cp = present ? R.v(e) : 0.0;
-                accv = cp;
-                if (f & EF_ACC) {
-                    const double sw = fixed_to_double((i128)(((u128)W.acc_hi[e] << 64) | (u128)W.acc_lo[e]), I.Fw);
-                    accv = present ? cp + sw : sw;
-                    ann += (present ? (i128)fx32(cp) : (i128)0) - (i128)fx32(accv);
-                    if (!(f & EF_D) && !is_zero(accv) && abs_lt(accv, I.cmin)) {
-                        const ulonglong2 k = R.k(e);
-                        u64 w[4];
-                        philox(k.x, k.y, (u64)it, (u64)PURPOSE_ANNIH, I.seed, I.replica, w);
-                        accv = round_stoch(accv, I.cmin, I.cmin_log2, I.cmin_pow2, w[0]);
-                    }
-                }
-                keep = !is_zero(accv) || (f & (EF_REF | EF_D));
-            }
-        }
-        // positions in the new bucket from a shared counter, one atomic per warp
-        const unsigned mk = __ballot_sync(0xffffffffu, keep);
-        int pb = 0;
-        if (lane == 0 && mk) pb = atomicAdd(&S.n_new, __popc(mk));
-        pb = __shfl_sync(0xffffffffu, pb, 0);
-        const int pos = pb + __popc(mk & below);
-        const bool write = keep && pos < CAP_M;
-        // the slots of new determinants go to the run's list (H_jj by k_new_diag)
-        const unsigned mn = __ballot_sync(0xffffffffu, write && e >= m);
-        int qb = 0;
-        if (lane == 0 && mn) qb = atomicAdd(&I.st->new_n, __popc(mn));
-        qb = __shfl_sync(0xffffffffu, qb, 0);
-        if (write) {
-            const ulonglong2 k = R.k(e);
-            const size_t dst = base + pos;
-            nkey[dst] = k;
-            nc[dst] = accv;
-            nfl[dst] = (uint8_t)(((f & EF_REF) ? DFLAG_REF : 0) | ((f & EF_D) ? DFLAG_D : 0));
-            if (e < m) nhd[dst] = R.hd_out(e);
-            else I.newdet[qb + __popc(mn & below)] = (unsigned)dst;
-            if (!abs_lt(accv, 0x1p31)) bad = true;
-            else nw += fx32(accv);
-            if (f & EF_REF) I.st->e_den = accv;
-            else {
-                const int lev = __popcll(k.x ^ I.ref_a) + __popcll(k.y ^ I.ref_b);
-                if (lev <= 4 && !is_zero(accv))  // E_num term on the grid 2^-Fe (R12)
-                    T.enm += to_fixed(hoff_generic(I, k.x, k.y, I.ref_a, I.ref_b) * accv, I.Fe);
-            }
-            if (f & EF_D) I.dc_buf[np][d_index_of(I, k.x, k.y)] = accv;
-            if (I.trial_bits && !is_zero(accv)) {  // trial-wave-function estimator (Sec. IV)
-                const int ts = trial_find(I, k.x, k.y);
-                if (ts >= 0) {
-                    tnum = tnum + __ldg(&I.trial_tab[ts].w) * accv;
-                    tden = tden + __ldg(&I.trial_tab[ts].cT) * accv;
-                }
-            }
-        }
-    }
-    // the table is read no more in this bucket: clear it for the next one
-    {
-        uint4 *tz = reinterpret_cast<uint4 *>(W.tab);
-        for (int q = t; q < (int)((sizeof(unsigned short) << TABBITS) / sizeof(uint4)); q += K3_THREADS)
-            tz[q] = make_uint4(0, 0, 0, 0);
-    }
-    if (bad) atomicOr(&I.st->err, ERRB_NUMERIC);
-    // bucket reductions (fixed order: lanes by xor tree, warps in index order)
-    // the integer totals (E_num's truncated terms among them) stay in the
-    // thread and are added to the run's accumulators when the block leaves
-    // the run; the trial sums are binary64, summed per bucket in a fixed order
-    // (lanes by xor tree, warps in index order)
-    T.rej += rejected;
-    T.ann += ann;
-    T.nw += nw;
-    if (I.trial_bits)
-        for (int mm = 16; mm >= 1; mm >>= 1) {
-            tnum = tnum + __shfl_xor_sync(0xffffffffu, tnum, mm);
-            tden = tden + __shfl_xor_sync(0xffffffffu, tden, mm);
-        }
-    if (lane == 0) {
-        S.red_t[warp][0] = tnum;
-        S.red_t[warp][1] = tden;
-    }
-    __syncthreads();
-    if (t == 0) {
-        const int total = S.n_new;
-        S.n_new = 0;  // next used after two more barriers
-        double tn = 0.0, td = 0.0;
-        if (I.trial_bits)
-            for (int k = 0; k < K3_THREADS / 32; k++) {
-                tn = tn + S.red_t[k][0];
-                td = td + S.red_t[k][1];
-            }
-        if (total > CAP_M) { atomicOr(&I.st->err, ERRB_MAIN_CAP); atomicMax(&I.st->need_main, total); }
-        T.ndet += total;
-        T.spawns += si + sn;
-        if (I.trial_bits) {
-            Partial &P = I.part[b];
-            P.t_num = tn;
-            P.t_den = td;
-        }
-        if (total <= CAP_M) I.cnt[np][b] = total;
-        I.scnt_i[b] = 0;
-        I.scnt_n[b] = 0;
-    }
-}
-
-// ------------------------------------------------------------------ staged annihilation
-// Bulk copies (cp.async.bulk, global -> this CTA's shared memory; source in
-// this GPU's own memory, no multicast), completion counted in bytes on an
-// mbarrier.  Addresses and sizes are multiples of 16 bytes.
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(u64 *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(u64 *bar, unsigned bytes)
-{
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_addr(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, u64 *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
-// one bounded probe of the barrier's phase (the hardware may suspend the thread a while)
-__device__ __forceinline__ bool mbar_test(u64 *bar, unsigned parity)
-{
-    unsigned ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok)
-                 : "r"(smem_addr(bar)), "r"(parity)
-                 : "memory");
-    return ok != 0;
-}
-constexpr long long MBAR_POLLS = 1LL << 24;  // bound on the polls of one wait
-__device__ __forceinline__ bool mbar_wait(u64 *bar, unsigned parity)
-{
-    for (long long k = 0; k < MBAR_POLLS; k++)
-        if (mbar_test(bar, parity)) return true;
-    return false;
-}
-
-template <int SCAP>
-struct K4Smem {
-    K3Shared sh;
-    u64 bar[2];
-    int binfo[2][8];  // per stage: bucket (-1: nothing staged), m, si, sn, swo, run, parity, error
-    long long bit[2];
-    double bS[2];
-    AStage<SCAP> st[2];
-    u64 acc_lo[CAP_M + SCAP], acc_hi[CAP_M + SCAP];
-    int eflag[CAP_M + SCAP];
-    unsigned short tab[1 << TABBITS];
-};
-static_assert(2 * (sizeof(K4Smem<STAGED_SCAP>) + 1024) <= 233472, "two staged annihilation blocks per SM");
-
-// What thread 0 knows of a unit before its copies go out: the run's state
-// (read once per run the block meets) and the bucket's counts, loaded one
-// bucket ahead of their use so that their latency is hidden
-struct StageMeta {
-    int u, ii, b, m, si, sn, par, err;
-    long long it;
-    double S;
-};
-
-__device__ __forceinline__ void meta_load(const DevInst *__restrict__ insts, const int *__restrict__ unit_start,
-                                          int n_inst, int u, StageMeta &M)
-{
-    M.u = u;
-    if (u < 0) return;
-    const int ii = find_inst(unit_start, n_inst, u);
-    const DevInst &I = insts[ii];
-    if (ii != M.ii) {
-        M.ii = ii;
-        M.err = *(volatile int *)&I.st->err;
-        M.par = I.st->parity;
-        M.it = I.st->iter;
-        M.S = I.st->S;
-    }
-    M.b = u - I.unit0;
-    M.m = I.cnt[M.par][M.b];
-    M.si = I.scnt_i[M.b];
-    M.sn = I.scnt_n[M.b];
-}
-
-// thread 0: the checks of k_annihilate on unit M.u, then the bulk copies of
-// its bucket into stage q (completion on bar[q]); the stage's info tells the
-// block whether and what to process
-template <int SCAP>
-__device__ void stage_issue(const DevInst *__restrict__ insts, const StageMeta &M, K4Smem<SCAP> &Sm, int q)
-{
-    int *bi = Sm.binfo[q];
-    bi[0] = -1;
-    if (M.u < 0 || M.err) return;
-    const DevInst &I = insts[M.ii];
-    const int par = M.par, b = M.b, m = M.m, si = M.si, sn = M.sn, cap_s = I.cap_s;
-    if (si + sn > cap_s) {
-        atomicOr(&I.st->err, ERRB_SPAWN_CAP);
-        atomicMax(&I.st->need_spawn, si + sn);
-        atomicAdd(&I.st->n_spawn_over, 1);
-        return;
-    }
-    if (m + si + sn > EMAX) {  // too large for shared memory: deferred to k_annihilate_big
-        I.big_list[atomicAdd(&I.st->big_n, 1)] = b;
-        return;
-    }
-    if (si + sn > SCAP) {
-        // more spawns than the stage holds, but within the working arrays: the
-        // block loads this bucket itself (no copies; the phase completes at once)
-        bi[1] = m; bi[2] = si; bi[3] = sn; bi[4] = 0; bi[5] = M.ii; bi[6] = par; bi[7] = 1;
-        Sm.bit[q] = M.it;
-        Sm.bS[q] = M.S;
-        bi[0] = b;
-        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(&Sm.bar[q]))
-                     : "memory");
-        return;
-    }
-    AStage<SCAP> &st = Sm.st[q];
-    const size_t base = (size_t)b * CAP_M, sbase = (size_t)b * cap_s;
-    // 16-byte multiples: C and H_ii rounded up to an even count, flags to 16
-    // (all within the bucket's CAP_M slots); the non-initiator weights start
-    // at an even slot (one slot early when cap_s - sn is odd)
-    const unsigned m2 = (unsigned)((m + 1) & ~1), m16 = (unsigned)((m + 15) & ~15);
-    const unsigned si2 = (unsigned)((si + 1) & ~1);
-    const int n0 = cap_s - sn, n0e = n0 & ~1;
-    const unsigned nw_cnt = (unsigned)(cap_s - n0e);
-    const unsigned bytes = (m ? (unsigned)m * 16u + m2 * 8u * 2u + m16 : 0u) + (unsigned)(si + sn) * 16u +
-                           (si ? si2 * 8u : 0u) + (sn ? nw_cnt * 8u : 0u);
-    bi[1] = m; bi[2] = si; bi[3] = sn; bi[4] = (int)si2 + (n0 - n0e); bi[5] = M.ii; bi[6] = par; bi[7] = 0;
-    Sm.bit[q] = M.it;
-    Sm.bS[q] = M.S;
-    bi[0] = b;
-    if (bytes == 0) {  // an empty bucket: complete the phase without copies
-        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(&Sm.bar[q]))
-                     : "memory");
-        return;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier generic accesses of the stage first
-    mbar_expect_tx(&Sm.bar[q], bytes);
-    if (m) {
-        bulk_g2s(st.wkey, I.key[par] + base, (unsigned)m * 16u, &Sm.bar[q]);
-        bulk_g2s(st.wc, I.c[par] + base, m2 * 8u, &Sm.bar[q]);
-        bulk_g2s(st.whd, I.hd[par] + base, m2 * 8u, &Sm.bar[q]);
-        bulk_g2s(st.wfl, I.fl[par] + base, m16, &Sm.bar[q]);
-    }
-    if (si) {
-        bulk_g2s(st.skey, I.skey + sbase, (unsigned)si * 16u, &Sm.bar[q]);
-        bulk_g2s(st.sw, I.sw + sbase, si2 * 8u, &Sm.bar[q]);
-    }
-    if (sn) {
-        bulk_g2s(st.skey + si, I.skey + sbase + n0, (unsigned)sn * 16u, &Sm.bar[q]);
-        bulk_g2s(st.sw + si2, I.sw + sbase + n0e, nw_cnt * 8u, &Sm.bar[q]);
-    }
-}
-
-// The three-phase annihilation with every bucket's records brought into
-// shared memory by bulk copies one bucket ahead: while a block works on one
-// bucket, the next one's keys, amplitudes, H_ii, flags and spawns are in
-// flight.  For runs without replica side lists or adaptive shift whose spawn
-// capacity fits the stage (the host picks this kernel then).
-__global__ void __launch_bounds__(K3_THREADS, 2) k_annihilate_staged(const DevInst *__restrict__ insts,
-                                                                     const int *__restrict__ unit_start, int n_inst,
-                                                                     int n_units)
-{
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    K4Smem<STAGED_SCAP> &Sm = *reinterpret_cast<K4Smem<STAGED_SCAP> *>(smem_raw);
-    K3Shared &S = Sm.sh;
-    const int t = threadIdx.x;
-    {
-        uint4 *tz = reinterpret_cast<uint4 *>(Sm.tab);
-        for (int q = t; q < (int)(sizeof(Sm.tab) / sizeof(uint4)); q += K3_THREADS) tz[q] = make_uint4(0, 0, 0, 0);
-    }
-    // the last thread (the least loaded in the phases of a bucket) issues the
-    // copies and keeps the counts of the bucket whose copies go out next
-    constexpr int ISSUER = K3_THREADS - 1;
-    StageMeta nxt;
-    nxt.ii = -1;
-    if (t == ISSUER) {
-        S.n_new = 0;
-        mbar_init(&Sm.bar[0], 1);
-        mbar_init(&Sm.bar[1], 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        StageMeta first;
-        first.ii = -1;
-        meta_load(insts, unit_start, n_inst, (int)blockIdx.x < n_units ? (int)blockIdx.x : -1, first);
-        stage_issue(insts, first, Sm, 0);
-        nxt.ii = first.ii;
-        nxt.err = first.err; nxt.par = first.par; nxt.it = first.it; nxt.S = first.S;
-        const int un = (int)blockIdx.x + (int)gridDim.x;
-        meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-    }
-    __syncthreads();
-    unsigned phase[2] = {0u, 0u};
-    const Work3 W3{Sm.acc_lo, Sm.acc_hi, Sm.eflag, Sm.tab};
-    AnniTotals T;
-    int q = 0, cur = -1;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x, q ^= 1) {
-        // the next bucket's copies go out while this one is processed; its
-        // stage was last read before the previous bucket's closing barrier
-        auto issue_next = [&]() {
-            stage_issue(insts, nxt, Sm, q ^ 1);
-            const int un = u + 2 * (int)gridDim.x;
-            meta_load(insts, unit_start, n_inst, un < n_units ? un : -1, nxt);
-        };
-        const int b = Sm.binfo[q][0];
-        if (b < 0) {
-            if (t == ISSUER) issue_next();
-            __syncthreads();  // binfo[q ^ 1] is written before anyone reads it
-            continue;
-        }
-        const bool ok = mbar_wait(&Sm.bar[q], phase[q]);
-        const int ii = Sm.binfo[q][5];
-        const DevInst &I = insts[ii];
-        if (__syncthreads_or(!ok)) {
-            // the copies did not land within the bound: report, wait once
-            // more (bounded) for them, stop (stage q ^ 1 holds none: its
-            // last copies were waited for one bucket ago)
-            if (t == 0) atomicOr(&I.st->err, ERRB_TIMEOUT);
-            mbar_wait(&Sm.bar[q], phase[q]);
-            return;
-        }
-        if (t == ISSUER) issue_next();
-        phase[q] ^= 1u;
-        if (ii != cur) {  // a new run: the previous run's totals are complete
-            if (cur >= 0) anni_flush(insts[cur], T);
-            cur = ii;
-        }
-        const int m = Sm.binfo[q][1], si = Sm.binfo[q][2], sn = Sm.binfo[q][3], swo = Sm.binfo[q][4];
-        const int par = Sm.binfo[q][6];
-        if (Sm.binfo[q][7]) {
-            // loaded by the block: the stage's contiguous key arrays (walkers,
-            // then spawns: CAP_M + SCAP = EMAX entries) and amplitude arrays
-            // (2 CAP_M >= EMAX) serve as the records of LoadStage
-            static_assert(CAP_M + STAGED_SCAP >= EMAX && 2 * CAP_M >= EMAX, "stage arrays hold EMAX records");
-            static_assert(offsetof(AStage<STAGED_SCAP>, skey) == offsetof(AStage<STAGED_SCAP>, wkey) +
-                                                                     sizeof(ulonglong2) * CAP_M &&
-                              offsetof(AStage<STAGED_SCAP>, whd) == offsetof(AStage<STAGED_SCAP>, wc) +
-                                                                    sizeof(double) * CAP_M,
-                          "walker and spawn key arrays, and amplitude and H_ii arrays, adjacent");
-            AStage<STAGED_SCAP> &st = Sm.st[q];
-            const LoadStage R{st.wkey, st.wc, m, si, sn, I.cap_s, (size_t)b * CAP_M, (size_t)b * I.cap_s, &I, par};
-            anni_bucket_3p(I, S, W3, R, b, par, Sm.bit[q], Sm.bS[q], m, si, sn, T);
-            continue;
-        }
-        const BulkStage<STAGED_SCAP> R{&Sm.st[q], m, si, swo};
-        anni_bucket_3p(I, S, W3, R, b, par, Sm.bit[q], Sm.bS[q], m, si, sn, T);
-    }
-    if (cur >= 0) anni_flush(insts[cur], T);
-}
-
-// GENERAL: the batch holds a run with replica side lists or adaptive shift,
-// whose buckets take the general path (anni_bucket); the others the
-// three-phase one.  Without it the kernel holds the three-phase path alone.
-template <bool GENERAL>
-__global__ void __launch_bounds__(K3_THREADS, 3) k_annihilate(const DevInst *__restrict__ insts,
-                                                              const int *__restrict__ unit_start, int n_inst, int n_units)
+__global__ void __launch_bounds__(K3_THREADS) k_annihilate_big(const DevInst *__restrict__ insts, int n_inst)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     K3Smem &Sm = *reinterpret_cast<K3Smem *>(smem_raw);
     K3Shared &S = Sm.sh;
-    Stage<unsigned short> W{Sm.key, Sm.val, Sm.acc_lo, Sm.acc_hi, Sm.nacc, Sm.eflag, Sm.tab, Sm.opos};
-    const int t = threadIdx.x;
-    // the three-phase path expects a cleared table and output counter; the
-    // general path (replica side lists, adaptive shift) leaves both used
-    bool clean = false;
-    // the run's state at the start of the iteration, read once per run a
-    // block meets
-    int cur = -1, err = 0, par = 0;
-    long long it = 0;
-    double shift = 0.0;
-    AnniTotals T;
-    for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
-        const int ii = find_inst(unit_start, n_inst, u);
-        const DevInst &I = insts[ii];
-        if (ii != cur) {
-            if (cur >= 0) anni_flush(insts[cur], T);  // the previous run's totals are complete
-            if (t == 0) {
-                S.hdr_err = *(volatile int *)&I.st->err;
-                S.hdr_par = I.st->parity;
-                S.hdr_it = I.st->iter;
-                S.hdr_S = I.st->S;
-            }
-            __syncthreads();
-            err = S.hdr_err;
-            par = S.hdr_par;
-            it = S.hdr_it;
-            shift = S.hdr_S;
-            cur = ii;
-            __syncthreads();
-        }
-        if (err) continue;
-        const int b = u - I.unit0;
-        const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
-        if (si + sn > I.cap_s) {
-            if (t == 0) {
-                atomicOr(&I.st->err, ERRB_SPAWN_CAP);
-                atomicMax(&I.st->need_spawn, si + sn);
-                atomicAdd(&I.st->n_spawn_over, 1);
-            }
-            continue;
-        }
-        if (m + si + sn > EMAX) {  // too large for shared memory: deferred to k_annihilate_big
-            if (t == 0) I.big_list[atomicAdd(&I.st->big_n, 1)] = b;
-            continue;
-        }
-        if (GENERAL && (I.side || I.adaptive)) {
-            anni_bucket<unsigned short>(I, S, W, TABBITS, b, par, it, shift, m, si, sn);
-            clean = false;
-            continue;
-        }
-        if (!clean) {
-            uint4 *tz = reinterpret_cast<uint4 *>(Sm.tab);
-            for (int q = t; q < (int)(sizeof(Sm.tab) / sizeof(uint4)); q += K3_THREADS) tz[q] = make_uint4(0, 0, 0, 0);
-            if (t == 0) S.n_new = 0;
-            __syncthreads();
-            clean = true;
-        }
-        const LoadStage R{Sm.key, Sm.val, m, si, sn, I.cap_s, (size_t)b * CAP_M, (size_t)b * I.cap_s, &I, par};
-        const Work3 W3{Sm.acc_lo, Sm.acc_hi, Sm.eflag, Sm.tab};
-        anni_bucket_3p(I, S, W3, R, b, par, it, shift, m, si, sn, T);
-    }
-    if (cur >= 0) anni_flush(insts[cur], T);
-}
-
-__global__ void __launch_bounds__(K3_THREADS) k_annihilate_big(const DevInst *__restrict__ insts, int n_inst)
-{
-    __shared__ K3Shared S;
     const int t = threadIdx.x;
     for (int ii = 0; ii < n_inst; ii++) {
         const DevInst &I = insts[ii];
@@ -1888,11 +1806,17 @@ __global__ void __launch_bounds__(K3_THREADS) k_annihilate_big(const DevInst *__
         const double shift = S.hdr_S;
         __syncthreads();
         if (err || nbig == 0) continue;
-        if (!I.big_scratch) {  // no scratch yet: report, the host allocates it and repeats the iteration
-            if (t == 0) atomicOr(&I.st->err, ERRB_SPAWN_CAP);
-            continue;
+        const Stage<unsigned short> Ws{Sm.key, Sm.val, Sm.acc_lo, Sm.acc_hi, Sm.nacc, Sm.eflag, Sm.tab, Sm.opos};
+        for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
+            const int b = I.big_list[q];
+            const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
+            if (m + si + sn <= EMAX) {
+                anni_bucket<unsigned short>(I, S, Ws, TABBITS, b, par, it, shift, m, si, sn);
+                __syncthreads();
+            }
         }
-        // this block's scratch slice
+        if (blockIdx.x >= BIG_BLOCKS) continue;
+        // beyond shared memory: this block's slice of the global scratch
         const int Ecap = CAP_M + I.cap_s, tabbits = I.big_tabbits;
         unsigned char *p = I.big_scratch + (size_t)blockIdx.x * I.big_stride;
         Stage<unsigned> W;
@@ -1904,10 +1828,16 @@ __global__ void __launch_bounds__(K3_THREADS) k_annihilate_big(const DevInst *__
         W.eflag = (int *)p; p += (size_t)Ecap * 4;
         W.opos = (unsigned *)p; p += (size_t)Ecap * 4;
         W.tab = (unsigned *)p;
-        for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
+        for (int q = blockIdx.x; q < nbig; q += BIG_BLOCKS) {
             const int b = I.big_list[q];
             const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
+            if (m + si + sn <= EMAX) continue;
+            if (!I.big_scratch) {  // no scratch yet: report, the host allocates it and repeats the iteration
+                if (t == 0) atomicOr(&I.st->err, ERRB_SPAWN_CAP);
+                break;
+            }
             anni_bucket<unsigned>(I, S, W, tabbits, b, par, it, shift, m, si, sn);
+            __syncthreads();
         }
     }
 }
@@ -1918,7 +1848,7 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
     const DevInst &I = insts[blockIdx.x];
     IterState *st = I.st;
     __shared__ int s_err;
-    __shared__ double s_r[K5_THREADS];
+    __shared__ double s_r[6][K5_THREADS / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int nbk = 1 << I.bb;
     const bool pair = I.partner > (int)blockIdx.x;  // the first replica reports the cross estimators
@@ -1947,34 +1877,36 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
     }
     if (e) return;
     // Binary64 sums of the estimators that have them (trial numerator and
-    // denominator; replica-pair terms), per tile of K5_THREADS buckets: one
-    // value per thread into shared memory and a halving tree, so that every
-    // binary64 add is a full-warp instruction (a partly active warp costs as
-    // much on this part's slow binary64 pipe); tile sums added in tile order.
+    // denominator; replica-pair terms): every thread adds its buckets in order,
+    // then a halving tree over the threads
     constexpr int NF = 6;  // words 0 .. 5 of a partial
     double dsum[NF];
 #pragma unroll
     for (int f = 0; f < NF; f++) dsum[f] = 0.0;
-    if (tree)
-        for (int tile0 = 0; tile0 < nbk; tile0 += K5_THREADS) {
+    if (tree) {
+        for (int u = t; u < nbk; u += K5_THREADS) {
+            const double *p = reinterpret_cast<const double *>(I.part + u);
+#pragma unroll
+            for (int f = 0; f < NF; f++)
+                if (f < 2 ? trial : pair) dsum[f] = dsum[f] + p[f];
+        }
+#pragma unroll
+        for (int f = 0; f < NF; f++) {
+            if (f < 2 ? !trial : !pair) continue;
+            double v = dsum[f];
+            for (int mm = 16; mm >= 1; mm >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, mm);
+            if (lane == 0) s_r[f][warp] = v;
+        }
+        __syncthreads();
+        if (warp == 0)
 #pragma unroll
             for (int f = 0; f < NF; f++) {
                 if (f < 2 ? !trial : !pair) continue;
-                const int u = tile0 + t;
-                s_r[t] = u < nbk ? reinterpret_cast<const double *>(I.part + u)[f] : 0.0;
-                __syncthreads();
-                for (int h = K5_THREADS / 2; h >= 32; h >>= 1) {
-                    if (t < h) s_r[t] = s_r[t] + s_r[t + h];
-                    __syncthreads();
-                }
-                if (warp == 0) {
-                    double v = s_r[lane];
-                    for (int mm = 16; mm >= 1; mm >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, mm);
-                    if (lane == 0) dsum[f] = dsum[f] + v;
-                }
-                __syncthreads();
+                double v = lane < K5_THREADS / 32 ? s_r[f][lane] : 0.0;
+                for (int mm = 16; mm >= 1; mm >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, mm);
+                dsum[f] = v;
             }
-        }
+    }
     if (warp != 0) return;
     // the shift state, loaded now so that its latency overlaps the totals'
     const long long it = st->iter, cnt0 = st->cnt, shift_start0 = st->shift_start, stop_iter = st->stop_iter;
@@ -2043,7 +1975,6 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
     st->parity = par0 ^ 1;
     st->heavy_n = 0;
     st->big_n = 0;
-    st->new_n = 0;
     if (I.semi_size > 0 && !semi_built && vary && it + 1 == shift_start + I.semi_start) flags |= ERRB_PAUSE_SEMI;
     if (I.trial_size > 0 && !trial_built && vary && it + 1 == shift_start + I.trial_start) flags |= ERRB_PAUSE_TRIAL;
     if (it + 1 >= stop_iter) flags |= ERRB_STOP;
@@ -2260,71 +2191,51 @@ void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cu
 
 cudaError_t init_kernels()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_annihilate<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(K3Smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_annihilate<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_annihilate_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(K4Smem<STAGED_SCAP>));
-    auto spawn_smem = [&](auto *f, size_t bytes, int blocks) {  // the resident blocks need their shared memory at once
+    cudaError_t e = cudaFuncSetAttribute(k_annihilate_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
+    auto warp_smem = [&](auto *f, size_t bytes, int blocks) {  // the resident blocks need their shared memory at once
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)((blocks * (bytes + 1024) * 100 + 233471) / 233472));
     };
-    spawn_smem(k_spawn<GEN_UNIFORM, false>, SP_SMEM, 4);
-    spawn_smem(k_spawn<GEN_PCHB, false>, SP_SMEM, 4);
-    spawn_smem(k_spawn<GEN_HOP, false>, SP_SMEM, 4);
-    spawn_smem(k_spawn_batch<false>, SP_SMEM, 4);
-    spawn_smem(k_spawn<GEN_UNIFORM, true>, SP_SMEM_ADAPT, 3);
-    spawn_smem(k_spawn<GEN_PCHB, true>, SP_SMEM_ADAPT, 3);
-    spawn_smem(k_spawn<GEN_HOP, true>, SP_SMEM_ADAPT, 3);
-    spawn_smem(k_spawn_batch<true>, SP_SMEM_ADAPT, 3);
-    spawn_smem(k_spawn_heavy, SP_SMEM_ADAPT, 3);
-    spawn_smem(k_spawn_heavy_batch, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_UNIFORM, false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_PCHB, false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_HOP, false>, SP_SMEM, 4);
+    warp_smem(k_spawn_batch<false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_UNIFORM, true>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_PCHB, true>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_HOP, true>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn_batch<true>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn_heavy, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn_heavy_batch, SP_SMEM_ADAPT, 3);
+    warp_smem(k_annihilate<false>, AN_SMEM, 3);
+    warp_smem(k_annihilate_batch<false>, AN_SMEM, 3);
+    warp_smem(k_annihilate<true>, AN_SMEM, 3);
+    warp_smem(k_annihilate_batch<true>, AN_SMEM, 3);
     return e;
 }
 
-size_t annihilate_smem_bytes() { return sizeof(K3Smem); }
-
-// Whether a run's buckets can go through the staged kernel: every array a
-// bulk copy reads on a 16-byte boundary (a caller-supplied allocator may
-// return less aligned memory) and an even spawn capacity; buckets whose
-// spawns exceed the stage are deferred to the large-bucket kernel
-bool staged_annihilation_fits(const DevInst &I)
+// annihilation of one run (`one`) or of a table of runs; extra: some run has
+// replica side lists or the adaptive shift.  g_anni_bps = 0: one resident
+// wave of blocks, else that many blocks per SM
+cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units,
+                              bool extra, cudaStream_t s)
 {
-    auto al = [](const void *p) { return ((uintptr_t)p & 15u) == 0; };
-    if (I.side || I.adaptive || (I.cap_s & 1)) return false;
-    for (int k = 0; k < 2; k++)
-        if (!al(I.key[k]) || !al(I.c[k]) || !al(I.hd[k]) || !al(I.fl[k])) return false;
-    return al(I.skey) && al(I.sw);
-}
-
-// general: some run of the batch has replica side lists or adaptive shift;
-// staged: every run fits the staged kernel (bulk copies one bucket ahead),
-// launched as one resident wave of blocks (two per SM)
-cudaError_t launch_annihilate(const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool general,
-                              bool staged, cudaStream_t s)
-{
-    if (staged && !general && g_anni_bps == 0) {
-        int grid = n_units < num_sms() * 2 ? n_units : num_sms() * 2;
-        if (grid < 1) grid = 1;
-        k_annihilate_staged<<<grid, K3_THREADS, sizeof(K4Smem<STAGED_SCAP>), s>>>(dinst, unit_start, n_inst, n_units);
-        return cudaGetLastError();
-    }
-    const size_t smem = sizeof(K3Smem);
-    const int bps = g_anni_bps > 0 ? g_anni_bps : 9;
-    int grid = n_units < num_sms() * bps ? n_units : num_sms() * bps;
-    if (grid < 1) grid = 1;
-    if (general) k_annihilate<true><<<grid, K3_THREADS, smem, s>>>(dinst, unit_start, n_inst, n_units);
-    else k_annihilate<false><<<grid, K3_THREADS, smem, s>>>(dinst, unit_start, n_inst, n_units);
+    const int bps = g_anni_bps > 0 ? g_anni_bps : 3;
+    const int need = (n_units + AN_WARPS - 1) / AN_WARPS;
+    const int grid = need < num_sms() * bps ? need : num_sms() * bps;
+    if (one && extra) k_annihilate<true><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
+    else if (one) k_annihilate<false><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
+    else if (extra) k_annihilate_batch<true><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
+    else k_annihilate_batch<false><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
     return cudaGetLastError();
 }
 
+// the buckets beyond a warp's records; every block takes those that fit
+// shared memory, the first BIG_BLOCKS the others
 void launch_annihilate_big(const DevInst *dinst, int n_inst, cudaStream_t s)
 {
-    k_annihilate_big<<<BIG_BLOCKS, K3_THREADS, 0, s>>>(dinst, n_inst);
+    k_annihilate_big<<<num_sms() * 3 > BIG_BLOCKS ? num_sms() * 3 : BIG_BLOCKS, K3_THREADS, sizeof(K3Smem), s>>>(dinst, n_inst);
 }
 
 void launch_finalize(const DevInst *dinst, int n_inst, cudaStream_t s)
@@ -2332,110 +2243,34 @@ void launch_finalize(const DevInst *dinst, int n_inst, cudaStream_t s)
     k_finalize<<<n_inst, K5_THREADS, 0, s>>>(dinst, n_inst);
 }
 
-// H_jj - E_ref of the determinants created in this iteration (new list,
-// parity ^ 1), four per warp with eight lanes each.  The terms (h_pp of
-// electron e1, or the pair e1 < e2) are listed once per block in shared
-// memory, and each warp keeps the occupied orbitals of its four determinants
-// there, so a term costs two shared loads and one table load; each lane group
-// sums its terms exactly and reduces over its eight lanes.
-constexpr int ND_PAIRS = 2080;  // n (n + 1) / 2 terms for up to 64 electrons
-
-// H_ii - E_ref of the determinants at the slots list[0 .. nn) of list `np`
-// (whole block; every thread calls it)
-__device__ void diag_list(const DevInst &I, const unsigned *__restrict__ list, int nn, int np,
-                          unsigned short *s_term, unsigned char (*s_orb)[4][64])
+// H_ii - E_ref of every determinant of list `par`, given by its slots (import)
+__global__ void __launch_bounds__(256) k_diag_list(const __grid_constant__ DevInst I, int par, const unsigned *list, int nn)
 {
+    __shared__ unsigned short s_pair[ND_PAIRS];
+    __shared__ unsigned char s_orb[8][4][ND_MAX];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarp = (int)((gridDim.x * blockDim.x) >> 5);
-    const ulonglong2 *nkey = I.key[np];
-    double *nhd = I.hd[np];
-    const int n = I.n, na = I.na, N = I.norb, T = n + n * (n - 1) / 2;
-    if (n > 64) {  // beyond the table: the generic warp sum
+    if (I.n > ND_MAX) {  // beyond the table: the generic warp sum
         for (int q = 2 * gw; q < nn; q += 2 * nwarp) {
             const unsigned d0 = list[q], d1 = q + 1 < nn ? list[q + 1] : d0;
-            const ulonglong2 k0 = nkey[d0], k1 = nkey[d1];
+            const ulonglong2 k0 = I.key[par][d0], k1 = I.key[par][d1];
             const u64 ka[2] = {k0.x, k1.x}, kb[2] = {k0.y, k1.y};
             double hdv[2];
             diag_exact_warp_multi<2>(I, ka, kb, hdv);
             if (lane == 0) {
-                nhd[d0] = hdv[0];
-                if (q + 1 < nn) nhd[d1] = hdv[1];
+                I.hd[par][d0] = hdv[0];
+                if (q + 1 < nn) I.hd[par][d1] = hdv[1];
             }
         }
         return;
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        if (t < n) { s_term[t] = (unsigned short)(t | (255 << 8)); continue; }
-        const int q = t - n;
-        int c = 1;
-        while ((c + 1) * c / 2 <= q) c++;
-        s_term[t] = (unsigned short)((q - c * (c - 1) / 2) | (c << 8));
-    }
-    __syncthreads();
-    // four determinants per warp, eight lanes each: lane group g takes
-    // determinant q + g (a short last round repeats determinant q and
-    // stores nothing for it), its lanes the terms sl, sl + 8, ...
-    const int g = lane >> 3, sl = lane & 7;
-    const i128 xref = (i128)(((u128)I.xref_hi << 64) | (u128)I.xref_lo);
-    for (int q = 4 * gw; q < nn; q += 4 * nwarp) {
-        const unsigned d = list[q + g < nn ? q + g : q];
-        const ulonglong2 key = nkey[d];
-        for (int e = sl; e < n; e += 8)
-            s_orb[wl][g][e] = (unsigned char)(e < na ? nth_set(key.x, e) : nth_set(key.y, e - na));
-        __syncwarp();
-        i128 part = 0;
-        for (int t0 = sl; t0 < T; t0 += 32) {
-            ulonglong2 v[4];
-#pragma unroll
-            for (int r = 0; r < 4; r++) {
-                const int t = t0 + 8 * r;
-                v[r] = make_ulonglong2(0, 0);
-                if (t < T) {
-                    const unsigned tm = s_term[t];
-                    const int e1 = (int)(tm & 0xffu), e2 = (int)(tm >> 8);
-                    const int p1 = s_orb[wl][g][e1];
-                    if (e2 == 255) v[r] = __ldg(I.hfx + p1);
-                    else v[r] = __ldg((((e1 < na) == (e2 < na)) ? I.JKfx : I.Jfx) + p1 * N + s_orb[wl][g][e2]);
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < 4; r++) part += (i128)(((u128)v[r].y << 64) | (u128)v[r].x);
-        }
-        for (int m = 4; m >= 1; m >>= 1) part += shfl_xor_i128(part, m);
-        if (sl == 0 && q + g < nn) nhd[d] = fixed_to_double(part - xref, I.F);
-        __syncwarp();
-    }
+    fill_pairs(s_pair);
+    for (int q = 4 * gw; q < nn; q += 4 * nwarp) diag_four(I, list + q, min(4, nn - q), par, s_pair, s_orb[wl]);
 }
 
-__global__ void __launch_bounds__(256) k_new_diag(const DevInst *__restrict__ insts, int n_inst)
+void launch_diag_list(const DevInst *one, int par, const unsigned *list, int nn, cudaStream_t s)
 {
-    __shared__ unsigned short s_term[ND_PAIRS];   // e1 | e2 << 8, e2 = 255 for h_pp
-    __shared__ unsigned char s_orb[8][4][64];
-    for (int ii = 0; ii < n_inst; ii++) {
-        const DevInst &I = insts[ii];
-        if (*(volatile int *)&I.st->err) continue;
-        diag_list(I, I.newdet, I.st->new_n, I.st->parity ^ 1, s_term, s_orb);
-    }
-}
-
-// H_ii - E_ref of every determinant of list `par`, given by its slots (import)
-__global__ void __launch_bounds__(256) k_diag_list(const DevInst *__restrict__ I, int par, const unsigned *list, int nn)
-{
-    __shared__ unsigned short s_term[ND_PAIRS];
-    __shared__ unsigned char s_orb[8][4][64];
-    diag_list(*I, list, nn, par, s_term, s_orb);
-}
-
-void launch_diag_list(const DevInst *dinst, int par, const unsigned *list, int nn, cudaStream_t s)
-{
-    if (nn > 0) k_diag_list<<<num_sms() * 3, 256, 0, s>>>(dinst, par, list, nn);
-}
-
-void launch_new_diag(const DevInst *dinst, int n_inst, cudaStream_t s)
-{
-    // one resident wave (3 blocks per SM at 80 registers): fewer blocks repeat the term-table set-up
-    k_new_diag<<<num_sms() * 3, 256, 0, s>>>(dinst, n_inst);
+    if (nn > 0) k_diag_list<<<num_sms() * 4, 256, 0, s>>>(*one, par, list, nn);
 }
 
 void launch_rebucket(const DevInst *src, const DevInst *dst, int nb_src, int parity, cudaStream_t s)

@@ -59,6 +59,8 @@ CASES = {
     "orb33_one_beta": (lambda: _abinitio(33, 4, 1, 4), 33, dict(tau=2e-4, c_min=0.3, initiator_threshold=1.0)),
     "orb20_heatbath": (lambda: _abinitio(20, 4, 3, 5), 20, dict(tau=5e-4, generator=1, initiator_threshold=3.0)),
     "orb20_adaptive": (lambda: _abinitio(20, 4, 3, 6), 20, dict(tau=5e-4, adaptive_shift=1, initiator_threshold=3.0)),
+    # no initiator but the reference: the spawns of heavily populated determinants are weighed too
+    "orb20_adaptive_heavy": (lambda: _abinitio(20, 4, 3, 7), 20, dict(tau=5e-4, adaptive_shift=1, initiator_threshold=1e6)),
     "hubbard_8x8": (lambda: dict(workloads.hubbard_2d(8, 8, 4.0)), 64, dict(tau=2e-3)),
 }
 
