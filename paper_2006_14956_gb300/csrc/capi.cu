@@ -129,8 +129,23 @@ static void dev_free(fciqmc_handle *h, void *ptr)
     else cudaFree(ptr);
 }
 
-// determinants per bucket a run starts with when its list is as long as expected
-constexpr double START_M = 140.0;
+// Bucket bits of a list of `dets` determinants: START_M per bucket where the
+// list is as long as expected; a short one gets more, smaller buckets (up to
+// SMALL_BB, down to SMALL_M per bucket), so that its warps take one round of
+// 32 records each instead of three or four, one after the other.  At 2^8, 2^9,
+// 2^10, 2^11, 2^12 a 4x4 lattice at 1e5 walkers takes 54, 54, 49, 51, 54 us an
+// iteration, a batch of 64 lattice runs of 1e4 to 1e6 walkers 1.59, 1.61, 1.65,
+// 1.73, 1.92 ms.
+constexpr double START_M = 140.0, SMALL_M = 24.0;
+constexpr int SMALL_BB = 10;
+constexpr double BUCKET_BYTES = 2.0 * CAP_M * 33 + CAP_S0 * 24.0 + 4.0 * CAP_M + 128;  // of device memory
+static int start_bits(double dets, bool spread)
+{
+    int bb = 0;
+    while ((double)(1LL << bb) * START_M < dets && bb < MAX_BB) bb++;
+    while (spread && bb < SMALL_BB && (double)(1LL << bb) * SMALL_M < dets) bb++;
+    return bb;
+}
 
 static int64_t pair_index(int64_t i, int64_t j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
 
@@ -287,12 +302,16 @@ static int enqueue_iteration(fciqmc_handle *h, cudaEvent_t *ev)
     if (ev) cudaEventRecord(ev[2], h->stream);
     if (h->nd > 0) launch_semistoch(h->dinst, 1, h->nd, h->stream);
     if (ev) cudaEventRecord(ev[3], h->stream);
-    cudaError_t e = launch_annihilate(&h->hi, h->dinst, h->dunit, 1, units, h->hi.side || h->hi.adaptive, h->stream);
-    if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("annihilation launch: ") + cudaGetErrorString(e));
-    launch_annihilate_big(h->dinst, 1, h->stream);
-    if (ev) cudaEventRecord(ev[4], h->stream);
-    if (ev) cudaEventRecord(ev[5], h->stream);
-    launch_finalize(h->dinst, 1, h->stream);
+    const cudaError_t e = launch_annihilate(&h->hi, h->dinst, h->dunit, 1, units, h->hi.side || h->hi.adaptive, h->stream);
+    if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("iteration launch: ") + cudaGetErrorString(e));
+    if (ev) {  // kernel by kernel
+        launch_annihilate_big(h->dinst, 1, h->stream);
+        cudaEventRecord(ev[4], h->stream);
+        cudaEventRecord(ev[5], h->stream);
+        launch_finalize(h->dinst, 1, h->stream);
+    } else {
+        launch_finish(&h->hi, h->stream);
+    }
     if (ev) cudaEventRecord(ev[6], h->stream);
     return FCIQMC_OK;
 }
@@ -433,6 +452,7 @@ static int reset_after_error(fciqmc_handle *h)
     h->hst.err = 0;
     h->hst.heavy_n = 0;
     h->hst.big_n = 0;
+    h->hst.done = 0;
     h->hst.need_spawn = 0;
     h->hst.need_main = 0;
     h->hst.n_spawn_over = 0;
@@ -1012,8 +1032,10 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
         for (int k = 0; k < h->nb; k++) fci *= (double)(N - k) / (double)(k + 1);
         if (P.max_dets <= 0) dets_hint = std::min(dets_hint, std::max(1.0, fci));
     }
-    int bb = 0;
-    while (((double)(1LL << bb)) * START_M < dets_hint && bb < MAX_BB) bb++;
+    // a given max_dets is kept to, and a memory limit that leaves little room
+    int bb = start_bits(dets_hint, P.max_dets <= 0);
+    if (P.max_device_bytes > 0 && 8.0 * (double)(1LL << bb) * BUCKET_BYTES > (double)P.max_device_bytes)
+        bb = start_bits(dets_hint, false);
     I.cap_s = CAP_S0;
     int rc = alloc_layout(h, I, bb);
     if (rc) return bail(rc, "out of device memory (walker buffers)");
@@ -1257,6 +1279,24 @@ int fciqmc_sync(fciqmc_handle *h)
 
 void *fciqmc_stream(fciqmc_handle *h) { return h ? (void *)h->stream : nullptr; }
 
+// Whether the run's buckets should be split before they overflow: the average
+// occupancy passes FILL_M, or determinants and spawns together pass what most
+// warps of the annihilation hold (buckets beyond that go to a block each,
+// several times slower) while there are more determinants than buckets.  The
+// second kind, the only one in a batch, is skipped where the memory limit has
+// no room for it.
+constexpr int FILL_E = 160, FILL_MIN = 1;
+static bool crowded(const fciqmc_handle *h, bool optional)
+{
+    if (h->hst.err || h->hist.empty() || h->bb >= MAX_BB) return false;
+    const fciqmc_iter_stats &r = h->hist.back();
+    const long long nbk = 1LL << h->bb;
+    if (!optional && r.ndet > nbk * FILL_M) return true;
+    if (r.ndet + r.spawns <= nbk * FILL_E || r.ndet < 2 * FILL_MIN * nbk) return false;
+    const long long layout = 2 * nbk * (2LL * CAP_M * 33 + (long long)h->hi.cap_s * 24 + 4LL * CAP_M + 128);
+    return h->p.max_device_bytes <= 0 || (long long)h->bytes + layout + (layout >> 4) < h->p.max_device_bytes;
+}
+
 // Runs iterations until target_iter, in chunks of graph replays; after each
 // chunk reads the device state and reacts to its flags (capacity growth with
 // a bit-identical repeat, semi-stochastic set-up, or a fatal error).
@@ -1308,10 +1348,7 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         }
         rc = pull_history(h, start, h->hst.iter);
         if (rc) return rc;
-        if (!h->hst.err && !h->hist.empty() && h->hist.back().ndet > (1LL << h->bb) * (long long)FILL_M &&
-            h->bb < MAX_BB) {
-            // keep head-room in the main buckets: split once the average
-            // occupancy passes FILL_M
+        if (crowded(h, false)) {
             rc = grow_buckets(h);
             if (rc) return rc;
             rc = reset_after_error(h);
@@ -1847,6 +1884,30 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
                 rc = write_state(h);
             }
         }
+        // crowded buckets are split between chunks; a replica pair keeps one layout
+        for (int i = 0; i < k && !rc; i++) {
+            fciqmc_handle *h = hs[i], *pt = h->partner;
+            if ((h->hst.err & ~ERRB_STOP) || (pt && (h->secondary || (pt->hst.err & ~ERRB_STOP)))) continue;
+            const int stop = h->hst.err;
+            h->hst.err = 0;
+            const bool split = crowded(h, true) || (pt && crowded(pt, true));
+            h->hst.err = stop;
+            if (!split) continue;
+            for (fciqmc_handle *g : {h, pt}) {
+                if (!g || rc) continue;
+                const int keep = g->hst.err;
+                const long long si = g->hst.stop_iter;
+                rc = grow_buckets(g);
+                if (!rc) rc = reset_after_error(g);
+                g->hst.err = keep;
+                g->hst.stop_iter = si;
+                if (!rc) rc = write_state(g);
+                if (!rc) rc = ensure_side(g);
+                if (!rc) rc = upload_inst(g);
+                if (rc) g->step_rc = rc;
+            }
+            changed = true;
+        }
         if (!rc && changed) rc = rebuild();
     }
     // restore the single-run state: no stop flag, own graph
@@ -2169,8 +2230,7 @@ static int64_t estimate_bytes(const Request &r)
     const int N = r.sys.kind == FCIQMC_HUBBARD ? r.sys.lx * r.sys.ly : r.sys.norb;
     const double np = (double)N * (N + 1) / 2, ne = np * (np + 1) / 2;
     double dets = r.p.max_dets > 0 ? (double)r.p.max_dets : std::min(std::max(4096.0, r.p.target_walkers), 8388608.0);
-    int bb = 0;
-    while (((double)(1LL << bb)) * (START_M * 0.64) < dets && bb < MAX_BB) bb++;
+    const int bb = start_bits(dets / 0.64, false);
     const double per_bucket = 2.0 * CAP_M * (16 + 8 + 8 + 1) + 5.0 * CAP_S0 * 24.0 + 2 * 8 + sizeof(Partial) + 3 * 4 +
                               4.0 * CAP_M;
     const double ecap = CAP_M + 4.0 * CAP_S0;

@@ -115,6 +115,7 @@ struct IterState {
     double e_den;
     alignas(128) int heavy_n;
     alignas(128) int big_n; // buckets deferred to the large-bucket kernel
+    int done;               // blocks done with them (k_finish)
 };
 
 struct TrialEnt;
@@ -166,7 +167,7 @@ struct DevInst {
     int *scnt_n;
     int cap_s;              // spawn capacity per bucket
     int big_tabbits;        // hash-table bits of the large-bucket path
-    int *big_list;          // deferred bucket ids (capacity = buckets)
+    int *big_list;          // deferred bucket ids, bit 30: beyond shared memory (capacity = buckets)
     unsigned *newdet;       // main-list slots of an imported list
     unsigned char *big_scratch;  // BIG_BLOCKS slices of big_stride bytes
     size_t big_stride;
@@ -238,6 +239,7 @@ cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const in
 cudaError_t init_kernels();
 void launch_annihilate_big(const DevInst *dinst, int n_inst, cudaStream_t s);
 void launch_finalize(const DevInst *dinst, int n_inst, cudaStream_t s);
+void launch_finish(const DevInst *one, cudaStream_t s);
 void launch_build_kidx(const DevInst *dinst, int parity, int nb, cudaStream_t s);
 cudaError_t launch_replica_cross(const DevInst *dinst, int n_inst, int max_buckets, cudaStream_t s);
 cudaError_t replica_kernel_init();

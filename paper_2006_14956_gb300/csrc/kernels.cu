@@ -709,26 +709,36 @@ __device__ __forceinline__ void heavy_body(const RUNS &runs, int n_inst)
     AdaptQueue *aq = reinterpret_cast<AdaptQueue *>(sp_raw + SP_WARPS * sizeof(SpawnWarp)) + warp;
     if (lane == 0) aq->n = 0;
     __syncwarp();
-    for (int ii = 0; ii < n_inst; ii++) {
-        const DevInst &I = runs.inst(ii);
-        const int nh = I.st->heavy_n;
-        const int err = __shfl_sync(0xffffffffu, *(volatile int *)&I.st->err, 0);  // one value for the whole warp
-        if ((int)blockIdx.x >= nh || err) continue;
-        const SpawnRun R{I.st->iter, I.st->S, I.st->parity, I.adaptive ? aq : nullptr};
-        int nq = 0;
-        for (int q = blockIdx.x; q < nh; q += gridDim.x) {
-            const HeavyChunk h = I.heavy[q];
-            for (unsigned a = 32u * warp; a < h.count; a += SP_THREADS)
-            {
-                attempts32<GEN_ANY>(I, W, nq, R, a + lane < h.count, make_ulonglong2(h.a, h.b), h.k0 + a + lane, h.cper,
-                                    h.flags, h.slot);
-                drain_adaptive(I, R, 32);  // each step below and above queues at most 32 more
-                if (nq >= 32) eval_singles(I, W, nq, R);
-                drain_adaptive(I, R, 32);
-            }
+    // lane l looks at run i0 + l (a look costs an L2 round trip: 64 runs one
+    // after the other took 100 us); only runs with work for this block follow
+    for (int i0 = 0; i0 < n_inst; i0 += 32) {
+        int nh_l = 0;
+        if (i0 + lane < n_inst) {
+            const IterState *st = runs.inst(i0 + lane).st;
+            const int err = *(volatile const int *)&st->err, n = *(volatile const int *)&st->heavy_n;
+            nh_l = err ? 0 : n;
         }
-        if (nq > 0) eval_singles(I, W, nq, R);
-        drain_adaptive(I, R, 1);
+        unsigned todo = __ballot_sync(0xffffffffu, (int)blockIdx.x < nh_l);
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int nh = __shfl_sync(0xffffffffu, nh_l, src);
+            const DevInst &I = runs.inst(i0 + src);
+            const SpawnRun R{I.st->iter, I.st->S, I.st->parity, I.adaptive ? aq : nullptr};
+            int nq = 0;
+            for (int q = blockIdx.x; q < nh; q += gridDim.x) {
+                const HeavyChunk h = I.heavy[q];
+                for (unsigned a = 32u * warp; a < h.count; a += SP_THREADS) {
+                    attempts32<GEN_ANY>(I, W, nq, R, a + lane < h.count, make_ulonglong2(h.a, h.b), h.k0 + a + lane, h.cper,
+                                    h.flags, h.slot);
+                    drain_adaptive(I, R, 32);  // each step below and above queues at most 32 more
+                    if (nq >= 32) eval_singles(I, W, nq, R);
+                    drain_adaptive(I, R, 32);
+                }
+            }
+            if (nq > 0) eval_singles(I, W, nq, R);
+            drain_adaptive(I, R, 1);
+        }
     }
 }
 
@@ -783,6 +793,8 @@ constexpr int AN_THREADS = 256, AN_WARPS = AN_THREADS / 32;
 constexpr int AW_E = 192;          // records per warp (bytes of the table index them: below 255)
 constexpr int AW_TAB = 512;
 constexpr unsigned AW_NONE = 0xffu;
+constexpr int BIG_SCRATCH = 1 << 30;  // big_list: the bucket needs the global scratch (written when it is deferred: a
+                                      // bucket's counts say nothing once another block has annihilated it)
 constexpr int ND_MAX = 64;         // electrons the pair table covers
 constexpr int ND_PAIRS = ND_MAX * (ND_MAX - 1) / 2;
 
@@ -1310,7 +1322,7 @@ __device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
                 atomicAdd(&I.st->n_spawn_over, 1);
             }
         } else if (m + si + sn > AW_E) {  // deferred to k_annihilate_big
-            if (lane == 0) I.big_list[atomicAdd(&I.st->big_n, 1)] = b;
+            if (lane == 0) I.big_list[atomicAdd(&I.st->big_n, 1)] = b | (m + si + sn > EMAX ? BIG_SCRATCH : 0);
         } else {
             anni_bucket_warp<EXTRA>(I, W, b, par, it, shift, m, si, sn, T, nq, ne);
         }
@@ -1785,73 +1797,98 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
     // again only after the next bucket's barriers
 }
 
+// one run's deferred buckets (whole block; every block of the launch calls it)
+__device__ void annihilate_deferred(const DevInst &I, K3Smem &Sm)
+{
+    K3Shared &S = Sm.sh;
+    const int t = threadIdx.x;
+    __syncthreads();
+    if (t == 0) {
+        S.hdr_err = *(volatile int *)&I.st->err;
+        S.hdr_par = I.st->parity;
+        S.hdr_it = I.st->iter;
+        S.hdr_S = I.st->S;
+        S.n_new = I.st->big_n;
+    }
+    __syncthreads();
+    const int err = S.hdr_err, par = S.hdr_par, nbig = S.n_new;
+    const long long it = S.hdr_it;
+    const double shift = S.hdr_S;
+    __syncthreads();
+    if (err || nbig == 0) return;
+    const Stage<unsigned short> Ws{Sm.key, Sm.val, Sm.acc_lo, Sm.acc_hi, Sm.nacc, Sm.eflag, Sm.tab, Sm.opos};
+    for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
+        const int b = I.big_list[q];
+        if (b & BIG_SCRATCH) continue;
+        anni_bucket<unsigned short>(I, S, Ws, TABBITS, b, par, it, shift, I.cnt[par][b], I.scnt_i[b], I.scnt_n[b]);
+        __syncthreads();
+    }
+    if (blockIdx.x >= BIG_BLOCKS) return;
+    // beyond shared memory: this block's slice of the global scratch
+    const int Ecap = CAP_M + I.cap_s, tabbits = I.big_tabbits;
+    unsigned char *p = I.big_scratch + (size_t)blockIdx.x * I.big_stride;
+    Stage<unsigned> W;
+    W.key = (ulonglong2 *)p; p += (size_t)Ecap * sizeof(ulonglong2);
+    W.val = (double *)p; p += (size_t)Ecap * sizeof(double);
+    W.acc_lo = (u64 *)p; p += (size_t)Ecap * 8;
+    W.acc_hi = (u64 *)p; p += (size_t)Ecap * 8;
+    W.nacc = (int *)p; p += (size_t)Ecap * 4;
+    W.eflag = (int *)p; p += (size_t)Ecap * 4;
+    W.opos = (unsigned *)p; p += (size_t)Ecap * 4;
+    W.tab = (unsigned *)p;
+    for (int q = blockIdx.x; q < nbig; q += BIG_BLOCKS) {
+        int b = I.big_list[q];
+        if (!(b & BIG_SCRATCH)) continue;
+        b &= ~BIG_SCRATCH;
+        if (!I.big_scratch) {  // no scratch yet: report, the host allocates it and repeats the iteration
+            if (t == 0) atomicOr(&I.st->err, ERRB_SPAWN_CAP);
+            break;
+        }
+        anni_bucket<unsigned>(I, S, W, tabbits, b, par, it, shift, I.cnt[par][b], I.scnt_i[b], I.scnt_n[b]);
+        __syncthreads();
+    }
+}
+
 __global__ void __launch_bounds__(K3_THREADS) k_annihilate_big(const DevInst *__restrict__ insts, int n_inst)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     K3Smem &Sm = *reinterpret_cast<K3Smem *>(smem_raw);
     K3Shared &S = Sm.sh;
     const int t = threadIdx.x;
-    for (int ii = 0; ii < n_inst; ii++) {
-        const DevInst &I = insts[ii];
-        if (t == 0) {
-            S.hdr_err = *(volatile int *)&I.st->err;
-            S.hdr_par = I.st->parity;
-            S.hdr_it = I.st->iter;
-            S.hdr_S = I.st->S;
-            S.n_new = I.st->big_n;
-        }
+    for (int i0 = 0; i0 < n_inst; i0 += K3_THREADS) {
+        // thread t looks at run i0 + t; only runs with deferred buckets follow
         __syncthreads();
-        const int err = S.hdr_err, par = S.hdr_par, nbig = S.n_new;
-        const long long it = S.hdr_it;
-        const double shift = S.hdr_S;
+        if (t == 0) S.side_n = 0;
         __syncthreads();
-        if (err || nbig == 0) continue;
-        const Stage<unsigned short> Ws{Sm.key, Sm.val, Sm.acc_lo, Sm.acc_hi, Sm.nacc, Sm.eflag, Sm.tab, Sm.opos};
-        for (int q = blockIdx.x; q < nbig; q += gridDim.x) {
-            const int b = I.big_list[q];
-            const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
-            if (m + si + sn <= EMAX) {
-                anni_bucket<unsigned short>(I, S, Ws, TABBITS, b, par, it, shift, m, si, sn);
-                __syncthreads();
-            }
+        bool work = false;
+        if (i0 + t < n_inst) {
+            const IterState *st = insts[i0 + t].st;
+            const int err = *(volatile const int *)&st->err, n = st->big_n;
+            work = n > 0 && !err;
         }
-        if (blockIdx.x >= BIG_BLOCKS) continue;
-        // beyond shared memory: this block's slice of the global scratch
-        const int Ecap = CAP_M + I.cap_s, tabbits = I.big_tabbits;
-        unsigned char *p = I.big_scratch + (size_t)blockIdx.x * I.big_stride;
-        Stage<unsigned> W;
-        W.key = (ulonglong2 *)p; p += (size_t)Ecap * sizeof(ulonglong2);
-        W.val = (double *)p; p += (size_t)Ecap * sizeof(double);
-        W.acc_lo = (u64 *)p; p += (size_t)Ecap * 8;
-        W.acc_hi = (u64 *)p; p += (size_t)Ecap * 8;
-        W.nacc = (int *)p; p += (size_t)Ecap * 4;
-        W.eflag = (int *)p; p += (size_t)Ecap * 4;
-        W.opos = (unsigned *)p; p += (size_t)Ecap * 4;
-        W.tab = (unsigned *)p;
-        for (int q = blockIdx.x; q < nbig; q += BIG_BLOCKS) {
-            const int b = I.big_list[q];
-            const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
-            if (m + si + sn <= EMAX) continue;
-            if (!I.big_scratch) {  // no scratch yet: report, the host allocates it and repeats the iteration
-                if (t == 0) atomicOr(&I.st->err, ERRB_SPAWN_CAP);
-                break;
-            }
-            anni_bucket<unsigned>(I, S, W, tabbits, b, par, it, shift, m, si, sn);
+        if (work) Sm.eflag[atomicAdd(&S.side_n, 1)] = i0 + t;
+        __syncthreads();
+        const int nwork = S.side_n;
+        const int mine = t < nwork ? Sm.eflag[t] : 0;  // the arrays are reused below: thread w keeps entry w
+        for (int w = 0; w < nwork; w++) {
+            if (t == w) S.n_new = mine;
             __syncthreads();
+            annihilate_deferred(insts[S.n_new], Sm);
         }
     }
 }
 
 // ------------------------------------------------------------------ finalize
-__global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restrict__ insts, int n_inst)
+// one run's iteration committed by one block; insts, self: the table the run
+// lies in (its replica partner is looked up there), NULL for a run alone
+__device__ __forceinline__ void finalize_run(const DevInst &I, const DevInst *insts, int self)
 {
-    const DevInst &I = insts[blockIdx.x];
     IterState *st = I.st;
     __shared__ int s_err;
     __shared__ double s_r[6][K5_THREADS / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int nbk = 1 << I.bb;
-    const bool pair = I.partner > (int)blockIdx.x;  // the first replica reports the cross estimators
+    const bool pair = insts && I.partner > self;  // the first replica reports the cross estimators
     const bool trial = I.trial_bits != 0;
     const bool tree = trial || pair;  // binary64 estimator sums need the whole block; otherwise warp 0 alone
     if (!tree && warp != 0) return;
@@ -1861,7 +1898,7 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
         // a replica commits its iteration only together with its partner: not
         // if the partner skipped it (a flag was up when its spawning began) or
         // failed in it
-        const IterState *pst = I.partner >= 0 ? insts[I.partner].st : nullptr;
+        const IterState *pst = insts && I.partner >= 0 ? insts[I.partner].st : nullptr;
         if (!e && pst && (*(volatile const int *)&pst->err_at_start ||
                           (*(volatile const int *)&pst->err & ERRB_STAGE))) {
             st->err = ERRB_PARTNER;
@@ -1979,6 +2016,37 @@ __global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restri
     if (I.trial_size > 0 && !trial_built && vary && it + 1 == shift_start + I.trial_start) flags |= ERRB_PAUSE_TRIAL;
     if (it + 1 >= stop_iter) flags |= ERRB_STOP;
     if (flags) st->err |= flags;
+}
+
+__global__ void __launch_bounds__(K5_THREADS) k_finalize(const DevInst *__restrict__ insts, int n_inst)
+{
+    finalize_run(insts[blockIdx.x], insts, (int)blockIdx.x);
+}
+
+// the end of one run's iteration in one launch: its deferred buckets, if any,
+// then the block that is done last commits it (a launch of their own for
+// buckets that are hardly ever there cost 2 to 6 us of 37 to 83 us)
+static_assert(K3_THREADS == K5_THREADS, "one block does both");
+__global__ void __launch_bounds__(K3_THREADS) k_finish(const __grid_constant__ DevInst I)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ int s_last;
+    const int nbig = I.st->big_n;  // changed by the committing block alone
+    if (nbig == 0) {
+        if (blockIdx.x) return;
+    } else {
+        annihilate_deferred(I, *reinterpret_cast<K3Smem *>(smem_raw));
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(&I.st->done, 1) == (int)gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        if (threadIdx.x == 0) I.st->done = 0;
+    }
+    finalize_run(I, nullptr, 0);
 }
 
 // ------------------------------------------------------------------ growth and import
@@ -2155,10 +2223,28 @@ void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps)
     *anni_bps = g_anni_bps;
 }
 
+// How a list's buckets are dealt to warps: as many warps per bucket as it
+// takes to reach every resident warp of the GPU, and the number of attempts
+// above which a determinant goes to the heavy queue (a warp draws its
+// attempts 32 at a time, one after the other)
+struct SpawnSplit {
+    int parts, grid;
+    unsigned heavy_min;
+};
+static SpawnSplit spawn_split(int n_units, int bps, bool alone)
+{
+    SpawnSplit p;
+    const int warps = num_sms() * 4 * SP_WARPS;
+    p.parts = 1;
+    while (p.parts < CAP_M / 32 && (long long)n_units * p.parts < 2 * warps) p.parts *= 2;
+    p.heavy_min = p.parts > 1 ? 64 : (alone ? HEAVY_ATT : HEAVY_ATT / 2);
+    const long long need = ((long long)n_units * p.parts + SP_WARPS - 1) / SP_WARPS;
+    p.grid = (int)(need < (long long)num_sms() * bps ? need : (long long)num_sms() * bps);
+    return p;
+}
+
 // spawning of one run (`one`, the host image of its descriptor) or of a table
-// of runs (one = NULL).  A bucket's slots are dealt to as many warps as it
-// takes to reach every resident warp of the GPU.  adaptive: some run uses the
-// adaptive shift.
+// of runs (one = NULL); adaptive: some run uses the adaptive shift
 template <int GEN>
 static void launch_spawn_one(const DevInst *one, int grid, int n_units, int parts, unsigned heavy_min, cudaStream_t s)
 {
@@ -2168,13 +2254,9 @@ static void launch_spawn_one(const DevInst *one, int grid, int n_units, int part
 void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s)
 {
-    const int bps = g_spawn_bps > 1 ? g_spawn_bps : (adaptive ? 3 : 4);
-    const int warps = num_sms() * 4 * SP_WARPS;
-    int parts = 1;
-    while (parts < CAP_M / 32 && (long long)n_units * parts < 2 * warps) parts *= 2;
-    const unsigned heavy_min = parts > 1 ? 64 : HEAVY_ATT;
-    const long long need = ((long long)n_units * parts + SP_WARPS - 1) / SP_WARPS;
-    const int grid = (int)(need < (long long)num_sms() * bps ? need : (long long)num_sms() * bps);
+    const SpawnSplit p = spawn_split(n_units, g_spawn_bps > 1 ? g_spawn_bps : (adaptive ? 3 : 4), one != nullptr);
+    const int grid = p.grid, parts = p.parts;
+    const unsigned heavy_min = p.heavy_min;
     if (one && one->kind == FCIQMC_HUBBARD) launch_spawn_one<GEN_HOP>(one, grid, n_units, parts, heavy_min, s);
     else if (one && one->pchb) launch_spawn_one<GEN_PCHB>(one, grid, n_units, parts, heavy_min, s);
     else if (one) launch_spawn_one<GEN_UNIFORM>(one, grid, n_units, parts, heavy_min, s);
@@ -2192,6 +2274,7 @@ void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cu
 cudaError_t init_kernels()
 {
     cudaError_t e = cudaFuncSetAttribute(k_annihilate_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
     auto warp_smem = [&](auto *f, size_t bytes, int blocks) {  // the resident blocks need their shared memory at once
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e == cudaSuccess)
@@ -2236,6 +2319,12 @@ cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const in
 void launch_annihilate_big(const DevInst *dinst, int n_inst, cudaStream_t s)
 {
     k_annihilate_big<<<num_sms() * 3 > BIG_BLOCKS ? num_sms() * 3 : BIG_BLOCKS, K3_THREADS, sizeof(K3Smem), s>>>(dinst, n_inst);
+}
+
+// the deferred buckets of one run and its commit
+void launch_finish(const DevInst *one, cudaStream_t s)
+{
+    k_finish<<<num_sms() * 3 > BIG_BLOCKS ? num_sms() * 3 : BIG_BLOCKS, K3_THREADS, sizeof(K3Smem), s>>>(*one);
 }
 
 void launch_finalize(const DevInst *dinst, int n_inst, cudaStream_t s)

@@ -81,3 +81,28 @@ def test_imported_list_at_the_edges_bit_exact(name, max_dets):
     o.step(3)
     assert_states_equal(fq.fciqmc_export_state(g), o.export())
     assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats(), first=0)
+
+
+@pytest.mark.parametrize("max_dets", [16, 4000])
+def test_crowded_buckets_bit_exact(max_dets):
+    """Hundreds of walkers on every determinant of a small space, alone and in
+    a batch: every bucket holds more spawns than a warp annihilates, some more
+    than fit shared memory, and the two kinds are annihilated side by side."""
+    fq = _fq()
+    sysd = workloads.hubbard_1d(8, 1.0, 4.0)
+    s = oracle.system_from_workload(sysd)
+    a, b = np.array(s.determinants(), np.uint64).T
+    rng = np.random.default_rng(5)
+    c = rng.normal(0.0, 1.0, a.size) * np.where(rng.random(a.size) < 0.3, 400.0, 20.0)
+    prm = dict(tau=0.01, target_walkers=1e9, seed=3, shift_damping=0.5, shift_interval=5, initiator_threshold=3.0)
+    o = oracle.Run(s, **prm)
+    o.import_state(a, b, c, 0, -2.0)
+    o.step(4)
+    gs = [fq.fciqmc_create(sysd, dict(prm, max_dets=max_dets)) for _ in range(4)]
+    for g in gs:
+        fq.fciqmc_import_state(g, a, b, c, 0, -2.0)
+    fq.fciqmc_step(gs[0], 4)
+    fq.fciqmc_step_batch(gs[1:], 4)
+    for g in gs:
+        assert_states_equal(fq.fciqmc_export_state(g), o.export())
+        assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
