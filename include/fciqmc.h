@@ -282,7 +282,7 @@ int64_t fciqmc_num_dets(fciqmc_handle *h);
  * in D.  *n_out receives the number of determinants (also when it exceeds
  * cap, in which case FCIQMC_ERR_CAPACITY is returned and nothing copied).
  * The list is compacted and radix-sorted on the device in transient scratch
- * (about 68 bytes per determinant, from the run's allocator); when
+ * (about 40 bytes per determinant, from the run's allocator); when
  * max_device_bytes leaves no room for it the sort runs on the host. */
 int fciqmc_export_state(fciqmc_handle *h, int64_t cap, uint64_t *alpha, uint64_t *beta, double *c,
                         double *hdiag, int32_t *flags, int64_t *n_out);

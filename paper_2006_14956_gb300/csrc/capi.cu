@@ -814,20 +814,32 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     // exact-sum scale F: every integral (and E_core) must lie on the grid 2^-F
     int lsb_min = 0, msb_max = -1100;
     bool any = false;
-    auto scan = [&](double x) {
-        if (x == 0.0) return true;
-        if (!std::isfinite(x)) return false;
-        u64 m;
-        int e;
-        decompose(x, &m, &e);
-        lsb_min = any ? std::min(lsb_min, e) : e;
-        msb_max = any ? std::max(msb_max, exponent_of(std::fabs(x))) : exponent_of(std::fabs(x));
-        any = true;
+    // lowest and highest set bit of the values by their bit patterns (x = m 2^e, m odd)
+    auto scan_all = [&](const double *x, size_t n) {
+        int lo = INT_MAX;
+        u64 top = 0;
+        for (size_t k = 0; k < n; k++) {
+            u64 b;
+            memcpy(&b, x + k, 8);
+            b &= ~(1ULL << 63);
+            const int ex = (int)(b >> 52);
+            const u64 m = (b & 0xFFFFFFFFFFFFFULL) | (ex ? 1ULL << 52 : 0ULL);
+            top = std::max(top, b);
+            if (m) lo = std::min(lo, (ex ? ex : 1) - 1075 + __builtin_ctzll(m));
+        }
+        if (top >> 52 == 0x7ff) return false;
+        if (top) {
+            double t;
+            memcpy(&t, &top, 8);
+            lsb_min = any ? std::min(lsb_min, lo) : lo;
+            msb_max = any ? std::max(msb_max, exponent_of(t)) : exponent_of(t);
+            any = true;
+        }
         return true;
     };
-    for (double x : h->h) if (!scan(x)) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite one-electron integral");
-    for (double x : h->eri) if (!scan(x)) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite two-electron integral");
-    if (!scan(h->ecore)) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite core energy");
+    if (!scan_all(h->h.data(), h->h.size())) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite one-electron integral");
+    if (!scan_all(h->eri.data(), h->eri.size())) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite two-electron integral");
+    if (!scan_all(&h->ecore, 1)) return bail(FCIQMC_ERR_INVALID_ARG, "non-finite core energy");
     const int n = h->na + h->nb;
     int F = any ? std::max(0, -lsb_min) : 0;
     int terms_bits = 0;
@@ -850,9 +862,9 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
         msb_max = -1100;
         any = false;
         lsb_min = 0;
-        for (double x : h->h) scan(x);
-        for (double x : h->eri) scan(x);
-        scan(h->ecore);
+        scan_all(h->h.data(), h->h.size());
+        scan_all(h->eri.data(), h->eri.size());
+        scan_all(&h->ecore, 1);
         F = any ? std::max(0, -lsb_min) : 0;
     }
     if (any && msb_max + F + terms_bits + 2 > 125)
@@ -874,28 +886,6 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
         h->own_stream = true;
     }
 
-    // fixed-point tables for the exact diagonal sums
-    std::vector<ulonglong2> hfx(N), Jfx((size_t)N * N), JKfx((size_t)N * N);
-    auto put = [](ulonglong2 &d, i128 v) { d.x = (u64)(u128)v; d.y = (u64)((u128)v >> 64); };
-    for (int p = 0; p < N; p++) {
-        put(hfx[p], host_fixed(h->h[(size_t)p * N + p], F));
-        for (int q = 0; q < N; q++) {
-            put(Jfx[(size_t)p * N + q], host_fixed(h->eri[pair_index(pair_index(p, p), pair_index(q, q))], F));
-            put(JKfx[(size_t)p * N + q], host_fixed(h->eri[pair_index(pair_index(p, p), pair_index(q, q))], F) -
-                                             host_fixed(h->eri[pair_index(pair_index(p, q), pair_index(q, p))], F));
-        }
-    }
-    // single-excitation terms: (ai|kk) and (ai|kk) - (ak|ki) per (a, i, k)
-    std::vector<ulonglong2> Sfx((size_t)N * N * N * 2);
-    for (int a = 0; a < N; a++)
-        for (int i = 0; i < N; i++)
-            for (int k = 0; k < N; k++) {
-                const i128 c = host_fixed(h->eri[pair_index(pair_index(a, i), pair_index(k, k))], F);
-                const i128 x = host_fixed(h->eri[pair_index(pair_index(a, k), pair_index(k, i))], F);
-                const size_t o = (((size_t)a * N + i) * N + k) * 2;
-                put(Sfx[o], c);
-                put(Sfx[o + 1], c - x);
-            }
     // X(ref): sum over occupied orbitals and occupied pairs
     std::vector<std::pair<int, int>> occ;
     for (int p = 0; p < N; p++) if ((h->ref_a >> p) & 1) occ.push_back({p, 0});
@@ -957,10 +947,10 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     // integrals and tables on the device
     double *dh = (double *)dev_alloc(h, h->h.size() * sizeof(double));
     double *deri = (double *)dev_alloc(h, h->eri.size() * sizeof(double));
-    ulonglong2 *dhfx = (ulonglong2 *)dev_alloc(h, hfx.size() * sizeof(ulonglong2));
-    ulonglong2 *dJ = (ulonglong2 *)dev_alloc(h, Jfx.size() * sizeof(ulonglong2));
-    ulonglong2 *dK = (ulonglong2 *)dev_alloc(h, JKfx.size() * sizeof(ulonglong2));
-    ulonglong2 *dS = (ulonglong2 *)dev_alloc(h, Sfx.size() * sizeof(ulonglong2));
+    ulonglong2 *dhfx = (ulonglong2 *)dev_alloc(h, (size_t)N * sizeof(ulonglong2));
+    ulonglong2 *dJ = (ulonglong2 *)dev_alloc(h, (size_t)N * N * sizeof(ulonglong2));
+    ulonglong2 *dK = (ulonglong2 *)dev_alloc(h, (size_t)N * N * sizeof(ulonglong2));
+    ulonglong2 *dS = (ulonglong2 *)dev_alloc(h, (size_t)N * N * N * 2 * sizeof(ulonglong2));
     int *dnbr = (int *)dev_alloc(h, std::max<size_t>(1, h->nbr.size()) * sizeof(int));
     h->dinst = (DevInst *)dev_alloc(h, sizeof(DevInst));
     h->dunit = (int *)dev_alloc(h, 2 * sizeof(int));
@@ -972,10 +962,8 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     cudaMemsetAsync(I.acc, 0, NSHARD * ACC_STRIDE * sizeof(u64), h->stream);
     cudaMemcpyAsync(dh, h->h.data(), h->h.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     cudaMemcpyAsync(deri, h->eri.data(), h->eri.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(dhfx, hfx.data(), hfx.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(dJ, Jfx.data(), Jfx.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(dK, JKfx.data(), JKfx.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(dS, Sfx.data(), Sfx.size() * sizeof(ulonglong2), cudaMemcpyHostToDevice, h->stream);
+    if (launch_tables(N, F, dh, deri, dhfx, dJ, dK, dS, h->stream) != cudaSuccess)
+        return bail(FCIQMC_ERR_CUDA, "integral table set-up failed");
     if (!h->nbr.empty()) cudaMemcpyAsync(dnbr, h->nbr.data(), h->nbr.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream);
     I.h = dh; I.eri = deri; I.hfx = dhfx; I.Jfx = dJ; I.JKfx = dK; I.Sfx = dS; I.nbr = dnbr;
     I.st = h->dstate;
@@ -1469,32 +1457,31 @@ static int export_state_impl(fciqmc_handle *h, int64_t cap, uint64_t *alpha, uin
     if (rc) return rc;
     const int par = h->hst.parity;
     const size_t nbk = (size_t)1 << h->bb, nm = nbk * CAP_M;
-    std::vector<int> cnt(nbk);
-    CUDA_TRY(h, cudaMemcpy(cnt.data(), h->hi.cnt[par], nbk * sizeof(int), cudaMemcpyDeviceToHost));
-    int64_t n = 0;
-    for (int x : cnt) n += x;
+    // on the device: counted, compacted, radix-sorted by (alpha, beta) and
+    // gathered; only the n live entries are copied out.  Transient scratch from
+    // the run's allocator; where it cannot be had, the same order is produced
+    // on the host.
+    // the group counts go to the list of deferred buckets, unused between iterations
+    static_assert(sizeof(int) * XC_GROUP >= 2 * sizeof(long long), "room for the group counts");
+    long long *gsum = (long long *)h->hi.big_list;
+    const long long *total = nullptr;
+    long long n = 0;
+    CUDA_TRY(h, export_count(h->hi.cnt[par], (int)nbk, gsum, &total, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(&n, total, sizeof(n), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     *n_out = n;
     if (n > cap) return fail(h, FCIQMC_ERR_CAPACITY, "export buffer too small");
     if (n > 0 && (!alpha || !beta || !c)) return FCIQMC_ERR_INVALID_ARG;
     if (n == 0) return FCIQMC_OK;
-    // on the device: compaction, radix sort by (alpha, beta), gather; only the
-    // n live entries are copied out.  Transient scratch from the run's
-    // allocator; where it cannot be had, the same order is produced on the host.
     {
-        std::vector<long long> off(nbk + 1, 0);
-        for (size_t b = 0; b < nbk; b++) off[b + 1] = off[b] + cnt[b];
-        const size_t off_bytes = ((nbk + 1) * sizeof(long long) + 255) & ~(size_t)255;
-        unsigned char *scr = (unsigned char *)dev_alloc(h, off_bytes + export_scratch_bytes(n));
-        if (scr) {
+        unsigned char *work = (unsigned char *)dev_alloc(h, export_scratch_bytes(n));
+        if (work) {
             const u64 *oa, *ob;
             const double *oc, *ohd;
             const int32_t *ofl;
-            cudaError_t e = cudaMemcpyAsync(scr, off.data(), (nbk + 1) * sizeof(long long), cudaMemcpyHostToDevice,
-                                            h->stream);
-            if (e == cudaSuccess)
-                e = export_sorted(h->hi.key[par], h->hi.c[par], h->hi.hd[par], h->hi.fl[par], h->hi.cnt[par],
-                                  (const long long *)scr, (int)nbk, n, h->norb, scr + off_bytes, &oa, &ob, &oc, &ohd,
-                                  &ofl, h->stream);
+            cudaError_t e = export_sorted(h->hi.key[par], h->hi.c[par], h->hi.hd[par], h->hi.fl[par], h->hi.cnt[par],
+                                          gsum, (int)nbk, n, h->norb, h->na, h->nb, work, &oa, &ob, &oc,
+                                          &ohd, &ofl, h->stream);
             if (e == cudaSuccess) e = cudaMemcpyAsync(alpha, oa, n * sizeof(u64), cudaMemcpyDeviceToHost, h->stream);
             if (e == cudaSuccess) e = cudaMemcpyAsync(beta, ob, n * sizeof(u64), cudaMemcpyDeviceToHost, h->stream);
             if (e == cudaSuccess) e = cudaMemcpyAsync(c, oc, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
@@ -1503,11 +1490,13 @@ static int export_state_impl(fciqmc_handle *h, int64_t cap, uint64_t *alpha, uin
             if (e == cudaSuccess && flags)
                 e = cudaMemcpyAsync(flags, ofl, n * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-            dev_free(h, scr);
+            dev_free(h, work);
             if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("export: ") + cudaGetErrorString(e));
             return FCIQMC_OK;
         }
     }
+    std::vector<int> cnt(nbk);
+    CUDA_TRY(h, cudaMemcpy(cnt.data(), h->hi.cnt[par], nbk * sizeof(int), cudaMemcpyDeviceToHost));
     std::vector<ulonglong2> k(nm);
     std::vector<double> cc(nm), hh(nm);
     std::vector<uint8_t> ff(nm);

@@ -46,6 +46,7 @@ constexpr int IMPORT_M = 160;         // determinants of an imported list per bu
 constexpr int MAX_BB = 24;            // at most 2^24 buckets: slot indices (bucket * CAP_M + position) fit 32 bits
 constexpr int CAP_S0 = 96;            // initial spawn capacity per bucket (grows at run time)
 constexpr int TABBITS = 12;           // shared-memory hash table of the large-bucket kernel (2 x EMAX slots)
+constexpr int XC_GROUP = 16;          // buckets per block of the export's compaction (two per warp)
 constexpr int BIG_BLOCKS = 64;        // blocks of the large-bucket annihilation kernel
 constexpr int K5_THREADS = 256;
 constexpr int KIDX = 512;             // slots of the per-bucket list index (adaptive shift)
@@ -246,6 +247,8 @@ cudaError_t replica_kernel_init();
 void launch_rebucket(const DevInst *src, const DevInst *dst, int nb_src, int parity, cudaStream_t s);
 void launch_diag(const DevInst *dinst, int parity, int nb, cudaStream_t s);
 void launch_diag_list(const DevInst *one, int par, const unsigned *list, int nn, cudaStream_t s);
+cudaError_t launch_tables(int N, int F, const double *h, const double *eri, ulonglong2 *hfx, ulonglong2 *J, ulonglong2 *JK,
+                          ulonglong2 *S, cudaStream_t s);
 cudaError_t launch_import_check(const u64 *a, const u64 *b, const double *c, long long n, int na, int nb, u64 normask,
                                 u64 ra, u64 rb, int *flags, cudaStream_t s);
 cudaError_t launch_import_count(const u64 *a, const u64 *b, long long n, int bb, int *cnt, int *over, cudaStream_t s);
@@ -272,10 +275,12 @@ void set_launch_geometry(int spawn_bps, int heavy_bps, int anni_bps);
 int launch_geometry_generation();
 void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps);
 cudaError_t ref_abs_sum(const DevInst *dinst, double *dpartial, double *out, cudaStream_t s);
+cudaError_t export_count(const int *cnt, int nbk, long long *gsum, const long long **total, cudaStream_t s);
 size_t export_scratch_bytes(long long n);
 cudaError_t export_sorted(const ulonglong2 *key, const double *c, const double *hd, const uint8_t *fl, const int *cnt,
-                          const long long *off, int nbk, long long n, int norb, void *scratch, const u64 **oa,
-                          const u64 **ob, const double **oc, const double **ohd, const int32_t **ofl, cudaStream_t s);
+                          const long long *gsum, int nbk, long long n, int norb, int na, int nb, void *scratch,
+                          const u64 **oa, const u64 **ob, const double **oc, const double **ohd, const int32_t **ofl,
+                          cudaStream_t s);
 
 // host helpers shared with capi.cu
 u64 det_hash_host(u64 a, u64 b);

@@ -2271,10 +2271,14 @@ void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cu
     else k_spawn_heavy_batch<<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(dinst, n_inst);
 }
 
+__global__ void k_diag_list_long(const __grid_constant__ DevInst I, int par, const unsigned *list, int nn);
 cudaError_t init_kernels()
 {
     cudaError_t e = cudaFuncSetAttribute(k_annihilate_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(K3Smem));
+    if (e == cudaSuccess)  // 64 orbitals at most
+        e = cudaFuncSetAttribute(k_diag_list_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)((2 * 64 * 64 + 64) * sizeof(ulonglong2)));
     auto warp_smem = [&](auto *f, size_t bytes, int blocks) {  // the resident blocks need their shared memory at once
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e == cudaSuccess)
@@ -2357,9 +2361,84 @@ __global__ void __launch_bounds__(256) k_diag_list(const __grid_constant__ DevIn
     for (int q = 4 * gw; q < nn; q += 4 * nwarp) diag_four(I, list + q, min(4, nn - q), par, s_pair, s_orb[wl]);
 }
 
+// the same for a long list: one determinant per lane, the tables in shared
+// memory.  A sum is n (n + 1) / 2 16-byte loads at scattered places; from
+// global memory every lane's load is an L1 line of its own (1.47 ms for 3e6
+// determinants of 20 electrons, 1.16 ms with one determinant per lane)
+constexpr int DL_THREADS = 1024;
+__global__ void __launch_bounds__(DL_THREADS, 1) k_diag_list_long(const __grid_constant__ DevInst I, int par,
+                                                                  const unsigned *list, int nn)
+{
+    extern __shared__ ulonglong2 dl_tab[];
+    const int N = I.norb, N2 = N * N;
+    ulonglong2 *JK = dl_tab, *J = dl_tab + N2, *hp = dl_tab + 2 * N2;
+    for (int q = threadIdx.x; q < N2; q += DL_THREADS) {
+        JK[q] = __ldg(I.JKfx + q);
+        J[q] = __ldg(I.Jfx + q);
+        if (q < N) hp[q] = __ldg(I.hfx + q);
+    }
+    __syncthreads();
+    const i128 xref = (i128)(((u128)I.xref_hi << 64) | (u128)I.xref_lo);
+    auto at = [](const ulonglong2 &v) { return (i128)(((u128)v.y << 64) | (u128)v.x); };
+    for (long long i = (long long)blockIdx.x * DL_THREADS + threadIdx.x; i < nn; i += (long long)gridDim.x * DL_THREADS) {
+        const unsigned d = list[i];
+        const ulonglong2 kk = I.key[par][d];
+        i128 x = -xref;
+        for (int s = 0; s < 2; s++) {
+            u64 w = s ? kk.y : kk.x;
+            while (w) {
+                const int p = __ffsll((long long)w) - 1;
+                w &= w - 1;
+                x += at(hp[p]);
+                for (u64 o = w; o; o &= o - 1) x += at(JK[p * N + __ffsll((long long)o) - 1]);
+                if (!s)
+                    for (u64 o = kk.y; o; o &= o - 1) x += at(J[p * N + __ffsll((long long)o) - 1]);
+            }
+        }
+        I.hd[par][d] = fixed_to_double(x, I.F);
+    }
+}
+
+// ------------------------------------------------------------------ integral tables
+// The fixed-point tables of a run (h_pp, (pp|qq), (pp|qq) - (pq|qp), and per
+// (a, i, k) the pair (ai|kk), (ai|kk) - (ak|ki)) from its integrals, one entry
+// per thread; every integral lies on the grid 2^-F (the host checked).  On the
+// host the 2 N^3 + 2 N^2 conversions of 50 orbitals took 7 of the 13 ms that
+// creating a run takes.
+__global__ void __launch_bounds__(256) k_tables(int N, int F, const double *__restrict__ h, const double *__restrict__ eri,
+                                                ulonglong2 *hfx, ulonglong2 *J, ulonglong2 *JK, ulonglong2 *S)
+{
+    auto fixed = [&](const double *p) { return to_fixed(__ldg(p), F); };
+    auto put = [](ulonglong2 *d, i128 v) { *d = make_ulonglong2((u64)(u128)v, (u64)((u128)v >> 64)); };
+    const long long n3 = (long long)N * N * N;
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n3; q += (long long)gridDim.x * blockDim.x) {
+        const int k = (int)(q % N), i = (int)(q / N % N), a = (int)(q / N / N);
+        const i128 c = fixed(eri + pidx(pidx(a, i), pidx(k, k))), x = fixed(eri + pidx(pidx(a, k), pidx(k, i)));
+        put(S + 2 * q, c);
+        put(S + 2 * q + 1, c - x);
+        if (a == i) {
+            put(J + a * N + k, c);        // (aa|kk)
+            put(JK + a * N + k, c - x);   // (aa|kk) - (ak|ka)
+            if (k == 0) put(hfx + a, fixed(h + a * N + a));
+        }
+    }
+}
+
+cudaError_t launch_tables(int N, int F, const double *h, const double *eri, ulonglong2 *hfx, ulonglong2 *J, ulonglong2 *JK,
+                          ulonglong2 *S, cudaStream_t s)
+{
+    const int blocks = (N * N * N + 255) / 256;
+    k_tables<<<blocks < num_sms() * 8 ? blocks : num_sms() * 8, 256, 0, s>>>(N, F, h, eri, hfx, J, JK, S);
+    return cudaGetLastError();
+}
+
 void launch_diag_list(const DevInst *one, int par, const unsigned *list, int nn, cudaStream_t s)
 {
-    if (nn > 0) k_diag_list<<<num_sms() * 4, 256, 0, s>>>(*one, par, list, nn);
+    // the line: a determinant for every thread of the long list's kernel (one
+    // block per SM, which first copies the tables)
+    const size_t smem = (size_t)(2 * one->norb * one->norb + one->norb) * sizeof(ulonglong2);
+    if (nn >= num_sms() * DL_THREADS) k_diag_list_long<<<num_sms(), DL_THREADS, smem, s>>>(*one, par, list, nn);
+    else if (nn > 0) k_diag_list<<<num_sms() * 4, 256, 0, s>>>(*one, par, list, nn);
 }
 
 void launch_rebucket(const DevInst *src, const DevInst *dst, int nb_src, int parity, cudaStream_t s)
