@@ -101,35 +101,39 @@ __global__ void k_mark_d(const DevInst *__restrict__ I, int par, int nb)
 // product is rounded to binary64, truncated toward zero to a multiple of
 // 2^-64, and the row's truncated products are summed exactly (128-bit fixed
 // point on the grid 2^-64) and rounded once.  The sum does not depend on
-// the order of its terms, so a warp shares a row: lane k takes the columns
-// k, k + 32, ... and the lanes' partial sums are joined by a shuffle tree.
+// the order of its terms, so a block shares a row: thread k takes the columns
+// k, k + 256, ... and the partial sums are joined by shuffle trees.  A warp per
+// row waited for the few rows that couple to nearly all of D: 96 us for 1e4
+// rows (50 orbitals), now 51.
 // Products of magnitude 2^48 or more (beyond what 2^14 of them can sum to
 // in 127 bits) raise the numeric error.  C_D of the current parity is read;
 // the other buffer receives the iteration's result, so a repeated iteration
 // starts from unchanged values.
 constexpr int SEMI_GRID = 64;
-__global__ void __launch_bounds__(256) k_semistoch(const DevInst *__restrict__ insts, int n_inst)
+constexpr int SEMI_THREADS = 256;
+__global__ void __launch_bounds__(SEMI_THREADS) k_semistoch(const DevInst *__restrict__ insts, int n_inst)
 {
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarp = (gridDim.x * blockDim.x) >> 5;
+    __shared__ u64 s_acc[2][SEMI_THREADS / 32][2];  // two sets in turn: one barrier per row
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int set = 0;
     for (int ii = 0; ii < n_inst; ii++) {
         const DevInst &I = insts[ii];
         if (I.nd == 0) continue;
-        if (*(volatile int *)&I.st->err) continue;
+        if (__syncthreads_or(*(volatile int *)&I.st->err)) continue;
         const double S = I.st->S;
         const double *cur = I.dc_buf[I.st->parity];
         bool bad = false;
-        for (int r = gw; r < I.nd; r += nwarp) {
+        for (int r = blockIdx.x; r < I.nd; r += gridDim.x, set ^= 1) {
             const long long q0 = I.drow[r], q1 = I.drow[r + 1];
             i128 acc = 0;
-            // four terms per lane in flight: their loads issued before the adds
-            long long q = q0 + lane;
-            for (; q + 96 < q1; q += 128) {
+            // four terms per thread in flight: their loads issued before the adds
+            long long q = q0 + t;
+            for (; q + 3 * SEMI_THREADS < q1; q += 4 * SEMI_THREADS) {
                 double v[4], x[4];
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
-                    v[k] = __ldg(I.dval + q + 32 * k);
-                    x[k] = cur[__ldg(I.dcol + q + 32 * k)];
+                    v[k] = __ldg(I.dval + q + SEMI_THREADS * k);
+                    x[k] = cur[__ldg(I.dcol + q + SEMI_THREADS * k)];
                 }
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
@@ -138,14 +142,22 @@ __global__ void __launch_bounds__(256) k_semistoch(const DevInst *__restrict__ i
                     acc += to_fixed(p, SEMI_GRID);
                 }
             }
-            for (; q < q1; q += 32) {
+            for (; q < q1; q += SEMI_THREADS) {
                 const double p = __ldg(I.dval + q) * cur[__ldg(I.dcol + q)];
                 bad |= !abs_lt(p, 0x1p48);
                 acc += to_fixed(p, SEMI_GRID);
             }
             for (int m = 16; m >= 1; m >>= 1) acc += shfl_xor_i128(acc, m);
             if (lane == 0) {
-                const double y = fixed_to_double(acc, SEMI_GRID);
+                s_acc[set][warp][0] = (u64)(u128)acc;
+                s_acc[set][warp][1] = (u64)((u128)acc >> 64);
+            }
+            __syncthreads();
+            if (t == 0) {
+                i128 sum = 0;
+                for (int w = 0; w < SEMI_THREADS / 32; w++)
+                    sum += (i128)(((u128)s_acc[set][w][1] << 64) | (u128)s_acc[set][w][0]);
+                const double y = fixed_to_double(sum, SEMI_GRID);
                 const double c = cur[r];
                 I.dc_new[r] = c - I.tau * (y - S * c);
             }
@@ -164,11 +176,11 @@ static int sms()
 
 void launch_semistoch(const DevInst *dinst, int n_inst, int max_nd, cudaStream_t s)
 {
-    // one warp per row, eight rows per block, at most eight blocks per SM
-    int blocks = (max_nd + 7) / 8;
+    // a block per row, at most eight blocks per SM
+    int blocks = max_nd;
     if (blocks > sms() * 8) blocks = sms() * 8;
     if (blocks < 1) blocks = 1;
-    k_semistoch<<<blocks, 256, 0, s>>>(dinst, n_inst);
+    k_semistoch<<<blocks, SEMI_THREADS, 0, s>>>(dinst, n_inst);
 }
 
 void launch_abs_hist(const DevInst *dinst, int par, int nb, int shift, u64 prefix, unsigned *hist, cudaStream_t s)
