@@ -1899,14 +1899,16 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         }
         if (!rc && changed) rc = rebuild();
     }
-    // restore the single-run state: no stop flag, own graph
+    // restore the single-run state: no stop flag; the run's own graph is
+    // captured again when it is next stepped alone (a run that lives in
+    // batches never needs it: 0.1 ms per run and call)
     for (int i = 0; i < k; i++) {
         fciqmc_handle *h = hs[i];
         if (read_state(h)) continue;
         h->hst.err &= ~ERRB_STOP;
         h->hst.stop_iter = LLONG_MAX;
         write_state(h);
-        capture_graph(h);
+        h->graph_gen = -1;
     }
     cleanup();
     dev_free(h0, dinst);
