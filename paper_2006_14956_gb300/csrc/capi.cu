@@ -2542,8 +2542,7 @@ extern "C" void fciqmc_free_system(fciqmc_system *sys)
 static int autotune_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t out[3])
 {
     if (!hs || k < 1 || n_iter < 1 || !out) return FCIQMC_ERR_INVALID_ARG;
-    // annihilation: 0 = the staged kernel (bulk copies one bucket ahead, two
-    // blocks per SM), else the plain-load kernel with that many blocks per SM
+    // annihilation: 0 = one resident wave, else that many blocks per SM
     const int spawn_c[] = {0, 1, 2, 4, 8, 16}, anni_c[] = {0, 3, 9, 24}, heavy_c[] = {1, 2, 4};
     int best_s = 1, best_h = 2, best_a = 0;
     double best = 1e300;

@@ -2200,12 +2200,10 @@ void launch_build_kidx(const DevInst *dinst, int parity, int nb, cudaStream_t s)
 }
 
 // launch geometry, chosen by fciqmc_autotune (grid blocks per SM; beyond the
-// resident count, here 4 per SM for the spawning kernel and 3 for the plain
-// annihilation kernel, the hardware hands the next block to whichever slot
-// frees first, which evens out buckets of unequal size)
-// g_spawn_bps = 0 and 1 select one resident wave of spawning blocks;
-// g_anni_bps = 0 selects the staged annihilation kernel (one resident wave,
-// bulk copies one bucket ahead) wherever the batch fits it
+// resident count, 4 per SM for the spawning kernel and 3 for the annihilation,
+// the hardware hands the next block to whichever slot frees first, which evens
+// out buckets of unequal size)
+// g_spawn_bps = 0 and 1 and g_anni_bps = 0 select one resident wave of blocks
 static int g_spawn_bps = 1, g_heavy_bps = 2, g_anni_bps = 0;
 static int g_geometry_gen = 0;  // changes with every set_launch_geometry
 int launch_geometry_generation() { return g_geometry_gen; }
