@@ -106,3 +106,31 @@ def test_crowded_buckets_bit_exact(max_dets):
     for g in gs:
         assert_states_equal(fq.fciqmc_export_state(g), o.export())
         assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
+
+
+@pytest.mark.parametrize("count", [2, 33, 70])
+def test_batch_deals_slices_and_crowded_buckets_of_all_runs(count):
+    """Runs with different numbers of heavy slices and crowded buckets (some
+    with none), fewer and more than a warp's 32 lanes: each equals its run alone."""
+    fq = _fq()
+    sysd = workloads.hubbard_1d(6, 1.0, 4.0)
+    s = oracle.system_from_workload(sysd)
+    a, b = np.array(s.determinants(), np.uint64).T
+    prm = dict(tau=0.01, target_walkers=1e9, shift_damping=0.5, shift_interval=5, initiator_threshold=3.0)
+    rng = np.random.default_rng(9)
+    runs = []
+    for i in range(count):
+        c = rng.normal(0.0, 1.0, a.size) * [1.0, 40.0, 600.0][i % 3]
+        runs.append((dict(prm, seed=100 + i, max_dets=[16, 4000][i % 2]), c))
+    gs = []
+    for p, c in runs + runs:
+        g = fq.fciqmc_create(sysd, p)
+        fq.fciqmc_import_state(g, a, b, c, 0, -2.0)
+        gs.append(g)
+    fq.fciqmc_step_batch(gs[:count], 3)
+    for g, h in zip(gs[:count], gs[count:]):
+        fq.fciqmc_step(h, 3)
+        assert_states_equal(fq.fciqmc_export_state(g), fq.fciqmc_export_state(h))
+        x, y = fq.fciqmc_iter_stats_get(g), fq.fciqmc_iter_stats_get(h)
+        for name in x:
+            np.testing.assert_array_equal(x[name], y[name], err_msg=name)
