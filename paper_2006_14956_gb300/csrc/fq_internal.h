@@ -117,6 +117,8 @@ struct IterState {
     alignas(128) int heavy_n;
     alignas(128) int big_n; // buckets deferred to the large-bucket kernel
     int done;               // blocks done with them (k_finish)
+    alignas(128) int claim_spawn;  // units claimed by warps that are through with those dealt to them, reset by
+    alignas(128) int claim_anni;   // the heavy-determinant kernel between spawning and annihilation
 };
 
 struct TrialEnt;

@@ -75,6 +75,7 @@ struct OneRun {
     const DevInst &I;
     __device__ __forceinline__ const DevInst &inst(int) const { return I; }
     __device__ __forceinline__ int find(int) const { return 0; }
+    __device__ __forceinline__ IterState *claims() const { return I.st; }
 };
 struct RunTable {
     static constexpr bool SINGLE = false;
@@ -83,7 +84,25 @@ struct RunTable {
     int n;
     __device__ __forceinline__ const DevInst &inst(int ii) const { return t[ii]; }
     __device__ __forceinline__ int find(int u) const { return find_inst(start, n, u); }
+    __device__ __forceinline__ IterState *claims() const { return t[0].st; }  // the first run counts for the launch
 };
+
+// How a launch's n units (buckets, or parts of them) come to its nw warps:
+// dealt out in turn, u = warp, warp + nw, ...  Over many rounds the warps drift
+// apart (heavily populated determinants, uneven buckets, SMs at different
+// distances from the data): with 27 rounds 14 % of the spawning's and 8 % of
+// the annihilation's warp time was idle at the end.  So from CLAIM_ROUNDS
+// rounds on (CLAIM kernels) the last quarter is claimed by whichever warp gets
+// there first.  50 orbitals, spawning and annihilation: 484 + 500 -> 447 +
+// 461 us at 7.7e6 determinants, 4.46 + 4.36 -> 4.17 + 4.18 ms at 7.6e7;
+// claiming the last half: 4.18 + 4.21 ms.  Below that it costs more than it
+// gives (3.4 rounds: 75 -> 78 us).
+constexpr int CLAIM_ROUNDS = 8;
+__host__ __device__ __forceinline__ int dealt_units(int n, int nw)
+{
+    const int rounds = n / nw;
+    return (rounds - rounds / 4) * nw;
+}
 
 struct AdaptQueue;
 // what the spawning code knows about the parent beyond its key: its
@@ -549,7 +568,7 @@ __device__ __noinline__ void queue_heavy(const DevInst &I, ulonglong2 kk, double
 // heavy_min attempts go to the heavy queue.  The loop holds every piece of
 // work once (code size): each turn evaluates a full window of attempts or of
 // singles, or else appends parents; a run's last turns empty what is left.
-template <int GEN, bool ADAPT, typename RUNS>
+template <int GEN, bool ADAPT, bool CLAIM, typename RUNS>
 __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int parts, unsigned heavy_min)
 {
     extern __shared__ __align__(16) unsigned char sp_raw[];
@@ -567,6 +586,8 @@ __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int pa
     unsigned long long att = 0;
     int cur = -1, err = 0;
     int v = gw, u = 0, ii = -1, b = 0, t = 0, m = 0;  // unit and part; next tile of bucket b
+    const int n_work = n_units * parts, dealt = CLAIM ? dealt_units(n_work, nw) : n_work;
+    int claim = 0;                                    // lane 0: the warp's next unit after the dealt ones
     bool have = false, drain = false;                 // v is set up (t, m valid); the run's list is done
     while (true) {
         if (ADAPT) {
@@ -587,8 +608,11 @@ __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int pa
         }
         // the next tile of this warp, in this run or another
         while (!have || t >= m) {
-            if (have) { v += nw; have = false; }
-            if (v >= n_units * parts) { ii = -1; break; }
+            if (have) {
+                v = !CLAIM || v + nw < dealt ? v + nw : dealt + __shfl_sync(0xffffffffu, claim, 0);
+                have = false;
+            }
+            if (v >= n_work) { ii = -1; break; }
             u = v / parts;
             ii = runs.find(u);
             if (ii != cur) break;
@@ -599,6 +623,7 @@ __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int pa
             } else {
                 m = t = 0;
             }
+            if (CLAIM && v + nw >= dealt && lane == 0) claim = atomicAdd(&runs.claims()->claim_spawn, 1);
             have = true;
         }
         const bool more = have && t < m;
@@ -684,19 +709,19 @@ __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int pa
     }
 }
 
-template <int GEN, bool ADAPT>
+template <int GEN, bool ADAPT, bool CLAIM>
 __global__ void __launch_bounds__(SP_THREADS, ADAPT ? 3 : 4) k_spawn(const __grid_constant__ DevInst I, int n_units,
                                                                      int parts, unsigned heavy_min)
 {
-    spawn_body<GEN, ADAPT>(OneRun{I}, n_units, parts, heavy_min);
+    spawn_body<GEN, ADAPT, CLAIM>(OneRun{I}, n_units, parts, heavy_min);
 }
 
-template <bool ADAPT>
+template <bool ADAPT, bool CLAIM>
 __global__ void __launch_bounds__(SP_THREADS, ADAPT ? 3 : 4) k_spawn_batch(const DevInst *__restrict__ insts,
                                                                         const int *__restrict__ unit_start, int n_inst,
                                                                         int n_units, int parts, unsigned heavy_min)
 {
-    spawn_body<GEN_ANY, ADAPT>(RunTable{insts, unit_start, n_inst}, n_units, parts, heavy_min);
+    spawn_body<GEN_ANY, ADAPT, CLAIM>(RunTable{insts, unit_start, n_inst}, n_units, parts, heavy_min);
 }
 
 // the slices of heavily populated determinants, one block each
@@ -709,6 +734,8 @@ __device__ __forceinline__ void heavy_body(const RUNS &runs, int n_inst)
     AdaptQueue *aq = reinterpret_cast<AdaptQueue *>(sp_raw + SP_WARPS * sizeof(SpawnWarp)) + warp;
     if (lane == 0) aq->n = 0;
     __syncwarp();
+    // between the spawning that claimed units and the annihilation that will
+    if (blockIdx.x == 0 && threadIdx.x == 0) runs.claims()->claim_spawn = runs.claims()->claim_anni = 0;
     // lane l looks at run i0 + l (a look costs an L2 round trip: 64 runs one
     // after the other took 100 us); only runs with work for this block follow.
     // The slices of all runs are dealt out in one sequence (`first` slices
@@ -1297,7 +1324,7 @@ __device__ __forceinline__ void anni_bucket_warp(const DevInst &I, AnniWarp &W, 
     }
 }
 
-template <bool EXTRA, typename RUNS>
+template <bool EXTRA, bool CLAIM, typename RUNS>
 __device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
 {
     extern __shared__ __align__(16) unsigned char an_raw[];
@@ -1310,7 +1337,10 @@ __device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
     int cur = -1, err = 0, par = 0, nq = 0, ne = 0;
     long long it = 0;
     double shift = 0.0;
-    for (int u = gw;; u += nw) {
+    const int dealt = CLAIM ? dealt_units(n_units, nw) : n_units;
+    int claim = 0;  // lane 0: the bucket after the next one, which is known already to be prefetched
+    auto after = [&](int x) { return x + nw < dealt ? x + nw : dealt + __shfl_sync(0xffffffffu, claim, 0); };
+    for (int u = gw, nx = gw + nw;; u = CLAIM ? nx : u + nw, nx = CLAIM ? after(nx) : nx) {
         const int ii = u < n_units ? runs.find(u) : -1;
         if (ii < 0 && cur < 0) return;  // a warp without buckets
         if (cur >= 0 && (nq >= 32 || (ii != cur && nq > 0))) new_diag(runs.inst(cur), W, nq, par ^ 1, pair, ii != cur);
@@ -1326,11 +1356,13 @@ __device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
             it = I.st->iter;
             shift = I.st->S;
         }
+        if (CLAIM && nx + nw >= dealt && lane == 0) claim = atomicAdd(&runs.claims()->claim_anni, 1);
         if (err) continue;
         const DevInst &I = runs.inst(cur);
         const int b = u - I.unit0;
         const int m = I.cnt[par][b], si = I.scnt_i[b], sn = I.scnt_n[b];
-        if (RUNS::SINGLE && u + nw < n_units) prefetch_bucket(I, b + nw, par);
+        const int next = CLAIM ? nx : u + nw;
+        if (RUNS::SINGLE && next < n_units) prefetch_bucket(I, next, par);
         if (si + sn > I.cap_s) {
             if (lane == 0) {
                 atomicOr(&I.st->err, ERRB_SPAWN_CAP);
@@ -1345,18 +1377,18 @@ __device__ __forceinline__ void anni_body(const RUNS &runs, int n_units)
     }
 }
 
-template <bool EXTRA>
+template <bool EXTRA, bool CLAIM>
 __global__ void __launch_bounds__(AN_THREADS, 3) k_annihilate(const __grid_constant__ DevInst I, int n_units)
 {
-    anni_body<EXTRA>(OneRun{I}, n_units);
+    anni_body<EXTRA, CLAIM>(OneRun{I}, n_units);
 }
 
-template <bool EXTRA>
+template <bool EXTRA, bool CLAIM>
 __global__ void __launch_bounds__(AN_THREADS, 3) k_annihilate_batch(const DevInst *__restrict__ insts,
                                                                             const int *__restrict__ unit_start,
                                                                             int n_inst, int n_units)
 {
-    anni_body<EXTRA>(RunTable{insts, unit_start, n_inst}, n_units);
+    anni_body<EXTRA, CLAIM>(RunTable{insts, unit_start, n_inst}, n_units);
 }
 
 // ------------------------------------------------------------------ large buckets
@@ -2263,13 +2295,19 @@ static SpawnSplit spawn_split(int n_units, int bps, bool alone)
     return p;
 }
 
+// whether the last units of a launch are claimed (with the adaptive shift and
+// with replica lists, whose kernels have no registers to spare, never)
+static bool claims(int n, int nw) { return n / nw >= CLAIM_ROUNDS; }
+
 // spawning of one run (`one`, the host image of its descriptor) or of a table
 // of runs (one = NULL); adaptive: some run uses the adaptive shift
 template <int GEN>
 static void launch_spawn_one(const DevInst *one, int grid, int n_units, int parts, unsigned heavy_min, cudaStream_t s)
 {
-    if (one->adaptive) k_spawn<GEN, true><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(*one, n_units, parts, heavy_min);
-    else k_spawn<GEN, false><<<grid, SP_THREADS, SP_SMEM, s>>>(*one, n_units, parts, heavy_min);
+    const bool claim = claims(n_units * parts, grid * SP_WARPS);
+    if (one->adaptive) k_spawn<GEN, true, false><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(*one, n_units, parts, heavy_min);
+    else if (claim) k_spawn<GEN, false, true><<<grid, SP_THREADS, SP_SMEM, s>>>(*one, n_units, parts, heavy_min);
+    else k_spawn<GEN, false, false><<<grid, SP_THREADS, SP_SMEM, s>>>(*one, n_units, parts, heavy_min);
 }
 void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s)
@@ -2280,8 +2318,9 @@ void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_star
     if (one && one->kind == FCIQMC_HUBBARD) launch_spawn_one<GEN_HOP>(one, grid, n_units, parts, heavy_min, s);
     else if (one && one->pchb) launch_spawn_one<GEN_PCHB>(one, grid, n_units, parts, heavy_min, s);
     else if (one) launch_spawn_one<GEN_UNIFORM>(one, grid, n_units, parts, heavy_min, s);
-    else if (adaptive) k_spawn_batch<true><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
-    else k_spawn_batch<false><<<grid, SP_THREADS, SP_SMEM, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
+    else if (adaptive) k_spawn_batch<true, false><<<grid, SP_THREADS, SP_SMEM_ADAPT, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
+    else if (claims(n_units * parts, grid * SP_WARPS)) k_spawn_batch<false, true><<<grid, SP_THREADS, SP_SMEM, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
+    else k_spawn_batch<false, false><<<grid, SP_THREADS, SP_SMEM, s>>>(dinst, unit_start, n_inst, n_units, parts, heavy_min);
 }
 
 void launch_spawn_heavy(const DevInst *one, const DevInst *dinst, int n_inst, cudaStream_t s)
@@ -2305,20 +2344,26 @@ cudaError_t init_kernels()
             e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      (int)((blocks * (bytes + 1024) * 100 + 233471) / 233472));
     };
-    warp_smem(k_spawn<GEN_UNIFORM, false>, SP_SMEM, 4);
-    warp_smem(k_spawn<GEN_PCHB, false>, SP_SMEM, 4);
-    warp_smem(k_spawn<GEN_HOP, false>, SP_SMEM, 4);
-    warp_smem(k_spawn_batch<false>, SP_SMEM, 4);
-    warp_smem(k_spawn<GEN_UNIFORM, true>, SP_SMEM_ADAPT, 3);
-    warp_smem(k_spawn<GEN_PCHB, true>, SP_SMEM_ADAPT, 3);
-    warp_smem(k_spawn<GEN_HOP, true>, SP_SMEM_ADAPT, 3);
-    warp_smem(k_spawn_batch<true>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_UNIFORM, false, false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_UNIFORM, false, true>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_PCHB, false, false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_PCHB, false, true>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_HOP, false, false>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_HOP, false, true>, SP_SMEM, 4);
+    warp_smem(k_spawn_batch<false, false>, SP_SMEM, 4);
+    warp_smem(k_spawn_batch<false, true>, SP_SMEM, 4);
+    warp_smem(k_spawn<GEN_UNIFORM, true, false>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_PCHB, true, false>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn<GEN_HOP, true, false>, SP_SMEM_ADAPT, 3);
+    warp_smem(k_spawn_batch<true, false>, SP_SMEM_ADAPT, 3);
     warp_smem(k_spawn_heavy, SP_SMEM_ADAPT, 3);
     warp_smem(k_spawn_heavy_batch, SP_SMEM_ADAPT, 3);
-    warp_smem(k_annihilate<false>, AN_SMEM, 3);
-    warp_smem(k_annihilate_batch<false>, AN_SMEM, 3);
-    warp_smem(k_annihilate<true>, AN_SMEM, 3);
-    warp_smem(k_annihilate_batch<true>, AN_SMEM, 3);
+    warp_smem(k_annihilate<false, false>, AN_SMEM, 3);
+    warp_smem(k_annihilate<false, true>, AN_SMEM, 3);
+    warp_smem(k_annihilate_batch<false, false>, AN_SMEM, 3);
+    warp_smem(k_annihilate_batch<false, true>, AN_SMEM, 3);
+    warp_smem(k_annihilate<true, false>, AN_SMEM, 3);
+    warp_smem(k_annihilate_batch<true, false>, AN_SMEM, 3);
     return e;
 }
 
@@ -2331,10 +2376,13 @@ cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const in
     const int bps = g_anni_bps > 0 ? g_anni_bps : 3;
     const int need = (n_units + AN_WARPS - 1) / AN_WARPS;
     const int grid = need < num_sms() * bps ? need : num_sms() * bps;
-    if (one && extra) k_annihilate<true><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
-    else if (one) k_annihilate<false><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
-    else if (extra) k_annihilate_batch<true><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
-    else k_annihilate_batch<false><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
+    const bool claim = claims(n_units, grid * AN_WARPS);
+    if (one && extra) k_annihilate<true, false><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
+    else if (one && claim) k_annihilate<false, true><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
+    else if (one) k_annihilate<false, false><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
+    else if (extra) k_annihilate_batch<true, false><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
+    else if (claim) k_annihilate_batch<false, true><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
+    else k_annihilate_batch<false, false><<<grid, AN_THREADS, AN_SMEM, s>>>(dinst, unit_start, n_inst, n_units);
     return cudaGetLastError();
 }
 
