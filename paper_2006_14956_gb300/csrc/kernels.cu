@@ -370,7 +370,7 @@ __device__ __forceinline__ int classify(const DevInst &I, u64 w0, u64 w1, unsign
 // There is no block barrier and an attempt never leaves the chip: at 7.3e7
 // determinants and 9.1e7 attempts (50 orbitals) a block-per-bucket draw with
 // 48-byte attempt records in global memory and a second kernel for the
-// evaluation took 8.6 ms; this takes 4.7 ms, issue slots 64 % used (the ten
+// evaluation took 8.6 ms; this takes 4.1 ms, issue slots 61 % used (the ten
 // Philox rounds' 32 x 32 products alone keep the heavy FMA pipe at 42 %).
 constexpr int SP_THREADS = 256, SP_WARPS = SP_THREADS / 32, RING = 64;
 constexpr int CHUNK_S = 512;  // attempts per slice of a heavily populated determinant
@@ -829,9 +829,9 @@ __device__ __forceinline__ int trial_find(const DevInst &I, u64 a, u64 b)
 // barriers per bucket, 128-bit shared accumulators, two blocks per SM) spent
 // 5.6 of 14 stall cycles per instruction at those barriers: 7.13 ms at 7.3e7
 // determinants and 3.5e7 spawns (50 orbitals), and 0.87 ms more for H_jj in a
-// kernel of its own; this takes 4.93 ms for both.  It is bound by instruction
-// fetch (the warps of an SM are at different places of a long code) and
-// latency, DRAM at 10 %.
+// kernel of its own; this takes 4.2 ms for both.  It is bound by instruction
+// issue (56 % of the slots; the warps of an SM are at different places of a
+// long code) and latency, DRAM at 17 %.
 constexpr int AN_THREADS = 256, AN_WARPS = AN_THREADS / 32;
 constexpr int AW_E = 192;          // records per warp (bytes of the table index them: below 255)
 constexpr int AW_TAB = 512;
