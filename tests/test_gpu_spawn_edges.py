@@ -134,3 +134,28 @@ def test_batch_deals_slices_and_crowded_buckets_of_all_runs(count):
         x, y = fq.fciqmc_iter_stats_get(g), fq.fciqmc_iter_stats_get(h)
         for name in x:
             np.testing.assert_array_equal(x[name], y[name], err_msg=name)
+
+
+@pytest.mark.parametrize("max_dets", [[16, 8000000], [8000000, 16, 4000000]])
+def test_batch_with_claimed_buckets(max_dets):
+    """Batches with so many buckets that both kernels claim the last of them
+    through the first run's counters, in a short or a long run: each run equals
+    the same run alone, twice over (the counters are cleared in between)."""
+    fq = _fq()
+    sysd = _abinitio(20, 4, 3, 8)
+    _, a, b, c = _list(sysd, 20, 700, 12)
+    prm = dict(tau=5e-4, target_walkers=1e9, shift_damping=0.5, shift_interval=5, initiator_threshold=3.0)
+    gs = []
+    for i, m in enumerate(max_dets + max_dets):
+        g = fq.fciqmc_create(sysd, dict(prm, seed=200 + i % len(max_dets), max_dets=m))
+        fq.fciqmc_import_state(g, a, b, c, 0, 0.1)
+        gs.append(g)
+    k = len(max_dets)
+    for _ in range(2):
+        fq.fciqmc_step_batch(gs[:k], 2)
+        for g, h in zip(gs[:k], gs[k:]):
+            fq.fciqmc_step(h, 2)
+            assert_states_equal(fq.fciqmc_export_state(g), fq.fciqmc_export_state(h))
+            x, y = fq.fciqmc_iter_stats_get(g), fq.fciqmc_iter_stats_get(h)
+            for name in x:
+                np.testing.assert_array_equal(x[name], y[name], err_msg=name)
