@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "fq_device.cuh"
+#include "warp_table.cuh"
 
 namespace fq {
 
@@ -824,8 +825,7 @@ __device__ __forceinline__ int trial_find(const DevInst &I, u64 a, u64 b)
 //      few enough that they are collected first.  Kept records go to the new
 //      bucket in order.  Sums are exact and rounded once, so no order matters.
 // New determinants wait in a queue of the warp for H_jj until there are 32.
-// The table needs no atomics: lanes claim a free slot by writing their record
-// and look who stayed.  A block of 256 threads per bucket of 1024 slots (three
+// The table needs no atomics (warp_table.cuh).  A block of 256 threads per bucket of 1024 slots (three
 // barriers per bucket, 128-bit shared accumulators, two blocks per SM) spent
 // 5.6 of 14 stall cycles per instruction at those barriers: 7.13 ms at 7.3e7
 // determinants and 3.5e7 spawns (50 orbitals), and 0.87 ms more for H_jj in a
@@ -1121,30 +1121,13 @@ __device__ __forceinline__ void anni_bucket_warp(const DevInst &I, AnniWarp &W, 
             W.val[e] = v;
         }
         __syncwarp();
-        unsigned s = (unsigned)det_hash(k.x, k.y) & tmask;
-        int target = -1;
-        bool open = on;
-        while (__any_sync(full, open)) {
-            unsigned x = AW_NONE;
-            if (open) {
-                x = W.tab[s];
-                if (x == AW_NONE) W.tab[s] = (unsigned char)e;
-            }
-            __syncwarp();
-            if (open) {
-                if (x == AW_NONE) x = W.tab[s];  // the claim that stayed
-                if ((int)x == e) { target = e; open = false; }
-                else {
-                    bool same = false;
-                    if (!walk) {  // walkers are distinct
-                        const ulonglong2 kk = W.key[x];
-                        same = kk.x == k.x && kk.y == k.y;
-                    }
-                    if (same) { target = (int)x; open = false; }
-                    else s = (s + 1) & tmask;
-                }
-            }
-        }
+        // (walkers are distinct: they are not compared)
+        const int target = warp_claim(W.tab, tmask, (unsigned)det_hash(k.x, k.y) & tmask, (unsigned char)e,
+                                      (unsigned char)AW_NONE, on, [&](unsigned char x) {
+                                          if (walk) return false;
+                                          const ulonglong2 kk = W.key[x];
+                                          return kk.x == k.x && kk.y == k.y;
+                                      });
         if (!walk && on) {
             const bool accepted = q < si || (target < m && !is_zero(W.val[target]));
             if (accepted || side) {
@@ -1285,24 +1268,13 @@ __device__ __forceinline__ void anni_bucket_warp(const DevInst &I, AnniWarp &W, 
         __syncwarp();
         for (int p0 = 0; p0 < total; p0 += 32) {
             const int p = p0 + lane;
-            bool open = p < total;
             unsigned s = 0;
-            if (open) {
+            if (p < total) {
                 const ulonglong2 k = I.key[np][base + p];
                 s = (unsigned)det_hash(k.x, k.y) & (unsigned)(KIDX - 1);
             }
-            while (__any_sync(full, open)) {
-                unsigned x = 1;
-                if (open) {
-                    x = kx[s];
-                    if (x == 0) kx[s] = (unsigned short)(p + 1);
-                }
-                __syncwarp();
-                if (open) {
-                    if (x == 0 && kx[s] == (unsigned short)(p + 1)) open = false;
-                    else s = (s + 1) & (unsigned)(KIDX - 1);
-                }
-            }
+            warp_claim(kx, (unsigned)(KIDX - 1), s, (unsigned short)(p + 1), (unsigned short)0, p < total,
+                       [](unsigned short) { return false; });
         }
         __syncwarp();
         for (int q = lane; q < KIDX; q += 32) I.kidx[np][(size_t)b * KIDX + q] = kx[q];
