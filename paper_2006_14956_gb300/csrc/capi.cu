@@ -15,6 +15,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "fq_internal.h"
@@ -108,7 +109,10 @@ static void *dev_alloc(fciqmc_handle *h, size_t bytes)
     if (h->p.max_device_bytes > 0 && h->bytes + bytes > (size_t)h->p.max_device_bytes) return nullptr;
     void *ptr = nullptr;
     if (h->p.alloc) ptr = h->p.alloc(bytes, h->p.alloc_ctx);
-    else if (cudaMalloc(&ptr, bytes) != cudaSuccess) ptr = nullptr;
+    else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+        ptr = nullptr;
+        cudaGetLastError();  // answered here: later calls ask for the last error of their launches
+    }
     if (ptr) {
         h->bufs.push_back({ptr, bytes});
         h->bytes += bytes;
@@ -224,58 +228,59 @@ static double pgen_class(const fciqmc_handle *h, int c)
 }
 
 // ------------------------------------------------------------------ layout
+static void free_layout(fciqmc_handle *h, DevInst &I)
+{
+    auto drop = [&](auto *&p) {
+        dev_free(h, p);
+        p = nullptr;
+    };
+    for (int k = 0; k < 2; k++) {
+        drop(I.key[k]); drop(I.c[k]); drop(I.hd[k]); drop(I.fl[k]); drop(I.cnt[k]); drop(I.facc[k]); drop(I.kidx[k]);
+    }
+    drop(I.skey); drop(I.sw); drop(I.scnt_i); drop(I.scnt_n); drop(I.part); drop(I.big_list); drop(I.newdet);
+}
+
+// buffers of 2^bb buckets for I, whose own ones (another descriptor may share
+// them) are left alone; on failure none is kept
 static int alloc_layout(fciqmc_handle *h, DevInst &I, int bb)
 {
     const size_t nbk = (size_t)1 << bb;
     const size_t nm = nbk * CAP_M, ns = nbk * (size_t)I.cap_s;
+    bool room = true, set = true;
+    auto take = [&](auto *&p, size_t n, bool zero) {
+        using T = std::remove_reference_t<decltype(*p)>;
+        p = room ? (T *)dev_alloc(h, n * sizeof(T)) : nullptr;
+        room = room && p;
+        if (p && zero) set = set && cudaMemsetAsync(p, 0, n * sizeof(T), h->stream) == cudaSuccess;
+    };
     for (int k = 0; k < 2; k++) {
-        I.key[k] = (ulonglong2 *)dev_alloc(h, nm * sizeof(ulonglong2));
-        I.c[k] = (double *)dev_alloc(h, nm * sizeof(double));
-        I.hd[k] = (double *)dev_alloc(h, nm * sizeof(double));
-        I.fl[k] = (uint8_t *)dev_alloc(h, nm);
-        I.cnt[k] = (int *)dev_alloc(h, nbk * sizeof(int));
-        if (!I.key[k] || !I.c[k] || !I.hd[k] || !I.fl[k] || !I.cnt[k]) return FCIQMC_ERR_OUT_OF_MEMORY;
-        if (cudaMemsetAsync(I.cnt[k], 0, nbk * sizeof(int), h->stream) != cudaSuccess) return FCIQMC_ERR_CUDA;
+        take(I.key[k], nm, false);
+        take(I.c[k], nm, false);
+        take(I.hd[k], nm, false);
+        take(I.fl[k], nm, false);
+        take(I.cnt[k], nbk, true);
     }
-    I.skey = (ulonglong2 *)dev_alloc(h, ns * sizeof(ulonglong2));
-    I.sw = (double *)dev_alloc(h, ns * sizeof(double));
-    I.scnt_i = (int *)dev_alloc(h, nbk * sizeof(int));
-    I.scnt_n = (int *)dev_alloc(h, nbk * sizeof(int));
-    I.part = (Partial *)dev_alloc(h, nbk * sizeof(Partial));
-    I.big_list = (int *)dev_alloc(h, nbk * sizeof(int));
-    I.newdet = (unsigned *)dev_alloc(h, nm * sizeof(unsigned));
-    if (!I.skey || !I.sw || !I.scnt_i || !I.scnt_n || !I.part || !I.big_list || !I.newdet) return FCIQMC_ERR_OUT_OF_MEMORY;
-    if (h->p.adaptive_shift)
-        for (int k = 0; k < 2; k++) {
-            I.facc[k] = (u64 *)dev_alloc(h, nm * 4 * sizeof(u64));
-            I.kidx[k] = (unsigned short *)dev_alloc(h, nbk * KIDX * sizeof(unsigned short));
-            if (!I.facc[k] || !I.kidx[k]) return FCIQMC_ERR_OUT_OF_MEMORY;
-            if (cudaMemsetAsync(I.kidx[k], 0, nbk * KIDX * sizeof(unsigned short), h->stream) != cudaSuccess ||
-                cudaMemsetAsync(I.facc[k], 0, nm * 4 * sizeof(u64), h->stream) != cudaSuccess)
-                return FCIQMC_ERR_CUDA;
-        }
-    cudaMemsetAsync(I.scnt_i, 0, nbk * sizeof(int), h->stream);
-    cudaMemsetAsync(I.scnt_n, 0, nbk * sizeof(int), h->stream);
-    cudaMemsetAsync(I.part, 0, nbk * sizeof(Partial), h->stream);
+    take(I.skey, ns, false);
+    take(I.sw, ns, false);
+    take(I.scnt_i, nbk, true);
+    take(I.scnt_n, nbk, true);
+    take(I.part, nbk, true);
+    take(I.big_list, nbk, false);
+    take(I.newdet, nm, false);
+    for (int k = 0; k < 2; k++) {
+        I.facc[k] = nullptr;
+        I.kidx[k] = nullptr;
+        if (!h->p.adaptive_shift) continue;
+        take(I.facc[k], nm * 4, true);
+        take(I.kidx[k], nbk * KIDX, true);
+    }
+    if (!room || !set) {
+        free_layout(h, I);
+        return room ? FCIQMC_ERR_CUDA : FCIQMC_ERR_OUT_OF_MEMORY;
+    }
     I.bb = bb;
     I.unit0 = 0;
     return FCIQMC_OK;
-}
-
-static void free_layout(fciqmc_handle *h, DevInst &I)
-{
-    for (int k = 0; k < 2; k++) {
-        dev_free(h, I.key[k]); dev_free(h, I.c[k]); dev_free(h, I.hd[k]); dev_free(h, I.fl[k]); dev_free(h, I.cnt[k]);
-        I.key[k] = nullptr; I.c[k] = nullptr; I.hd[k] = nullptr; I.fl[k] = nullptr; I.cnt[k] = nullptr;
-    }
-    dev_free(h, I.skey); dev_free(h, I.sw); dev_free(h, I.scnt_i); dev_free(h, I.scnt_n); dev_free(h, I.part);
-    dev_free(h, I.big_list); dev_free(h, I.newdet);
-    for (int k = 0; k < 2; k++) {
-        dev_free(h, I.facc[k]); dev_free(h, I.kidx[k]);
-        I.facc[k] = nullptr; I.kidx[k] = nullptr;
-    }
-    I.skey = nullptr; I.sw = nullptr; I.scnt_i = nullptr; I.scnt_n = nullptr; I.part = nullptr; I.big_list = nullptr;
-    I.newdet = nullptr;
 }
 
 static int upload_inst(fciqmc_handle *h)
@@ -371,7 +376,10 @@ static int grow_buckets(fciqmc_handle *h)
     int rc = alloc_layout(h, nI, h->bb + 1);
     if (rc) return fail(h, rc, "out of device memory while growing the walker buffers");
     DevInst *tmp = (DevInst *)dev_alloc(h, 2 * sizeof(DevInst));
-    if (!tmp) return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory");
+    if (!tmp) {
+        free_layout(h, nI);
+        return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory");
+    }
     CUDA_TRY(h, cudaMemcpyAsync(tmp, &h->hi, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(tmp + 1, &nI, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
     const int par = h->hst.parity;
@@ -407,7 +415,10 @@ static int grow_spawn_capacity(fciqmc_handle *h, long long need)
     size_t stride = (size_t)Ecap * (sizeof(ulonglong2) + sizeof(double) + 8 + 8 + 4 + 4 + 4) + ((size_t)4 << tabbits);
     stride = (stride + 255) & ~(size_t)255;
     unsigned char *scr = (unsigned char *)dev_alloc(h, stride * BIG_BLOCKS);
-    if (!nk || !nw || !scr) return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (spawn buffers)");
+    if (!nk || !nw || !scr) {
+        dev_free(h, nk); dev_free(h, nw); dev_free(h, scr);
+        return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (spawn buffers)");
+    }
     dev_free(h, I.skey); dev_free(h, I.sw); dev_free(h, I.big_scratch);
     I.skey = nk; I.sw = nw; I.cap_s = ncap;
     I.big_scratch = scr; I.big_stride = stride; I.big_tabbits = tabbits;
