@@ -55,7 +55,8 @@ struct fciqmc_handle {
     IterState *dstate = nullptr;
     cudaGraphExec_t graph = nullptr;
     int graph_kernels = 0;  // kernel nodes of the captured iteration
-    int graph_gen = -1;     // launch-configuration generation the graph was captured with
+    int graph_gen = -1;     // launch-configuration generation the graph was captured with (-1: none, capture again)
+    bool inst_stale = false;  // the device copy of `hi` is out of date
     bool profiling = false;
     double ktime[6] = {0, 0, 0, 0, 0, 0};  // spawn, heavy, annihilate, finalize, semistoch, new-determinant H_jj
     // layout
@@ -283,6 +284,15 @@ static int alloc_layout(fciqmc_handle *h, DevInst &I, int bb)
     return FCIQMC_OK;
 }
 
+// `hi` has changed: neither its device copy nor the graph, which holds it by
+// value, may be used until upload_inst and capture_graph have followed (an
+// error may lie between)
+static void inst_changed(fciqmc_handle *h)
+{
+    h->inst_stale = true;
+    h->graph_gen = -1;
+}
+
 static int upload_inst(fciqmc_handle *h)
 {
     CUDA_TRY(h, cudaMemcpyAsync(h->dinst, &h->hi, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
@@ -294,6 +304,7 @@ static int upload_inst(fciqmc_handle *h)
         h->kidx_dirty = false;
     }
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    h->inst_stale = false;
     return FCIQMC_OK;
 }
 
@@ -339,6 +350,7 @@ static int count_kernel_nodes(cudaGraph_t g)
 static int capture_graph(fciqmc_handle *h)
 {
     if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
+    h->graph_gen = -1;
     cudaGraph_t g;
     CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     int rc = enqueue_iteration(h, nullptr);
@@ -346,11 +358,20 @@ static int capture_graph(fciqmc_handle *h)
     if (rc) return rc;
     if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
     h->graph_kernels = count_kernel_nodes(g);
-    h->graph_gen = launch_geometry_generation();
     e = cudaGraphInstantiate(&h->graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(h, FCIQMC_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    h->graph_gen = launch_geometry_generation();
     return FCIQMC_OK;
+}
+
+// the device descriptor and the graph of the run as it is now: after a change
+// of the launch configuration, a batch, or a call that failed half-way
+static int make_current(fciqmc_handle *h)
+{
+    int rc = h->inst_stale ? upload_inst(h) : FCIQMC_OK;
+    if (!rc && (!h->graph || h->graph_gen != launch_geometry_generation())) rc = capture_graph(h);
+    return rc;
 }
 
 static int read_state(fciqmc_handle *h)
@@ -393,6 +414,7 @@ static int grow_buckets(fciqmc_handle *h)
     free_layout(h, h->hi);
     h->hi = nI;
     h->bb = nI.bb;
+    inst_changed(h);
     if (h->hst.err & ERRB_MAIN_CAP) return fail(h, FCIQMC_ERR_CAPACITY, "bucket overflow while splitting");
     return FCIQMC_OK;
 }
@@ -422,6 +444,7 @@ static int grow_spawn_capacity(fciqmc_handle *h, long long need)
     dev_free(h, I.skey); dev_free(h, I.sw); dev_free(h, I.big_scratch);
     I.skey = nk; I.sw = nw; I.cap_s = ncap;
     I.big_scratch = scr; I.big_stride = stride; I.big_tabbits = tabbits;
+    inst_changed(h);
     return FCIQMC_OK;
 }
 
@@ -434,6 +457,7 @@ static int ensure_side(fciqmc_handle *h)
     if (I.side && I.side_cap == cap && h->side_nbk == nbk) return FCIQMC_OK;
     dev_free(h, I.side);
     dev_free(h, I.side_cnt);
+    inst_changed(h);
     I.side = (SideEnt *)dev_alloc(h, (size_t)nbk * cap * sizeof(SideEnt));
     I.side_cnt = (int *)dev_alloc(h, (size_t)nbk * sizeof(int));
     if (!I.side || !I.side_cnt) return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (replica lists)");
@@ -452,6 +476,7 @@ static int grow_heavy(fciqmc_handle *h)
     h->hi.heavy = nh;
     h->hi.heavy_cap = ncap;
     h->heavy_cap = ncap;
+    inst_changed(h);
     return FCIQMC_OK;
 }
 
@@ -1201,10 +1226,8 @@ static int step_impl(fciqmc_handle *h, int64_t n_iter)
     }
     int rc = read_state(h);
     if (rc) return rc;
-    if (h->graph && h->graph_gen != launch_geometry_generation()) {  // the launch configuration changed
-        rc = capture_graph(h);
-        if (rc) return rc;
-    }
+    rc = make_current(h);
+    if (rc) return rc;
     return step_to(h, h->hst.iter + n_iter);
 }
 
@@ -1228,10 +1251,8 @@ static int step_async_impl(fciqmc_handle *h, int64_t n_iter)
         if (rc) return rc;
         h->async_base = h->hst.iter;
         h->async_target = h->hst.iter;
-        if (h->graph && h->graph_gen != launch_geometry_generation()) {  // the launch configuration changed
-            rc = capture_graph(h);
-            if (rc) return rc;
-        }
+        rc = make_current(h);
+        if (rc) return rc;
     }
     for (int64_t k = 0; k < n_iter; k++) CUDA_TRY(h, cudaGraphLaunch(h->graph, h->stream));
     h->async_target += n_iter;
@@ -1617,6 +1638,7 @@ static int import_device(fciqmc_handle *h, int64_t n, const uint64_t *alpha, con
         free_layout(h, h->hi);
         h->hi = nI;
         h->bb = nI.bb;
+        inst_changed(h);
     }
     const int par = 0;
     CUDA_TRY(h, cudaMemsetAsync(h->hi.cnt[par], 0, ((size_t)1 << h->bb) * sizeof(int), s));
@@ -1665,6 +1687,7 @@ static int import_host(fciqmc_handle *h, int64_t n, const uint64_t *alpha, const
         free_layout(h, h->hi);
         h->hi = nI;
         h->bb = nI.bb;
+        inst_changed(h);
     }
     const size_t nbk = (size_t)1 << h->bb, nm = nbk * CAP_M;
     std::vector<int> cnt_b(nbk, 0);
@@ -1782,6 +1805,10 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         if (rc) return rc;
         rc = read_state(h);
         if (rc) return rc;
+        if (h->inst_stale) {  // a call that failed half-way
+            rc = upload_inst(h);
+            if (rc) return rc;
+        }
         if (h->hst.err) {  // leftover flags (e.g. a pending semi-stochastic set-up)
             int retries = 0;
             rc = handle_flags(h, &retries);

@@ -11,8 +11,9 @@ pytestmark = pytest.mark.gpu
 
 
 def _determinants(norb, na, nb, n, seed):
+    """n distinct determinants, the reference (lowest orbitals) among them: an import adds it where it is absent."""
     rng = np.random.default_rng(seed)
-    key = set()
+    key = {((1 << na) - 1, (1 << nb) - 1)}
     while len(key) < n:
         for _ in range(n - len(key)):
             a = sum(1 << int(p) for p in rng.choice(norb, na, replace=False))
@@ -43,3 +44,46 @@ def test_import_that_does_not_fit_leaves_the_run_and_its_memory_alone(use_torch)
     o.step(20)
     assert_states_equal(fq.fciqmc_export_state(g), o.export())
     assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
+
+
+class _Refusing:
+    """PyTorch's allocator, answering NULL to requests of the sizes in `refuse`."""
+    refuse = ()
+
+    @classmethod
+    def install(cls, fq, monkeypatch):
+        base = fq._TorchAllocator
+
+        class Refusing(base):
+            def _alloc(self, nbytes, ctx):
+                return None if nbytes in cls.refuse else super()._alloc(nbytes, ctx)
+
+        monkeypatch.setattr(fq, "_TorchAllocator", Refusing)
+        monkeypatch.setattr(cls, "refuse", ())
+        return cls
+
+
+def test_a_step_after_a_call_that_failed_half_way_uses_the_buffers_of_now(monkeypatch):
+    """An import that has replaced the buckets and then finds no memory for
+    the selection of D fails; the run stands at the imported list."""
+    fq = _fq()
+    alloc = _Refusing.install(fq, monkeypatch)
+    sysd = workloads.small_abinitio(12, 4, 4, seed=9)
+    prm = dict(DAMP, tau=0.002, target_walkers=1e5, initiator_threshold=3.0, seed=22)
+    g = fq.fciqmc_create(sysd, dict(prm, max_dets=100, semistoch_size=50, semistoch_start=5))
+    fq.fciqmc_step(g, 2)
+    a, b = _determinants(12, 4, 4, 3000, 2)
+    c = np.random.default_rng(3).normal(0.0, 2.0, a.size)
+    shift = (5, 0.1, 1, 0, 0, sum(int(x) for x in np.floor(np.abs(c) * 2.0 ** 32)))
+    alloc.refuse = (65536 * 4,)  # the histogram of the selection
+    with pytest.raises(fq.FciqmcError) as e:
+        fq.fciqmc_import_state(g, a, b, c, *shift)
+    assert e.value.code == fq.FCIQMC_ERR_OUT_OF_MEMORY
+    alloc.refuse = ()
+    o = oracle.Run(oracle.system_from_workload(sysd), **prm)
+    o.import_state(a, b, c, *shift)
+    for step in (lambda: fq.fciqmc_step(g, 2), lambda: fq.fciqmc_step_batch([g], 2),
+                 lambda: (fq.fciqmc_step_async(g, 2), fq.fciqmc_sync(g))):
+        step()
+        o.step(2)
+        assert_states_equal(fq.fciqmc_export_state(g), o.export())
