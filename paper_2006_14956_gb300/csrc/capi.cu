@@ -84,6 +84,7 @@ struct fciqmc_handle {
     bool secondary = false;
     bool paired = false;
     int side_nbk = 0;
+    int split_refused = -1;  // bucket bits at which there was no memory for an early split
     // asynchronous stepping
     bool pending = false;
     long long async_base = 0, async_target = 0;
@@ -284,6 +285,15 @@ static int alloc_layout(fciqmc_handle *h, DevInst &I, int bb)
     return FCIQMC_OK;
 }
 
+// device bytes of a layout of 2^bb buckets (alloc_layout), with a replica's lists (ensure_side)
+static long long layout_bytes(const fciqmc_handle *h, int bb, int cap_s)
+{
+    long long per = 2LL * (CAP_M * (16 + 8 + 8 + 1) + 4) + cap_s * 24LL + 3 * 4 + (long long)sizeof(Partial) + CAP_M * 4LL;
+    if (h->p.adaptive_shift) per += 2LL * (CAP_M * 4 * 8 + KIDX * 2);
+    if (h->paired) per += (CAP_M + cap_s) * (long long)sizeof(SideEnt) + 4;
+    return per << bb;
+}
+
 // `hi` has changed: neither its device copy nor the graph, which holds it by
 // value, may be used until upload_inst and capture_graph have followed (an
 // error may lie between)
@@ -388,34 +398,120 @@ static int write_state(fciqmc_handle *h)
     return FCIQMC_OK;
 }
 
-// split every bucket in two (one more hash bit)
+// per-bucket determinant lists of a replica for the layout of I, whose own
+// ones are left alone; on failure none is kept
+static int alloc_side(fciqmc_handle *h, DevInst &I)
+{
+    const size_t nbk = (size_t)1 << I.bb;
+    I.side_cap = CAP_M + I.cap_s;
+    I.side = (SideEnt *)dev_alloc(h, nbk * I.side_cap * sizeof(SideEnt));
+    I.side_cnt = I.side ? (int *)dev_alloc(h, nbk * sizeof(int)) : nullptr;
+    if (I.side_cnt) return cudaMemsetAsync(I.side_cnt, 0, nbk * sizeof(int), h->stream) == cudaSuccess ? FCIQMC_OK
+                                                                                                     : FCIQMC_ERR_CUDA;
+    dev_free(h, I.side);
+    I.side = nullptr;
+    return FCIQMC_ERR_OUT_OF_MEMORY;
+}
+
+// A split of every bucket in two (one more hash bit): all its memory first
+// (side: a replica's lists as well), so that nothing of the run has changed
+// when there is none
+struct Split {
+    DevInst I{};
+    DevInst *table = nullptr;  // the old and the new descriptor on the device
+    bool side = false;
+};
+
+static void drop_split(fciqmc_handle *h, Split &s)
+{
+    free_layout(h, s.I);
+    if (s.side) {
+        dev_free(h, s.I.side);
+        dev_free(h, s.I.side_cnt);
+    }
+    dev_free(h, s.table);
+    s = Split();
+}
+
+static int prepare_split(fciqmc_handle *h, Split &s, bool side)
+{
+    s.I = h->hi;
+    if (s.I.cap_s > CAP_S0) s.I.cap_s /= 2;  // each new bucket receives about half the spawns
+    int rc = alloc_layout(h, s.I, h->bb + 1);
+    if (!rc && side && h->paired) {
+        s.side = true;
+        rc = alloc_side(h, s.I);
+    }
+    if (!rc && !(s.table = (DevInst *)dev_alloc(h, 2 * sizeof(DevInst)))) rc = FCIQMC_ERR_OUT_OF_MEMORY;
+    if (rc) drop_split(h, s);
+    return rc;
+}
+
+static int commit_split(fciqmc_handle *h, Split &s)
+{
+    CUDA_TRY(h, cudaMemcpyAsync(s.table, &h->hi, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(s.table + 1, &s.I, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
+    const int par = h->hst.parity;
+    launch_rebucket(s.table, s.table + 1, 1 << h->bb, par, h->stream);
+    if (h->p.adaptive_shift) launch_build_kidx(s.table + 1, par, 1 << s.I.bb, h->stream);
+    CUDA_TRY(h, cudaGetLastError());
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    int rc = read_state(h);
+    if (rc) return rc;
+    dev_free(h, s.table);
+    free_layout(h, h->hi);
+    if (s.side) {
+        dev_free(h, h->hi.side);
+        dev_free(h, h->hi.side_cnt);
+        h->side_nbk = 1 << s.I.bb;
+    }
+    h->hi = s.I;
+    h->bb = s.I.bb;
+    inst_changed(h);
+    if (h->hst.err & ERRB_MAIN_CAP) return fail(h, FCIQMC_ERR_CAPACITY, "bucket overflow while splitting");
+    return FCIQMC_OK;
+}
+
+// a split the run cannot do without
 static int grow_buckets(fciqmc_handle *h)
 {
     if (h->bb >= MAX_BB) return fail(h, FCIQMC_ERR_CAPACITY, "walker list exceeds 2^24 buckets");
-    DevInst nI = h->hi;
-    if (nI.cap_s > CAP_S0) nI.cap_s /= 2;  // each new bucket receives about half the spawns
-    int rc = alloc_layout(h, nI, h->bb + 1);
+    Split s;
+    const int rc = prepare_split(h, s, false);
     if (rc) return fail(h, rc, "out of device memory while growing the walker buffers");
-    DevInst *tmp = (DevInst *)dev_alloc(h, 2 * sizeof(DevInst));
-    if (!tmp) {
-        free_layout(h, nI);
-        return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory");
+    return commit_split(h, s);
+}
+
+// A split that only saves time, of a run and of its replica partner, which
+// keeps the same layout.  Without the memory for both it is left out, and
+// under a memory limit it also leaves room for the next doubling, one that
+// the run may not be able to do without.
+static int split_early(fciqmc_handle *h, bool *done)
+{
+    *done = false;
+    fciqmc_handle *g[2] = {h, h->partner};
+    Split s[2];
+    for (fciqmc_handle *x : g) {
+        if (!x) continue;
+        if (x->split_refused == x->bb) return FCIQMC_OK;
+        const long long next = layout_bytes(x, x->bb + 1, x->hi.cap_s), after = layout_bytes(x, x->bb + 2, x->hi.cap_s);
+        if (x->p.max_device_bytes > 0 &&
+            (long long)x->bytes - layout_bytes(x, x->bb, x->hi.cap_s) + next + after > x->p.max_device_bytes)
+            return FCIQMC_OK;
     }
-    CUDA_TRY(h, cudaMemcpyAsync(tmp, &h->hi, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(h, cudaMemcpyAsync(tmp + 1, &nI, sizeof(DevInst), cudaMemcpyHostToDevice, h->stream));
-    const int par = h->hst.parity;
-    launch_rebucket(tmp, tmp + 1, 1 << h->bb, par, h->stream);
-    if (h->p.adaptive_shift) launch_build_kidx(tmp + 1, par, 1 << nI.bb, h->stream);
-    CUDA_TRY(h, cudaGetLastError());
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    int rc2 = read_state(h);
-    if (rc2) return rc2;
-    dev_free(h, tmp);
-    free_layout(h, h->hi);
-    h->hi = nI;
-    h->bb = nI.bb;
-    inst_changed(h);
-    if (h->hst.err & ERRB_MAIN_CAP) return fail(h, FCIQMC_ERR_CAPACITY, "bucket overflow while splitting");
+    for (int k = 0; k < 2; k++) {
+        if (!g[k]) continue;
+        const int rc = prepare_split(g[k], s[k], true);
+        if (!rc) continue;
+        if (k) drop_split(g[0], s[0]);
+        h->split_refused = h->bb;  // not tried again before the layout changes
+        return rc == FCIQMC_ERR_OUT_OF_MEMORY ? FCIQMC_OK : fail(h, rc, "splitting the buckets");
+    }
+    for (int k = 0; k < 2; k++) {
+        const int rc = g[k] ? commit_split(g[k], s[k]) : FCIQMC_OK;
+        if (rc) return rc;
+    }
+    *done = true;
     return FCIQMC_OK;
 }
 
@@ -458,11 +554,8 @@ static int ensure_side(fciqmc_handle *h)
     dev_free(h, I.side);
     dev_free(h, I.side_cnt);
     inst_changed(h);
-    I.side = (SideEnt *)dev_alloc(h, (size_t)nbk * cap * sizeof(SideEnt));
-    I.side_cnt = (int *)dev_alloc(h, (size_t)nbk * sizeof(int));
-    if (!I.side || !I.side_cnt) return fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (replica lists)");
-    CUDA_TRY(h, cudaMemsetAsync(I.side_cnt, 0, (size_t)nbk * sizeof(int), h->stream));
-    I.side_cap = cap;
+    const int rc = alloc_side(h, I);
+    if (rc) return fail(h, rc, "out of device memory (replica lists)");
     h->side_nbk = nbk;
     return FCIQMC_OK;
 }
@@ -1299,22 +1392,19 @@ int fciqmc_sync(fciqmc_handle *h)
 
 void *fciqmc_stream(fciqmc_handle *h) { return h ? (void *)h->stream : nullptr; }
 
-// Whether the run's buckets should be split before they overflow: the average
-// occupancy passes FILL_M, or determinants and spawns together pass what most
-// warps of the annihilation hold (buckets beyond that go to a block each,
-// several times slower) while there are more determinants than buckets.  The
-// second kind, the only one in a batch, is skipped where the memory limit has
-// no room for it.
-constexpr int FILL_E = 160, FILL_MIN = 1;
-static bool crowded(const fciqmc_handle *h, bool optional)
+// Whether the run's buckets had better be split before they overflow: the
+// average occupancy passes FILL_M (not in a batch), or determinants and spawns
+// together pass what most warps of the annihilation hold (buckets beyond that
+// go to a block each, several times slower) while there are at least two
+// determinants to a bucket.
+constexpr int FILL_E = 160;
+static bool crowded(const fciqmc_handle *h, bool batch)
 {
-    if (h->hst.err || h->hist.empty() || h->bb >= MAX_BB) return false;
+    if ((h->hst.err & ~ERRB_STOP) || h->hist.empty() || h->bb >= MAX_BB) return false;
     const fciqmc_iter_stats &r = h->hist.back();
     const long long nbk = 1LL << h->bb;
-    if (!optional && r.ndet > nbk * FILL_M) return true;
-    if (r.ndet + r.spawns <= nbk * FILL_E || r.ndet < 2 * FILL_MIN * nbk) return false;
-    const long long layout = 2 * nbk * (2LL * CAP_M * 33 + (long long)h->hi.cap_s * 24 + 4LL * CAP_M + 128);
-    return h->p.max_device_bytes <= 0 || (long long)h->bytes + layout + (layout >> 4) < h->p.max_device_bytes;
+    if (!batch && r.ndet > nbk * FILL_M) return true;
+    return r.ndet + r.spawns > nbk * FILL_E && r.ndet >= 2 * nbk;
 }
 
 // Runs iterations until target_iter, in chunks of graph replays; after each
@@ -1368,9 +1458,12 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         }
         rc = pull_history(h, start, h->hst.iter);
         if (rc) return rc;
-        if (crowded(h, false)) {
-            rc = grow_buckets(h);
+        bool split = crowded(h, false);
+        if (split) {
+            rc = split_early(h, &split);
             if (rc) return rc;
+        }
+        if (split) {
             rc = reset_after_error(h);
             if (rc) return rc;
             rc = upload_inst(h);
@@ -1915,21 +2008,17 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         for (int i = 0; i < k && !rc; i++) {
             fciqmc_handle *h = hs[i], *pt = h->partner;
             if ((h->hst.err & ~ERRB_STOP) || (pt && (h->secondary || (pt->hst.err & ~ERRB_STOP)))) continue;
-            const int stop = h->hst.err;
-            h->hst.err = 0;
-            const bool split = crowded(h, true) || (pt && crowded(pt, true));
-            h->hst.err = stop;
+            bool split = crowded(h, true) || (pt && crowded(pt, true));
             if (!split) continue;
+            const int keep[2] = {h->hst.err, pt ? pt->hst.err : 0};
+            rc = split_early(h, &split);
+            if (rc) h->step_rc = rc;
+            if (rc || !split) continue;
             for (fciqmc_handle *g : {h, pt}) {
                 if (!g || rc) continue;
-                const int keep = g->hst.err;
-                const long long si = g->hst.stop_iter;
-                rc = grow_buckets(g);
-                if (!rc) rc = reset_after_error(g);
-                g->hst.err = keep;
-                g->hst.stop_iter = si;
+                rc = reset_after_error(g);
+                g->hst.err = keep[g == pt];
                 if (!rc) rc = write_state(g);
-                if (!rc) rc = ensure_side(g);
                 if (!rc) rc = upload_inst(g);
                 if (rc) g->step_rc = rc;
             }

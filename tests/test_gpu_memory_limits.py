@@ -47,8 +47,9 @@ def test_import_that_does_not_fit_leaves_the_run_and_its_memory_alone(use_torch)
 
 
 class _Refusing:
-    """PyTorch's allocator, answering NULL to requests of the sizes in `refuse`."""
+    """PyTorch's allocator, answering NULL to requests of the sizes in `refuse` after the first `skip` of them."""
     refuse = ()
+    skip = 0
 
     @classmethod
     def install(cls, fq, monkeypatch):
@@ -56,10 +57,12 @@ class _Refusing:
 
         class Refusing(base):
             def _alloc(self, nbytes, ctx):
-                return None if nbytes in cls.refuse else super()._alloc(nbytes, ctx)
+                cls.skip -= nbytes in cls.refuse
+                return None if nbytes in cls.refuse and cls.skip < 0 else super()._alloc(nbytes, ctx)
 
         monkeypatch.setattr(fq, "_TorchAllocator", Refusing)
         monkeypatch.setattr(cls, "refuse", ())
+        monkeypatch.setattr(cls, "skip", 0)
         return cls
 
 
@@ -87,3 +90,53 @@ def test_a_step_after_a_call_that_failed_half_way_uses_the_buffers_of_now(monkey
         step()
         o.step(2)
         assert_states_equal(fq.fciqmc_export_state(g), o.export())
+
+
+EARLY = {"alone": dict(), "plain": dict(), "adaptive": dict(adaptive_shift=1), "pair": dict(replicas=2)}
+
+
+@pytest.mark.parametrize("kind", sorted(EARLY))
+def test_early_split_that_does_not_fit_is_left_out(monkeypatch, kind):
+    """Buckets that hold more walkers and spawns than a warp annihilates (in a
+    run alone also those that are half full) are split to save time.  Where the
+    memory for that is missing (any limit from the run's own bytes to several
+    splits; an allocator that refuses a run or one replica of a pair), the run
+    finishes on what it has."""
+    fq = _fq()
+    alloc = _Refusing.install(fq, monkeypatch)
+    sysd = dict(workloads.hubbard_1d(8, 1.0, 4.0), n_beta=3, ref=(0x55, 0x2a))
+    s = oracle.system_from_workload(sysd)
+    a, b = (x.copy() for x in np.array(s.determinants(), np.uint64).T)
+    c = 4.5 * np.random.default_rng(4).choice([-1.0, 1.0], a.size)  # 122 walkers and 45 spawns to a bucket, evenly
+    prm = dict(DAMP, tau=0.01, target_walkers=1e9, initiator_threshold=3.0, seed=31, max_dets=4000, **EARLY[kind])
+    o = oracle.Run(s, **{k: v for k, v in prm.items() if k not in ("max_dets", "replicas")})
+    o.import_state(a, b, c, 0, 4.0)
+    o.step(20)
+
+    def run(limit, refuse=(), skip=0):
+        g = fq.fciqmc_create(sysd, dict(prm, max_device_bytes=limit))
+        both = [g] if kind != "pair" else [g, fq.fciqmc_replica(g, 1)]
+        for r in both:
+            fq.fciqmc_import_state(r, a, b, c, 0, 4.0)
+        first = fq.fciqmc_layout(g)
+        alloc.refuse, alloc.skip = refuse, skip
+        for _ in range(5):
+            if kind == "alone":
+                fq.fciqmc_step(g, 4)
+            else:
+                fq.fciqmc_step_batch(both, 4)
+        alloc.refuse = ()
+        assert_states_equal(fq.fciqmc_export_state(g), o.export())
+        last = [fq.fciqmc_layout(r) for r in both]
+        assert all(x == last[0] for x in last)
+        assert last[0]["cap_spawn"] == first["cap_spawn"]  # no growth that the run could not do without
+        return first, last[0]
+
+    first, last = run(0)
+    assert first["buckets"] == 32 and last["buckets"] > 32
+    keys = 2 * first["buckets"] * first["cap_main"] * 16  # bytes of a key array of the split layout, two of them to a run
+    for skip in (0, 2) if kind == "pair" else (0,):
+        assert run(0, (keys,), skip) == (first, first)
+    for more in np.linspace(16 << 10, 6 << 20, 13).astype(int):
+        limit = first["device_bytes"] + int(more)
+        assert run(limit)[1]["device_bytes"] <= limit
