@@ -1870,6 +1870,17 @@ int fciqmc_import_state(fciqmc_handle *h, int64_t n, const uint64_t *alpha, cons
 
 int64_t fciqmc_iter_stats_count(fciqmc_handle *h) { return h ? (int64_t)h->hist.size() : -1; }
 
+// A replica whose growth failed half-way has fewer buckets than its partner or
+// no lists: the join would read lists that are not there, or report zeros
+static int make_pair_whole(fciqmc_handle *h)
+{
+    int rc = FCIQMC_OK;
+    while (!rc && h->partner && h->bb < h->partner->bb) rc = grow_buckets(h);
+    if (!rc) rc = ensure_side(h);
+    if (!rc && h->inst_stale) rc = upload_inst(h);
+    return rc;
+}
+
 // Many runs per launch: one descriptor table covering the buckets of all
 // runs, one captured iteration graph; each run stops at its own target via
 // the stop iteration, and capacity flags are handled run by run.
@@ -1909,6 +1920,10 @@ static int step_batch_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter)
         }
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
         target[i] = h->hst.iter + n_iter;
+    }
+    for (int i = 0; i < k; i++) {
+        const int rc = make_pair_whole(hs[i]);
+        if (rc) return rc;
     }
     DevInst *dinst = (DevInst *)dev_alloc(h0, (size_t)k * sizeof(DevInst));
     int *dunit = (int *)dev_alloc(h0, (size_t)(k + 1) * sizeof(int));

@@ -140,3 +140,36 @@ def test_early_split_that_does_not_fit_is_left_out(monkeypatch, kind):
     for more in np.linspace(16 << 10, 6 << 20, 13).astype(int):
         limit = first["device_bytes"] + int(more)
         assert run(limit)[1]["device_bytes"] <= limit
+
+
+@pytest.mark.parametrize("refused", ["partner_split", "first_lists", "second_lists"])
+def test_pair_goes_on_whole_after_a_growth_that_failed_half_way(monkeypatch, refused):
+    """The first replica's first iteration needs more buckets, and the second
+    follows.  The allocator refuses them to the second replica, or the lists of the join to one of the two: the call
+    fails, and the next one, with memory, gives what the oracle's pair gives,
+    cross estimators included."""
+    from tests.test_gpu_replicas import check_pair
+    fq = _fq()
+    alloc = _Refusing.install(fq, monkeypatch)
+    sysd = dict(workloads.hubbard_1d(8, 1.0, 4.0), n_beta=3, ref=(0x55, 0x2a))
+    s = oracle.system_from_workload(sysd)
+    a, b = (x.copy() for x in np.array(s.determinants(), np.uint64).T)
+    c = 9.0 * np.random.default_rng(5).choice([-1.0, 1.0], a.size)  # 97 spawns to each of 32 buckets
+    prm = dict(DAMP, tau=0.01, target_walkers=1e9, initiator_threshold=3.0, seed=33)
+    g = fq.fciqmc_create(sysd, dict(prm, max_dets=4000, replicas=2))
+    pair = oracle.Pair(s, **prm)
+    for r in (0, 1):
+        fq.fciqmc_import_state(fq.fciqmc_replica(g, r), a, b, c / (1 + 4 * r), 0, 4.0)
+        pair.r[r].import_state(a, b, c / (1 + 4 * r), 0, 4.0)
+    lay = fq.fciqmc_layout(g)
+    assert (lay["buckets"], lay["cap_spawn"]) == (32, 96)
+    keys, lists = 64 * lay["cap_main"] * 16, 64 * (lay["cap_main"] + lay["cap_spawn"]) * 48
+    alloc.refuse = (keys,) if refused == "partner_split" else (lists,)
+    alloc.skip = {"partner_split": 2, "first_lists": 0, "second_lists": 1}[refused]
+    with pytest.raises(fq.FciqmcError) as e:
+        fq.fciqmc_step(g, 24)
+    assert e.value.code == fq.FCIQMC_ERR_OUT_OF_MEMORY
+    alloc.refuse = ()
+    fq.fciqmc_step(g, 24 - fq.fciqmc_export_shift(g)["iteration"])
+    pair.step(24)
+    check_pair(fq, g, pair)
