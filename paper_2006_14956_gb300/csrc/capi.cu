@@ -135,14 +135,16 @@ static void dev_free(fciqmc_handle *h, void *ptr)
     else cudaFree(ptr);
 }
 
-// Bucket bits of a list of `dets` determinants: START_M per bucket where the
-// list is as long as expected; a short one gets more, smaller buckets (up to
+// Bucket bits of a list of `dets` determinants: at most START_M per bucket
+// where the list is as long as expected, so 1.2 to 2.4 slots per determinant
+// (with 140 per bucket up to 2.7: a list of 1e7 took 2.1 GB where 1.0 do).
+// With `spread` a short one gets more, smaller buckets (up to
 // SMALL_BB, down to SMALL_M per bucket), so that its warps take one round of
 // 32 records each instead of three or four, one after the other.  At 2^8, 2^9,
 // 2^10, 2^11, 2^12 a 4x4 lattice at 1e5 walkers takes 54, 54, 49, 51, 54 us an
 // iteration, a batch of 64 lattice runs of 1e4 to 1e6 walkers 1.59, 1.61, 1.65,
 // 1.73, 1.92 ms.
-constexpr double START_M = 140.0, SMALL_M = 24.0;
+constexpr double START_M = 160.0, SMALL_M = 24.0;
 constexpr int SMALL_BB = 10;
 constexpr double BUCKET_BYTES = 2.0 * CAP_M * 33 + CAP_S0 * 24.0 + 4.0 * CAP_M + 128;  // of device memory
 static int start_bits(double dets, bool spread)
@@ -1149,12 +1151,14 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
         for (int k = 0; k < h->nb; k++) fci *= (double)(N - k) / (double)(k + 1);
         if (P.max_dets <= 0) dets_hint = std::min(dets_hint, std::max(1.0, fci));
     }
-    // a given max_dets is kept to, and a memory limit that leaves little room
+    // not spread: a list of a stated length (max_dets; it is still split when
+    // crowded), and where the memory limit or the allocator leaves little room
+    const int tight = start_bits(dets_hint, false);
     int bb = start_bits(dets_hint, P.max_dets <= 0);
-    if (P.max_device_bytes > 0 && 8.0 * (double)(1LL << bb) * BUCKET_BYTES > (double)P.max_device_bytes)
-        bb = start_bits(dets_hint, false);
+    if (P.max_device_bytes > 0 && 8.0 * (double)(1LL << bb) * BUCKET_BYTES > (double)P.max_device_bytes) bb = tight;
     I.cap_s = CAP_S0;
     int rc = alloc_layout(h, I, bb);
+    if (rc == FCIQMC_ERR_OUT_OF_MEMORY && bb > tight) rc = alloc_layout(h, I, bb = tight);
     if (rc) return bail(rc, "out of device memory (walker buffers)");
     h->bb = bb;
     h->heavy_cap = std::max(4096, (int)std::min(1e6, 4.0 * P.target_walkers / HEAVY_ATT));

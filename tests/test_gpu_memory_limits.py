@@ -173,3 +173,22 @@ def test_pair_goes_on_whole_after_a_growth_that_failed_half_way(monkeypatch, ref
     fq.fciqmc_step(g, 24 - fq.fciqmc_export_shift(g)["iteration"])
     pair.step(24)
     check_pair(fq, g, pair)
+
+
+@pytest.mark.parametrize("dets", [145, 145 << 6, 155 << 10, 160 << 11, 161 << 11])
+def test_a_list_of_a_stated_length_gets_few_slots_per_determinant(dets):
+    """At most 160 determinants to a bucket of 192 slots, in a power of two of buckets: below 2.4 slots each."""
+    fq = _fq()
+    lay = fq.fciqmc_layout(fq.fciqmc_create(workloads.small_abinitio(12, 4, 4, seed=9), dict(tau=0.002, max_dets=dets)))
+    assert dets / 160 <= lay["buckets"] < dets / 80 + 1
+
+
+def test_create_without_room_for_spread_buckets_takes_fewer(monkeypatch):
+    fq = _fq()
+    alloc = _Refusing.install(fq, monkeypatch)
+    sysd = workloads.small_abinitio(12, 4, 4, seed=9)
+    prm = dict(tau=0.002, target_walkers=1e4)
+    lay = fq.fciqmc_layout(fq.fciqmc_create(sysd, prm))
+    alloc.refuse = (lay["buckets"] * lay["cap_main"] * 16,)
+    few = fq.fciqmc_layout(fq.fciqmc_create(sysd, prm))
+    assert few["buckets"] < lay["buckets"] and few["device_bytes"] < lay["device_bytes"]
