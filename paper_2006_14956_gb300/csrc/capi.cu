@@ -146,13 +146,25 @@ static void dev_free(fciqmc_handle *h, void *ptr)
 // 1.73, 1.92 ms.
 constexpr double START_M = 160.0, SMALL_M = 24.0;
 constexpr int SMALL_BB = 10;
-constexpr double BUCKET_BYTES = 2.0 * CAP_M * 33 + CAP_S0 * 24.0 + 4.0 * CAP_M + 128;  // of device memory
 static int start_bits(double dets, bool spread)
 {
     int bb = 0;
     while ((double)(1LL << bb) * START_M < dets && bb < MAX_BB) bb++;
     while (spread && bb < SMALL_BB && (double)(1LL << bb) * SMALL_M < dets) bb++;
     return bb;
+}
+
+// the list length a run is laid out for (capped: buffers grow on demand), before
+// the size of its space is looked at
+static double expected_dets(const fciqmc_params &P)
+{
+    return P.max_dets > 0 ? (double)P.max_dets : std::min(std::max(4096.0, P.target_walkers), 8388608.0);
+}
+
+// slices its queue of heavily populated determinants holds at first
+static int heavy_slices(const fciqmc_params &P)
+{
+    return std::max(4096, (int)std::min(1e6, 4.0 * P.target_walkers / HEAVY_ATT));
 }
 
 static int64_t pair_index(int64_t i, int64_t j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; }
@@ -288,11 +300,11 @@ static int alloc_layout(fciqmc_handle *h, DevInst &I, int bb)
 }
 
 // device bytes of a layout of 2^bb buckets (alloc_layout), with a replica's lists (ensure_side)
-static long long layout_bytes(const fciqmc_handle *h, int bb, int cap_s)
+static long long layout_bytes(const fciqmc_params &P, bool paired, int bb, int cap_s)
 {
     long long per = 2LL * (CAP_M * (16 + 8 + 8 + 1) + 4) + cap_s * 24LL + 3 * 4 + (long long)sizeof(Partial) + CAP_M * 4LL;
-    if (h->p.adaptive_shift) per += 2LL * (CAP_M * 4 * 8 + KIDX * 2);
-    if (h->paired) per += (CAP_M + cap_s) * (long long)sizeof(SideEnt) + 4;
+    if (P.adaptive_shift) per += 2LL * (CAP_M * 4 * 8 + KIDX * 2);
+    if (paired) per += (CAP_M + cap_s) * (long long)sizeof(SideEnt) + 4;
     return per << bb;
 }
 
@@ -496,9 +508,9 @@ static int split_early(fciqmc_handle *h, bool *done)
     for (fciqmc_handle *x : g) {
         if (!x) continue;
         if (x->split_refused == x->bb) return FCIQMC_OK;
-        const long long next = layout_bytes(x, x->bb + 1, x->hi.cap_s), after = layout_bytes(x, x->bb + 2, x->hi.cap_s);
+        auto bytes = [&](int bb) { return layout_bytes(x->p, x->paired, bb, x->hi.cap_s); };
         if (x->p.max_device_bytes > 0 &&
-            (long long)x->bytes - layout_bytes(x, x->bb, x->hi.cap_s) + next + after > x->p.max_device_bytes)
+            (long long)x->bytes - bytes(x->bb) + bytes(x->bb + 1) + bytes(x->bb + 2) > x->p.max_device_bytes)
             return FCIQMC_OK;
     }
     for (int k = 0; k < 2; k++) {
@@ -1144,7 +1156,7 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
 
     // bucket layout: average occupancy well below the per-bucket capacity
     // start at the expected size (capped: buffers grow on demand)
-    double dets_hint = P.max_dets > 0 ? (double)P.max_dets : std::min(std::max(4096.0, P.target_walkers), 8388608.0);
+    double dets_hint = expected_dets(P);
     {
         double fci = 1.0;  // C(N, n_alpha) C(N, n_beta)
         for (int k = 0; k < h->na; k++) fci *= (double)(N - k) / (double)(k + 1);
@@ -1155,13 +1167,13 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     // crowded), and where the memory limit or the allocator leaves little room
     const int tight = start_bits(dets_hint, false);
     int bb = start_bits(dets_hint, P.max_dets <= 0);
-    if (P.max_device_bytes > 0 && 8.0 * (double)(1LL << bb) * BUCKET_BYTES > (double)P.max_device_bytes) bb = tight;
+    if (P.max_device_bytes > 0 && 8 * layout_bytes(P, P.replicas == 2, bb, CAP_S0) > P.max_device_bytes) bb = tight;
     I.cap_s = CAP_S0;
     int rc = alloc_layout(h, I, bb);
     if (rc == FCIQMC_ERR_OUT_OF_MEMORY && bb > tight) rc = alloc_layout(h, I, bb = tight);
     if (rc) return bail(rc, "out of device memory (walker buffers)");
     h->bb = bb;
-    h->heavy_cap = std::max(4096, (int)std::min(1e6, 4.0 * P.target_walkers / HEAVY_ATT));
+    h->heavy_cap = heavy_slices(P);
     I.heavy = (HeavyChunk *)dev_alloc(h, (size_t)h->heavy_cap * sizeof(HeavyChunk));
     I.heavy_cap = h->heavy_cap;
     if (!I.heavy) return bail(FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (heavy queue)");
@@ -2359,23 +2371,26 @@ struct fciqmc_server {
     double now() const { return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count(); }
 };
 
-// device memory a request needs when admitted: its initial layout and
-// integrals, and the first growth of the spawn regions (to 4 CAP_S0 slots per
-// bucket, old and new buffers held together, with the large-bucket scratch)
+// device memory a request needs when admitted: what fciqmc_create allocates
+// for it (the layout chosen there, or a larger one: for a list half as long
+// again, and in a small space), and the first growth of the spawn regions (to
+// 4 CAP_S0 slots per bucket, old and new buffers held together, with the
+// large-bucket scratch)
 static int64_t estimate_bytes(const Request &r)
 {
-    const int N = r.sys.kind == FCIQMC_HUBBARD ? r.sys.lx * r.sys.ly : r.sys.norb;
-    const double np = (double)N * (N + 1) / 2, ne = np * (np + 1) / 2;
-    double dets = r.p.max_dets > 0 ? (double)r.p.max_dets : std::min(std::max(4096.0, r.p.target_walkers), 8388608.0);
-    const int bb = start_bits(dets / 0.64, false);
-    const double per_bucket = 2.0 * CAP_M * (16 + 8 + 8 + 1) + 5.0 * CAP_S0 * 24.0 + 2 * 8 + sizeof(Partial) + 3 * 4 +
-                              4.0 * CAP_M;
-    const double ecap = CAP_M + 4.0 * CAP_S0;
+    // binary64: the sizes of a lattice have not been looked at yet
+    const double N = r.sys.kind == FCIQMC_HUBBARD ? (double)r.sys.lx * r.sys.ly : (double)r.sys.norb;
+    const double np = N * (N + 1) / 2, ne = np * (np + 1) / 2, nss = N * (N - 1) / 2;
+    const double dets = expected_dets(r.p);
+    const int bb = std::max(start_bits(dets, r.p.max_dets <= 0), start_bits(dets / 0.64, false));
+    double bytes = 8.0 * (N * N + ne) + 16.0 * (N + 2 * N * N + 2 * N * N * N) + 4096.0 * sizeof(fciqmc_iter_stats) +
+                   (double)heavy_slices(r.p) * sizeof(HeavyChunk) + 65536.0;
+    if (r.p.generator == 1 && r.sys.kind == FCIQMC_ABINITIO) bytes += 16.0 * (N * N * N * N + nss * nss + N * N + nss);
+    const int ecap = CAP_M + 4 * CAP_S0;
     int tb = TABBITS;
-    while ((double)(1 << tb) < 2.0 * ecap) tb++;
-    const double scratch = (double)BIG_BLOCKS * (ecap * 52.0 + 4.0 * (double)(1 << tb) + 256.0);
-    return (int64_t)((double)(1LL << bb) * per_bucket + scratch + 8.0 * (N * N + ne) + 48.0 * N * N +
-                     4096.0 * 88 + 1.0e6);
+    while ((1 << tb) < 2 * ecap) tb++;
+    const double scratch = BIG_BLOCKS * (ecap * 52.0 + (4 << tb) + 256.0);
+    return (int64_t)std::min(9e18, bytes + (double)layout_bytes(r.p, false, bb, 5 * CAP_S0) + scratch);
 }
 
 extern "C" {

@@ -192,3 +192,28 @@ def test_create_without_room_for_spread_buckets_takes_fewer(monkeypatch):
     alloc.refuse = (lay["buckets"] * lay["cap_main"] * 16,)
     few = fq.fciqmc_layout(fq.fciqmc_create(sysd, prm))
     assert few["buckets"] < lay["buckets"] and few["device_bytes"] < lay["device_bytes"]
+
+
+REQUESTS = {
+    "lattice": (workloads.hubbard_2d(4, 4, 4.0), dict(tau=0.005, target_walkers=1e4)),
+    "adaptive": (workloads.small_abinitio(12, 4, 4, seed=9), dict(tau=0.002, target_walkers=3e4, adaptive_shift=1)),
+    "heatbath": (workloads.config_abinitio_24()[0], dict(tau=2e-4, target_walkers=1e4, generator=1)),
+    "stated_length": (workloads.config_abinitio_24()[0], dict(tau=2e-4, max_dets=150000)),
+}
+
+
+@pytest.mark.parametrize("kind", sorted(REQUESTS))
+def test_server_counts_at_least_what_create_takes(kind):
+    """A second request of the same kind is not admitted into a budget that it
+    would exceed as soon as it is created, and is into one with room."""
+    fq = _fq()
+    sysd, prm = REQUESTS[kind]
+    prm = dict(DAMP, seed=41, max_device_bytes=8 << 30, **prm)
+    size = fq.fciqmc_layout(fq.fciqmc_create(sysd, prm, use_torch=False))["device_bytes"]
+    for budget, second in ((2 * size - 1, "queued"), (8 * size, "running")):
+        srv = fq.fciqmc_server_create(budget, max_active=8)
+        ids = [fq.fciqmc_server_submit(srv, sysd, prm, target_sigma=1e-12, max_iters=50) for _ in range(2)]
+        fq.fciqmc_server_tick(srv, 1)
+        got = [fq.fciqmc_server_poll(srv, i)["state_name"] for i in ids]
+        assert got == ["running", second], budget
+        fq.fciqmc_server_destroy(srv)
