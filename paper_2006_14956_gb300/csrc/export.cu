@@ -61,6 +61,10 @@ __device__ __forceinline__ u64 word_rank(u64 w)
     return r;
 }
 
+// the low `bits` bits, 0 to 64 (a shift by 64 has no value in C++)
+__host__ __device__ constexpr u64 low_mask(int bits) { return bits >= 64 ? ~0ULL : (1ULL << bits) - 1ULL; }
+static_assert(low_mask(0) == 0 && low_mask(8) == 255 && low_mask(56) == ~0ULL >> 8 && low_mask(64) == ~0ULL, "low_mask");
+
 // ------------------------------------------------------------------ compaction
 // determinants of every group of XC_GROUP buckets, one thread each
 __global__ void __launch_bounds__(XS_THREADS) k_export_count(const int *__restrict__ cnt, int nbk, int ng, long long *gsum)
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(XS_THREADS) k_export_compact(const ulonglong2 
             const u128 r = ((u128)word_rank(k.x) << bits_b) | word_rank(k.y);
             const long long o = o0 + before + e;
             hi[o] = (u64)(r >> lo_bits);
-            if (lo) lo[o] = (u64)r & ((1ULL << lo_bits) - 1ULL);
+            if (lo) lo[o] = (u64)r & low_mask(lo_bits);
             idx[o] = (unsigned)s;
         }
     }

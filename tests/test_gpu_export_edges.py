@@ -58,3 +58,9 @@ def test_imported_list_comes_back_sorted_with_exact_diagonals(norb, na, nb, n):
     for k in np.unique(np.concatenate([[0, a.size - 1], rng.integers(0, a.size, 300)])):
         want = s.hdiag_rel(int(got["alpha"][k]), int(got["beta"][k]))
         assert bits(np.array([got["hdiag"][k]]))[0] == bits(np.array([want]))[0], k
+
+
+@pytest.mark.parametrize("norb,na,nb,n", [(64, 32, 32, 5000), (64, 31, 30, 4097), (63, 31, 32, 5003)])
+def test_ranks_of_more_than_120_bits(norb, na, nb, n):
+    """Half-filled words of 63 and 64 orbitals: 120 and 122 bits of rank; with 122 the low word is used whole."""
+    test_imported_list_comes_back_sorted_with_exact_diagonals(norb, na, nb, n)
