@@ -2703,10 +2703,28 @@ extern "C" void fciqmc_free_system(fciqmc_system *sys)
 static int autotune_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t out[3])
 {
     if (!hs || k < 1 || n_iter < 1 || !out) return FCIQMC_ERR_INVALID_ARG;
-    // annihilation: 0 = one resident wave, else that many blocks per SM
-    const int spawn_c[] = {0, 1, 2, 4, 8, 16}, anni_c[] = {0, 3, 9, 24}, heavy_c[] = {1, 2, 4};
+    // spawning 0 or 1, annihilation 0: one resident wave, else blocks per SM
+    const int spawn_c[] = {1, 0, 2, 4, 8, 16}, anni_c[] = {0, 3, 9, 24}, heavy_c[] = {1, 2, 4};
     int best_s = 1, best_h = 2, best_a = 0;
     double best = 1e300;
+    bool adaptive = false;
+    for (int i = 0; i < k; i++) {
+        if (!hs[i]) return FCIQMC_ERR_INVALID_ARG;
+        adaptive = adaptive || hs[i]->hi.adaptive;
+    }
+    // a configuration that gives these runs the launch of an earlier one (a
+    // resident wave under another name, or a list too short for the grid) is
+    // not chosen in its place: noise would decide between equals
+    std::vector<int> seen;
+    auto known = [&](int sb, int ab, bool spawn) {
+        int units = 0, g[2];
+        for (int i = 0; i < k; i++) units += 1 << hs[i]->bb;
+        batch_grids(units, adaptive, sb, ab, &g[0], &g[1]);
+        const int grid = g[spawn ? 0 : 1];
+        if (std::find(seen.begin(), seen.end(), grid) != seen.end()) return true;
+        seen.push_back(grid);
+        return false;
+    };
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -2728,17 +2746,20 @@ static int autotune_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t 
     };
     // one sweep per kernel, the others held at their current best
     for (int sb : spawn_c) {
+        const bool same = known(sb, best_a, true);
         double ms;
         int rc = timed(sb, best_h, best_a, &ms);
         if (rc) return rc;
-        if (ms < best) { best = ms; best_s = sb; }
+        if (!same && ms < best) { best = ms; best_s = sb; }
     }
     best = 1e300;
+    seen.clear();
     for (int ab : anni_c) {
+        const bool same = known(best_s, ab, false);
         double ms;
         int rc = timed(best_s, best_h, ab, &ms);
         if (rc) return rc;
-        if (ms < best) { best = ms; best_a = ab; }
+        if (!same && ms < best) { best = ms; best_a = ab; }
     }
     best = 1e300;
     for (int hb : heavy_c) {

@@ -275,6 +275,7 @@ cudaError_t launch_trial_w(const DevInst *dinst, const ulonglong2 *tkey, const d
 long long connections_per_det(int na, int nb, int ma, int mb);
 void set_launch_geometry(int spawn_bps, int heavy_bps, int anni_bps);
 int launch_geometry_generation();
+void batch_grids(int n_units, bool adaptive, int spawn_bps, int anni_bps, int *spawn, int *anni);
 void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps);
 cudaError_t ref_abs_sum(const DevInst *dinst, double *dpartial, double *out, cudaStream_t s);
 cudaError_t export_count(const int *cnt, int nbk, long long *gsum, const long long **total, cudaStream_t s);

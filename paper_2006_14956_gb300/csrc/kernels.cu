@@ -2267,6 +2267,21 @@ static SpawnSplit spawn_split(int n_units, int bps, bool alone)
     return p;
 }
 
+static int spawn_blocks(int spawn_bps, bool adaptive) { return spawn_bps > 1 ? spawn_bps : (adaptive ? 3 : 4); }
+static int anni_grid(int n_units, int anni_bps)
+{
+    const int need = (n_units + AN_WARPS - 1) / AN_WARPS, full = num_sms() * (anni_bps > 0 ? anni_bps : 3);
+    return need < full ? need : full;
+}
+
+// the grids a launch configuration gives a batch of n_units buckets (for
+// fciqmc_autotune: configurations of the same grid are the same launch)
+void batch_grids(int n_units, bool adaptive, int spawn_bps, int anni_bps, int *spawn, int *anni)
+{
+    *spawn = spawn_split(n_units, spawn_blocks(spawn_bps, adaptive), false).grid;
+    *anni = anni_grid(n_units, anni_bps);
+}
+
 // whether the last units of a launch are claimed (with the adaptive shift and
 // with replica lists, whose kernels have no registers to spare, never)
 static bool claims(int n, int nw) { return n / nw >= CLAIM_ROUNDS; }
@@ -2284,7 +2299,7 @@ static void launch_spawn_one(const DevInst *one, int grid, int n_units, int part
 void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s)
 {
-    const SpawnSplit p = spawn_split(n_units, g_spawn_bps > 1 ? g_spawn_bps : (adaptive ? 3 : 4), one != nullptr);
+    const SpawnSplit p = spawn_split(n_units, spawn_blocks(g_spawn_bps, adaptive), one != nullptr);
     const int grid = p.grid, parts = p.parts;
     const unsigned heavy_min = p.heavy_min;
     if (one && one->kind == FCIQMC_HUBBARD) launch_spawn_one<GEN_HOP>(one, grid, n_units, parts, heavy_min, s);
@@ -2345,9 +2360,7 @@ cudaError_t init_kernels()
 cudaError_t launch_annihilate(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units,
                               bool extra, cudaStream_t s)
 {
-    const int bps = g_anni_bps > 0 ? g_anni_bps : 3;
-    const int need = (n_units + AN_WARPS - 1) / AN_WARPS;
-    const int grid = need < num_sms() * bps ? need : num_sms() * bps;
+    const int grid = anni_grid(n_units, g_anni_bps);
     const bool claim = claims(n_units, grid * AN_WARPS);
     if (one && extra) k_annihilate<true, false><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
     else if (one && claim) k_annihilate<false, true><<<grid, AN_THREADS, AN_SMEM, s>>>(*one, n_units);
