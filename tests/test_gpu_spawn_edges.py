@@ -159,3 +159,21 @@ def test_batch_with_claimed_buckets(max_dets):
             x, y = fq.fciqmc_iter_stats_get(g), fq.fciqmc_iter_stats_get(h)
             for name in x:
                 np.testing.assert_array_equal(x[name], y[name], err_msg=name)
+
+
+def test_more_than_64_electrons_bit_exact():
+    """Beyond the table of electron pairs: H_ii of an imported list and of new
+    determinants by the sums that need no table."""
+    fq = _fq()
+    sysd = _abinitio(64, 34, 33, 10)
+    prm = dict(target_walkers=1e9, seed=79, shift_damping=0.5, shift_interval=5, tau=2e-5, initiator_threshold=3.0)
+    s, a, b, c = _list(sysd, 64, 300, 14)
+    g = fq.fciqmc_create(sysd, prm)
+    o = oracle.Run(s, **prm)
+    fq.fciqmc_import_state(g, a, b, c, 0, 0.1)
+    o.import_state(a, b, c, 0, 0.1)
+    fq.fciqmc_step(g, 3)
+    o.step(3)
+    assert o.export()["alpha"].size > 310  # new determinants among them
+    assert_states_equal(fq.fciqmc_export_state(g), o.export())
+    assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats(), first=0)
