@@ -1543,6 +1543,13 @@ static int handle_flags(fciqmc_handle *h, int *retries)
     }
     if (err & ERRB_HEAVY_CAP) {
         rc = grow_heavy(h);
+        if (rc == FCIQMC_ERR_OUT_OF_MEMORY && h->hi.heavy_floor < HEAVY_ATT) {
+            // short lists also queue determinants of a single slice, to save
+            // time: without room for those the queue is kept for the others
+            h->hi.heavy_floor = HEAVY_ATT;
+            inst_changed(h);
+            rc = FCIQMC_OK;
+        }
         if (rc) return rc;
     }
     rc = ensure_side(h);

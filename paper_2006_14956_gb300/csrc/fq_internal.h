@@ -176,6 +176,7 @@ struct DevInst {
     size_t big_stride;
     HeavyChunk *heavy;
     int heavy_cap;
+    unsigned heavy_floor;   // attempts up to which a determinant is never sliced (0, or HEAVY_ATT: no room for more slices)
     Partial *part;
     u64 *acc;  // exact totals of the iteration: NSHARD lines of ACC_STRIDE words (see ACC_*)
     IterState *st;

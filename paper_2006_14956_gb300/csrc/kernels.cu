@@ -669,7 +669,7 @@ __device__ __forceinline__ void spawn_body(const RUNS &runs, int n_units, int pa
                     cper = c / (double)max(nat, 1u);
                 } else {
                     att += nat;
-                    if (nat > heavy_min) {
+                    if (nat > max(heavy_min, I.heavy_floor)) {
                         queue_heavy(I, kk, c, nat, fl, slot);
                         valid = false;
                     } else if (nat & (nat - 1)) {

@@ -217,3 +217,32 @@ def test_server_counts_at_least_what_create_takes(kind):
         got = [fq.fciqmc_server_poll(srv, i)["state_name"] for i in ids]
         assert got == ["running", second], budget
         fq.fciqmc_server_destroy(srv)
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_slices_that_only_save_time_are_left_out_without_room(batch):
+    """4900 determinants of 100 walkers on a short list, one slice each, for a
+    queue of 4096 that cannot grow: the warps draw them where they find them."""
+    fq = _fq()
+    sysd = workloads.hubbard_1d(8, 1.0, 4.0)
+    s = oracle.system_from_workload(sysd)
+    a, b = (x.copy() for x in np.array(s.determinants(), np.uint64).T)
+    c = 100.0 * np.random.default_rng(6).choice([-1.0, 1.0], a.size)
+    c[:20] *= 40.0  # some with several slices
+    prm = dict(DAMP, tau=1e-5, target_walkers=1e5, initiator_threshold=3.0, seed=35)
+    sizes = dict(prm, max_dets=8000)
+    free = fq.fciqmc_layout(fq.fciqmc_create(sysd, sizes))
+    g = fq.fciqmc_create(sysd, dict(sizes, max_device_bytes=free["device_bytes"] + (200 << 10)))
+    assert fq.fciqmc_layout(g) == free
+    o = oracle.Run(s, **prm)
+    fq.fciqmc_import_state(g, a, b, c, 0, 4.0)
+    o.import_state(a, b, c, 0, 4.0)
+    for _ in range(2):
+        if batch:
+            fq.fciqmc_step_batch([g], 2)
+        else:
+            fq.fciqmc_step(g, 2)
+        o.step(2)
+    assert_states_equal(fq.fciqmc_export_state(g), o.export())
+    assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
+    assert fq.fciqmc_layout(g) == free
