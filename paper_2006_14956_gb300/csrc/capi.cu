@@ -1320,6 +1320,7 @@ int64_t fciqmc_semistoch_info(fciqmc_handle *h, int64_t *nnz)
 }
 
 static int step_to(fciqmc_handle *h, long long target_iter);
+static int split_if_crowded(fciqmc_handle *h);
 
 static int step_impl(fciqmc_handle *h, int64_t n_iter)
 {
@@ -1391,7 +1392,7 @@ static int sync_impl(fciqmc_handle *h)
     long long from = std::max<long long>(h->async_base, h->hst.iter - h->ring_cap);
     rc = pull_history(h, from, h->hst.iter);
     if (rc) return rc;
-    if (!h->hst.err) return FCIQMC_OK;
+    if (!h->hst.err) return split_if_crowded(h);
     return step_to(h, h->async_target);
 }
 
@@ -1421,6 +1422,17 @@ static bool crowded(const fciqmc_handle *h, bool batch)
     const long long nbk = 1LL << h->bb;
     if (!batch && r.ndet > nbk * FILL_M) return true;
     return r.ndet + r.spawns > nbk * FILL_E && r.ndet >= 2 * nbk;
+}
+
+// the early split of a run alone, after iterations whose rows are in its history
+static int split_if_crowded(fciqmc_handle *h)
+{
+    bool done = crowded(h, false);
+    int rc = done ? split_early(h, &done) : FCIQMC_OK;
+    if (rc || !done) return rc;
+    rc = reset_after_error(h);
+    if (!rc) rc = upload_inst(h);
+    return rc ? rc : capture_graph(h);
 }
 
 // Runs iterations until target_iter, in chunks of graph replays; after each
@@ -1474,19 +1486,8 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         }
         rc = pull_history(h, start, h->hst.iter);
         if (rc) return rc;
-        bool split = crowded(h, false);
-        if (split) {
-            rc = split_early(h, &split);
-            if (rc) return rc;
-        }
-        if (split) {
-            rc = reset_after_error(h);
-            if (rc) return rc;
-            rc = upload_inst(h);
-            if (rc) return rc;
-            rc = capture_graph(h);
-            if (rc) return rc;
-        }
+        rc = split_if_crowded(h);
+        if (rc) return rc;
     }
     if (h->profiling && kn > 0)
         for (int j = 0; j < 6; j++) h->ktime[j] = kt[j] / (double)kn;

@@ -246,3 +246,25 @@ def test_slices_that_only_save_time_are_left_out_without_room(batch):
     assert_states_equal(fq.fciqmc_export_state(g), o.export())
     assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
     assert fq.fciqmc_layout(g) == free
+
+
+def test_asynchronous_blocks_split_crowded_buckets_too():
+    """A list that a run alone would split (122 walkers to a bucket of 192) is split at the end of an asynchronous block."""
+    fq = _fq()
+    sysd = dict(workloads.hubbard_1d(8, 1.0, 4.0), n_beta=3, ref=(0x55, 0x2a))
+    s = oracle.system_from_workload(sysd)
+    a, b = (x.copy() for x in np.array(s.determinants(), np.uint64).T)
+    c = 4.5 * np.random.default_rng(4).choice([-1.0, 1.0], a.size)
+    prm = dict(DAMP, tau=0.01, target_walkers=1e9, initiator_threshold=3.0, seed=31)
+    g = fq.fciqmc_create(sysd, dict(prm, max_dets=4000))
+    o = oracle.Run(s, **prm)
+    fq.fciqmc_import_state(g, a, b, c, 0, 4.0)
+    o.import_state(a, b, c, 0, 4.0)
+    assert fq.fciqmc_layout(g)["buckets"] == 32
+    for _ in range(3):
+        fq.fciqmc_step_async(g, 4)
+        fq.fciqmc_sync(g)
+        o.step(4)
+        assert fq.fciqmc_layout(g)["buckets"] == 64
+    assert_states_equal(fq.fciqmc_export_state(g), o.export())
+    assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
