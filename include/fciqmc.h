@@ -453,8 +453,8 @@ int fciqmc_get_launch_config(int32_t out[3]);
 /* Device timing of the kernels of the last fciqmc_step call (milliseconds per
  * iteration, averaged), measured with CUDA events on the handle's stream:
  * out[0] spawn, out[1] heavy-determinant spawn, out[2] annihilation,
- * out[3] finalize, out[4] semi-stochastic; out[5] was H_jj of the determinants
- * created in the iteration, which is now part of the annihilation (out[2]).
+ * out[3] finalize, out[4] semi-stochastic; out[5] = 0 (H_jj of the determinants
+ * created in the iteration is part of the annihilation, out[2]).
  * Enabled by fciqmc_set_profiling. */
 int fciqmc_set_profiling(fciqmc_handle *h, int32_t on);
 int fciqmc_kernel_times(fciqmc_handle *h, double out[6]);

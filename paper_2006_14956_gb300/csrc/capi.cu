@@ -58,7 +58,7 @@ struct fciqmc_handle {
     int graph_gen = -1;     // launch-configuration generation the graph was captured with (-1: none, capture again)
     bool inst_stale = false;  // the device copy of `hi` is out of date
     bool profiling = false;
-    double ktime[6] = {0, 0, 0, 0, 0, 0};  // spawn, heavy, annihilate, finalize, semistoch, new-determinant H_jj
+    double ktime[6] = {0, 0, 0, 0, 0, 0};  // spawn, heavy, annihilate, finalize, semistoch, 0
     // layout
     int bb = 0;
     int heavy_cap = 0;
@@ -347,12 +347,11 @@ static int enqueue_iteration(fciqmc_handle *h, cudaEvent_t *ev)
     if (ev) {  // kernel by kernel
         launch_annihilate_big(h->dinst, 1, h->stream);
         cudaEventRecord(ev[4], h->stream);
-        cudaEventRecord(ev[5], h->stream);
         launch_finalize(h->dinst, 1, h->stream);
+        cudaEventRecord(ev[5], h->stream);
     } else {
         launch_finish(&h->hi, h->stream);
     }
-    if (ev) cudaEventRecord(ev[6], h->stream);
     return FCIQMC_OK;
 }
 
@@ -1446,7 +1445,8 @@ static int step_to(fciqmc_handle *h, long long target_iter)
     int retries = 0;
     std::vector<cudaEvent_t> evs;
     double kt[6] = {0, 0, 0, 0, 0, 0};
-    static const int slot_of[6] = {0, 1, 4, 2, 5, 3};  // event interval -> ktime slot
+    constexpr int NEV = 6;  // events of an iteration
+    static const int slot_of[NEV - 1] = {0, 1, 4, 2, 3};  // event interval -> ktime slot
     long long kn = 0;
     long long chunk_max = 16;  // grows after clean chunks; an error costs at most one chunk of no-op replays
     for (;;) {
@@ -1461,10 +1461,10 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         const long long chunk = std::min<long long>(std::min<long long>(target_iter - start, h->ring_cap), chunk_max);
         chunk_max = std::min<long long>(chunk_max * 2, h->ring_cap);
         if (h->profiling) {
-            evs.resize((size_t)chunk * 7);
+            evs.resize((size_t)chunk * NEV);
             for (auto &e : evs) cudaEventCreate(&e);
             for (long long k = 0; k < chunk; k++) {
-                rc = enqueue_iteration(h, evs.data() + 7 * k);
+                rc = enqueue_iteration(h, evs.data() + NEV * k);
                 if (rc) return rc;
             }
         } else {
@@ -1475,9 +1475,9 @@ static int step_to(fciqmc_handle *h, long long target_iter)
         if (h->profiling) {
             const long long done = h->hst.iter - start;
             for (long long k = 0; k < done; k++)
-                for (int j = 0; j < 6; j++) {
+                for (int j = 0; j < NEV - 1; j++) {
                     float ms = 0.f;
-                    cudaEventElapsedTime(&ms, evs[7 * k + j], evs[7 * k + j + 1]);
+                    cudaEventElapsedTime(&ms, evs[NEV * k + j], evs[NEV * k + j + 1]);
                     kt[slot_of[j]] += ms;
                 }
             kn += done;

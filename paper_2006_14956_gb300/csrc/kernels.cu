@@ -825,8 +825,9 @@ __device__ __forceinline__ int trial_find(const DevInst &I, u64 a, u64 b)
 //      few enough that they are collected first.  Kept records go to the new
 //      bucket in order.  Sums are exact and rounded once, so no order matters.
 // New determinants wait in a queue of the warp for H_jj until there are 32.
-// The table needs no atomics (warp_table.cuh).  A block of 256 threads per bucket of 1024 slots (three
-// barriers per bucket, 128-bit shared accumulators, two blocks per SM) spent
+// The table needs no atomics (warp_table.cuh).  A block of 256 threads per
+// bucket of 1024 slots (three barriers per bucket, 128-bit shared
+// accumulators, two blocks per SM) spent
 // 5.6 of 14 stall cycles per instruction at those barriers: 7.13 ms at 7.3e7
 // determinants and 3.5e7 spawns (50 orbitals), and 0.87 ms more for H_jj in a
 // kernel of its own; this takes 4.2 ms for both.  It is bound by instruction
@@ -1383,9 +1384,8 @@ struct Stage {
     IDX *tab;         // hash table: element index + 1, 0 = empty
     IDX *opos;        // output position of kept owners
 };
-enum { EF_OWNER = 1, EF_OCC = 2, EF_KEEP = 4, EF_ACC = 8, EF_REF = 16, EF_D = 32, EF_REJ = 64, EF_RREC = 128 };
-// EF_REJ: a rejected spawn arrived (owners); EF_RREC: this spawn was rejected;
-// EF_ACC: an accepted spawn arrived (owners, three-phase path)
+enum { EF_OWNER = 1, EF_OCC = 2, EF_KEEP = 4, EF_REF = 16, EF_D = 32, EF_REJ = 64, EF_RREC = 128 };
+// EF_REJ: a rejected spawn arrived (owners); EF_RREC: this spawn was rejected
 
 struct K3Shared {
     int wsum[K3_THREADS / 32];
@@ -1646,7 +1646,6 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
         if (t == 0) I.side_cnt[b] = m + S.side_n;
     }
     // 4. owners: sum = C' + exact spawn sum, then Eq. (3) with the annihilation draw
-    int nk = 0;
     for (int e = t; e < E; e += K3_THREADS) {
         const int f = W.eflag[e];
         if (!(f & EF_OWNER)) continue;
@@ -1666,10 +1665,7 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
             }
         }
         W.val[e] = accv;
-        if (!is_zero(accv) || (f & (EF_REF | EF_D))) {
-            W.eflag[e] = f | EF_KEEP;
-            nk++;
-        }
+        if (!is_zero(accv) || (f & (EF_REF | EF_D))) W.eflag[e] = f | EF_KEEP;
     }
     // 5. output positions in element order
     int total;
@@ -1683,7 +1679,6 @@ __device__ void anni_bucket(const DevInst &I, K3Shared &S, Stage<IDX> W, int tab
     if (overflow && t == 0) { atomicOr(&I.st->err, ERRB_MAIN_CAP); atomicMax(&I.st->need_main, total); }
     for (int e = e0; e < e1; e++)
         if (W.eflag[e] & EF_KEEP) W.opos[e] = (IDX)(o++);
-    (void)nk;
     __syncthreads();
 
     // 6. write the new bucket; reductions
