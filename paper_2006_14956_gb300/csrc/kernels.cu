@@ -1042,7 +1042,10 @@ __device__ __forceinline__ void fill_pairs(unsigned short *pair)
 
 // H_jj of queued new determinants: 32 at a time, one per lane (half the
 // instructions of eight lanes per determinant, and no reduction); a run's
-// last few by eight lanes each (a quarter of the latency)
+// last few by eight lanes each (a quarter of the latency).  On short lists
+// every warp ends with a few: 40 orbitals, 2e4 walkers 43.5 us per iteration,
+// 61.5 with those by a lane each (24 orbitals 40.9 and 48.5, 50 orbitals at
+// 1e5 54.8 and 71.7); with the line at 31 in place of 8 they are the same.
 __device__ __forceinline__ void new_diag(const DevInst &I, AnniWarp &W, int &nq, int np, const unsigned short *pair, bool all)
 {
     __syncwarp();
@@ -2245,18 +2248,22 @@ void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps)
 // How a list's buckets are dealt to warps: as many warps per bucket as it
 // takes to reach every resident warp of the GPU, and the number of attempts
 // above which a determinant goes to the heavy queue (a warp draws its
-// attempts 32 at a time, one after the other)
+// attempts 32 at a time, one after the other).  On a short list, where one
+// determinant's windows are the launch's longest chain, that is 64: a 4x4
+// lattice at 1e5 walkers takes 2.38 ms per 40 iterations, 2.64 with 512 (the
+// 8-site ring at 1e4, 20 iterations: 0.907 and 0.888).  On long lists and in
+// batches 64, 256 and 512 are the same within 1 %.
 struct SpawnSplit {
     int parts, grid;
     unsigned heavy_min;
 };
-static SpawnSplit spawn_split(int n_units, int bps, bool alone)
+static SpawnSplit spawn_split(int n_units, int bps)
 {
     SpawnSplit p;
     const int warps = num_sms() * 4 * SP_WARPS;
     p.parts = 1;
     while (p.parts < CAP_M / 32 && (long long)n_units * p.parts < 2 * warps) p.parts *= 2;
-    p.heavy_min = p.parts > 1 ? 64 : (alone ? HEAVY_ATT : HEAVY_ATT / 2);
+    p.heavy_min = p.parts > 1 ? 64 : HEAVY_ATT;
     const long long need = ((long long)n_units * p.parts + SP_WARPS - 1) / SP_WARPS;
     p.grid = (int)(need < (long long)num_sms() * bps ? need : (long long)num_sms() * bps);
     return p;
@@ -2273,7 +2280,7 @@ static int anni_grid(int n_units, int anni_bps)
 // fciqmc_autotune: configurations of the same grid are the same launch)
 void batch_grids(int n_units, bool adaptive, int spawn_bps, int anni_bps, int *spawn, int *anni)
 {
-    *spawn = spawn_split(n_units, spawn_blocks(spawn_bps, adaptive), false).grid;
+    *spawn = spawn_split(n_units, spawn_blocks(spawn_bps, adaptive)).grid;
     *anni = anni_grid(n_units, anni_bps);
 }
 
@@ -2294,7 +2301,7 @@ static void launch_spawn_one(const DevInst *one, int grid, int n_units, int part
 void launch_spawn(const DevInst *one, const DevInst *dinst, const int *unit_start, int n_inst, int n_units, bool adaptive,
                   cudaStream_t s)
 {
-    const SpawnSplit p = spawn_split(n_units, spawn_blocks(g_spawn_bps, adaptive), one != nullptr);
+    const SpawnSplit p = spawn_split(n_units, spawn_blocks(g_spawn_bps, adaptive));
     const int grid = p.grid, parts = p.parts;
     const unsigned heavy_min = p.heavy_min;
     if (one && one->kind == FCIQMC_HUBBARD) launch_spawn_one<GEN_HOP>(one, grid, n_units, parts, heavy_min, s);
