@@ -130,7 +130,8 @@ typedef struct {
     int64_t semistoch_start;
     int64_t max_dets;
     int64_t max_spawns;
-    int64_t max_device_bytes; /* growth beyond this fails with FCIQMC_ERR_OUT_OF_MEMORY (0 = no limit) */
+    int64_t max_device_bytes; /* growth that a run needs fails beyond this with FCIQMC_ERR_OUT_OF_MEMORY, growth
+                                 that only saves time is left out (0 = no limit) */
     void *stream;
     void *(*alloc)(size_t bytes, void *ctx);
     void (*free)(void *ptr, void *ctx);
@@ -431,8 +432,8 @@ void fciqmc_server_destroy(fciqmc_server *srv);
 /* Autotuner of the launch configuration: times n_iter iterations of the
  * batch hs[0..k-1] (advancing it) for each candidate, keeps the fastest for
  * every later launch in the process, and writes it to out[3] (spawn, heavy,
- * annihilation).  Of candidates that are the same launch for these runs only
- * the first can be chosen.  Candidates: for the spawning kernel 0 or 1 = one resident
+ * annihilation).  Candidates that are the same launch for these runs count as
+ * one, reported as the first of them.  Candidates: for the spawning kernel 0 or 1 = one resident
  * wave of blocks (four 256-thread blocks per SM), 2, 4, 8, 16 = that many
  * blocks per SM; the heavy-spawning kernel's grid (1, 2, 4 blocks per SM);
  * for the annihilation 0 = one resident wave of blocks (three 256-thread

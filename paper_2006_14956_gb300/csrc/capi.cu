@@ -2722,16 +2722,16 @@ static int autotune_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t 
     }
     // a configuration that gives these runs the launch of an earlier one (a
     // resident wave under another name, or a list too short for the grid) is
-    // not chosen in its place: noise would decide between equals
-    std::vector<int> seen;
-    auto known = [&](int sb, int ab, bool spawn) {
+    // one more timing of that one: noise would decide between equals
+    std::vector<std::pair<int, int>> seen;  // grid, first configuration that gives it
+    auto first_of = [&](int sb, int ab, bool spawn) {
         int units = 0, g[2];
         for (int i = 0; i < k; i++) units += 1 << hs[i]->bb;
         batch_grids(units, adaptive, sb, ab, &g[0], &g[1]);
-        const int grid = g[spawn ? 0 : 1];
-        if (std::find(seen.begin(), seen.end(), grid) != seen.end()) return true;
-        seen.push_back(grid);
-        return false;
+        for (const auto &e : seen)
+            if (e.first == g[spawn ? 0 : 1]) return e.second;
+        seen.push_back({g[spawn ? 0 : 1], spawn ? sb : ab});
+        return spawn ? sb : ab;
     };
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -2754,20 +2754,20 @@ static int autotune_impl(fciqmc_handle **hs, int32_t k, int64_t n_iter, int32_t 
     };
     // one sweep per kernel, the others held at their current best
     for (int sb : spawn_c) {
-        const bool same = known(sb, best_a, true);
+        const int first = first_of(sb, best_a, true);
         double ms;
         int rc = timed(sb, best_h, best_a, &ms);
         if (rc) return rc;
-        if (!same && ms < best) { best = ms; best_s = sb; }
+        if (ms < best) { best = ms; best_s = first; }
     }
     best = 1e300;
     seen.clear();
     for (int ab : anni_c) {
-        const bool same = known(best_s, ab, false);
+        const int first = first_of(best_s, ab, false);
         double ms;
         int rc = timed(best_s, best_h, ab, &ms);
         if (rc) return rc;
-        if (!same && ms < best) { best = ms; best_a = ab; }
+        if (ms < best) { best = ms; best_a = first; }
     }
     best = 1e300;
     for (int hb : heavy_c) {
