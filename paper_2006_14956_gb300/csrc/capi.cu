@@ -873,7 +873,8 @@ fciqmc_handle *fciqmc_replica(fciqmc_handle *h, int32_t r)
     return nullptr;
 }
 
-static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 replica, fciqmc_handle **out)
+// spread: a short list may get more, smaller buckets (start_bits)
+static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 replica, bool spread, fciqmc_handle **out)
 {
     if (!out) return fail(nullptr, FCIQMC_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
@@ -1165,7 +1166,7 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     // not spread: a list of a stated length (max_dets; it is still split when
     // crowded), and where the memory limit or the allocator leaves little room
     const int tight = start_bits(dets_hint, false);
-    int bb = start_bits(dets_hint, P.max_dets <= 0);
+    int bb = start_bits(dets_hint, spread && P.max_dets <= 0);
     if (P.max_device_bytes > 0 && 8 * layout_bytes(P, P.replicas == 2, bb, CAP_S0) > P.max_device_bytes) bb = tight;
     I.cap_s = CAP_S0;
     int rc = alloc_layout(h, I, bb);
@@ -1208,20 +1209,16 @@ static int create_run(const fciqmc_system *sys, const fciqmc_params *prm, u64 re
     return FCIQMC_OK;
 }
 
-static int create_impl(const fciqmc_system *sys, const fciqmc_params *prm, fciqmc_handle **out)
+// a replica pair: same system and parameters, the second replica with Philox
+// key word 1 = 1, on the first one's stream
+static int create_pair(const fciqmc_system *sys, const fciqmc_params *prm, bool spread, fciqmc_handle **out)
 {
-    if (prm && (prm->replicas < 0 || prm->replicas > 2)) {
-        if (out) *out = nullptr;
-        return fail(nullptr, FCIQMC_ERR_INVALID_ARG, "replicas must be 1 or 2");
-    }
-    int rc = create_run(sys, prm, 0, out);
-    if (rc || prm->replicas != 2) return rc;
-    // the second replica: same system and parameters, Philox key word 1 = 1,
-    // on the first replica's stream
+    int rc = create_run(sys, prm, 0, spread, out);
+    if (rc) return rc;
     fciqmc_handle *h = *out, *h2 = nullptr;
     fciqmc_params p2 = *prm;
     p2.stream = h->stream;
-    rc = create_run(sys, &p2, 1, &h2);
+    rc = create_run(sys, &p2, 1, spread, &h2);
     if (rc) {
         fciqmc_destroy(h);
         *out = nullptr;
@@ -1230,6 +1227,7 @@ static int create_impl(const fciqmc_system *sys, const fciqmc_params *prm, fciqm
     h->partner = h2; h2->partner = h; h2->secondary = true;
     h->paired = h2->paired = true;
     rc = replica_kernel_init() == cudaSuccess ? FCIQMC_OK : fail(h, FCIQMC_ERR_CUDA, "replica kernel set-up failed");
+    if (!rc && h->bb != h2->bb) rc = fail(h, FCIQMC_ERR_OUT_OF_MEMORY, "out of device memory (second replica)");
     if (!rc) rc = ensure_side(h);
     if (!rc) rc = ensure_side(h2);
     if (!rc) rc = upload_inst(h);
@@ -1242,6 +1240,18 @@ static int create_impl(const fciqmc_system *sys, const fciqmc_params *prm, fciqm
         *out = nullptr;
     }
     return rc;
+}
+
+static int create_impl(const fciqmc_system *sys, const fciqmc_params *prm, fciqmc_handle **out)
+{
+    if (prm && (prm->replicas < 0 || prm->replicas > 2)) {
+        if (out) *out = nullptr;
+        return fail(nullptr, FCIQMC_ERR_INVALID_ARG, "replicas must be 1 or 2");
+    }
+    if (!prm || prm->replicas != 2) return create_run(sys, prm, 0, true, out);
+    // both replicas have one layout: without room for two spread ones, two tight ones
+    const int rc = create_pair(sys, prm, true, out);
+    return rc == FCIQMC_ERR_OUT_OF_MEMORY ? create_pair(sys, prm, false, out) : rc;
 }
 
 int fciqmc_create(const fciqmc_system *sys, const fciqmc_params *prm, fciqmc_handle **out)

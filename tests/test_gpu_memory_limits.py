@@ -268,3 +268,22 @@ def test_asynchronous_blocks_split_crowded_buckets_too():
         assert fq.fciqmc_layout(g)["buckets"] == 64
     assert_states_equal(fq.fciqmc_export_state(g), o.export())
     assert_stats_equal(fq.fciqmc_iter_stats_get(g), o.stats())
+
+
+@pytest.mark.parametrize("skip,which", [(0, "keys"), (2, "keys"), (1, "lists")])
+def test_create_a_pair_with_one_layout_for_both(monkeypatch, skip, which):
+    """The spread layout's keys refused to the first or to the second replica, or its lists to the second: both get
+    the tight one."""
+    fq = _fq()
+    alloc = _Refusing.install(fq, monkeypatch)
+    sysd = workloads.small_abinitio(12, 4, 4, seed=9)
+    prm = dict(DAMP, tau=0.002, target_walkers=1e4, initiator_threshold=3.0, seed=36, replicas=2)
+    lay = fq.fciqmc_layout(fq.fciqmc_create(sysd, prm))
+    keys = lay["buckets"] * lay["cap_main"] * 16
+    alloc.refuse = (keys if which == "keys" else lay["buckets"] * (lay["cap_main"] + lay["cap_spawn"]) * 48,)
+    alloc.skip = skip
+    g = fq.fciqmc_create(sysd, prm)
+    alloc.refuse = ()
+    a, b = (fq.fciqmc_layout(fq.fciqmc_replica(g, r)) for r in (0, 1))
+    assert a == b and a["buckets"] < lay["buckets"]
+    fq.fciqmc_step(g, 10)
