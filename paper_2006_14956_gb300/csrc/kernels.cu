@@ -2251,8 +2251,10 @@ void get_launch_geometry(int *spawn_bps, int *heavy_bps, int *anni_bps)
 // attempts 32 at a time, one after the other).  On a short list, where one
 // determinant's windows are the launch's longest chain, that is 64: a 4x4
 // lattice at 1e5 walkers takes 2.38 ms per 40 iterations, 2.64 with 512 (the
-// 8-site ring at 1e4, 20 iterations: 0.907 and 0.888).  On long lists and in
-// batches 64, 256 and 512 are the same within 1 %.
+// 8-site ring at 1e4, 20 iterations: 0.907 and 0.888).  On a long list it is
+// half a slice: a batch of eight served requests takes 362 ms, 374 with 512;
+// 64 lattice runs and 50 orbitals at 1e7 walkers are the same with 64, 256 and
+// 512 within 1 %.
 struct SpawnSplit {
     int parts, grid;
     unsigned heavy_min;
@@ -2263,7 +2265,7 @@ static SpawnSplit spawn_split(int n_units, int bps)
     const int warps = num_sms() * 4 * SP_WARPS;
     p.parts = 1;
     while (p.parts < CAP_M / 32 && (long long)n_units * p.parts < 2 * warps) p.parts *= 2;
-    p.heavy_min = p.parts > 1 ? 64 : HEAVY_ATT;
+    p.heavy_min = p.parts > 1 ? 64 : HEAVY_ATT / 2;
     const long long need = ((long long)n_units * p.parts + SP_WARPS - 1) / SP_WARPS;
     p.grid = (int)(need < (long long)num_sms() * bps ? need : (long long)num_sms() * bps);
     return p;
